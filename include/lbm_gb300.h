@@ -148,9 +148,10 @@ int lbm_set_state(lbm_handle *h, const double *f, const double *g, const double 
 int lbm_save(lbm_handle *h, const char *path);
 int lbm_load(lbm_handle *h, const char *path);
 
-/* Launch shape of the step kernel (no counterpart in the paper): each CTA walks `rows`
- * consecutive rows of a strip (0 = automatic: the length that minimises the waves of
- * resident CTAs times the rows each walks).  Affects speed only, never the results. */
+/* Launch shape of the step (no counterpart in the paper): rows > 0: each CTA walks `rows`
+ * consecutive rows of a 128-column strip; 0 = automatic: 2-D tiles on channels too small to
+ * fill the GPU with strips, else strips with the length that minimises the waves of resident
+ * CTAs times the rows each walks.  Affects speed only, never the results. */
 int lbm_set_segment(lbm_handle *h, int32_t rows);
 
 /* Test hook for the fault path (not part of the method).  The step kernel stages its
@@ -163,11 +164,11 @@ int lbm_set_segment(lbm_handle *h, int32_t rows);
  * normal stepping.  No GPU fault or trap is involved. */
 int lbm_test_stall_copies(lbm_handle *h, int32_t on);
 
-/* Autotuner (no counterpart in the paper): times `reps` launches of the step kernel for
- * each candidate segment length (the automatic choice, then 8 .. 256 rows below ny) and
- * keeps the fastest; *rows (may be NULL) receives its row count.  The kernel is re-launched
- * from the same input buffer, so the state and the step count are unchanged.
- * Synchronises. */
+/* Autotuner (no counterpart in the paper): times `reps` launches of the step for each
+ * candidate shape (2-D tiles, strips with the automatic segment length, strips of 8 .. 256 rows
+ * below ny) and keeps the fastest; *rows (may be NULL) receives the rows of its segments or
+ * tiles.  The kernel is re-launched from the same input buffer, so the state and the step
+ * count are unchanged.  Synchronises. */
 int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows);
 
 /* Bytes the step kernel moves per lattice node and step (populations read and written
@@ -224,8 +225,9 @@ int lbm_batch_create(int32_t n, const lbm_domain *domains, const lbm_params *par
 /* Steps per chunk and residual check (even, >= 2; default 100). */
 int lbm_batch_set_check_interval(lbm_batch *b, int32_t K);
 
-/* Autotuner for the batch launch: times `reps` launches per candidate segment length and
- * keeps the fastest (state untouched); *rows receives it.  Synchronises. */
+/* Autotuner for the batch launch: times `reps` launches per candidate shape (tiles, segment
+ * lengths) and keeps the fastest (state untouched); *rows receives the rows of its tiles or
+ * segments.  Synchronises. */
 int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows);
 
 /* Advance every active channel by nsteps (a multiple of K).  Synchronises after every
@@ -244,7 +246,7 @@ int lbm_batch_fields(lbm_batch *b, int32_t c, double *phi, double *u, double *v,
 int lbm_batch_diag(lbm_batch *b, int32_t c, double *residual, int64_t *steps);
 int lbm_batch_init_fields(lbm_batch *b, int32_t c, const double *phi, const double *u, const double *v,
                           const double *T, const double *dp);
-/* Number of channels, CTAs per batch launch and rows per CTA segment. */
+/* Number of channels, CTAs per batch launch and rows per CTA (segment or tile). */
 int lbm_batch_size(const lbm_batch *b, int32_t *n, int32_t *ctas, int32_t *rows);
 void lbm_batch_destroy(lbm_batch *b);
 

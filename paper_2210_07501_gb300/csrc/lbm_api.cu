@@ -20,6 +20,11 @@
 
 using namespace lbm;
 
+// The launch shapes of a channel: tiles, marching strips, and the rule's choice.
+struct Shapes {
+    StepShape tile, march, automatic;
+};
+
 struct lbm_handle {
     lbm_domain dom;
     lbm_params prm;
@@ -44,7 +49,8 @@ struct lbm_handle {
     double *staging;        // lazily allocated [9][ny][nx] doubles for state I/O
     int cur;
     int64_t step, check_interval, launches;
-    int seg_rows;           // rows per CTA segment of the step kernel (0 = automatic)
+    Shapes shapes;
+    StepShape shape;        // how steps are launched: shapes.automatic unless set or tuned
     unsigned int tx_extra;  // lbm_test_stall_copies: extra bytes each copy stage waits for
     int64_t last_check_step, prev_check_step;
     bool have_check, have_prev_check;
@@ -154,7 +160,36 @@ static cudaError_t dispatch(const lbm_handle *h, Args... args)
 template <typename R, typename S, int QF, int QT> struct StepFn {
     static cudaError_t run(const lbm_handle *h, int src, double *macro)
     {
-        return launch_step<R, S, QF, QT>(make_args<R, S>(h, src, macro), h->stream, h->seg_rows);
+        const StepArgs<R, S> A = make_args<R, S>(h, src, macro);
+        if (h->shape.rows > 0) return launch_march<R, S, QF, QT>(A, h->stream, h->shape.rows);
+        // the stall hook acts on the copies that only the march has
+        if (h->tx_extra) return launch_march<R, S, QF, QT>(A, h->stream, h->shapes.march.rows);
+        return launch_tile<R, S, QF, QT>(A, h->stream, h->shape.tx, h->shape.ty);
+    }
+};
+
+// Channels up to this many nodes (batches: in total) step on tiles, larger ones in marching strips.
+// The march reads no row twice and reaches the copy bandwidth once its strips fill the GPU for
+// several waves; the tiles win while they do not.  Measured (us a step, march / tiles): FP32 20.6 / 9.6
+// at 1024 x 256, 74 / 70 at 2048 x 1024, 136 / 135 at 4096 x 1024, 486 / 513 at 8192 x 2048.
+// FP16 storage is never bandwidth bound: 31 / 12 at 1024 x 256, 628 / 529 at 8192 x 2048.
+static long long tile_nodes_max(int prec)
+{
+    return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 1LL << 22 : 1LL << 19);
+}
+// ny_total: the channel's rows (a batch: those of all its channels, put one on top of the other)
+template <typename R, typename S, int QF, int QT> struct ShapesFn {
+    static cudaError_t run(const lbm_handle *h, long long ny_total, Shapes *out)
+    {
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        out->tile = StepShape{0, 0, 0};
+        choose_tile<R, S, QF, QT>(h->nx, ny_total, sms, &out->tile.tx, &out->tile.ty);
+        out->march = StepShape{auto_segment<R, S, QF, QT>(h->nx, h->ny), 0, 0};
+        out->automatic = h->nx * ny_total <= tile_nodes_max(h->prec) ? out->tile : out->march;
+        return cudaGetLastError();
     }
 };
 template <typename R, typename S, int QF, int QT> struct InitFn {
@@ -439,6 +474,9 @@ int lbm_create(const lbm_domain *domain, const lbm_params *params, void *stream,
         for (int k = 0; k < 3; ++k) cudaMemsetAsync(h->pop[b][k], 0, (size_t)Q[k] * h->plane * h->esize, h->stream);
         cudaMemsetAsync(h->dp[b], 0, (size_t)h->plane * h->rsize, h->stream);
     }
+    e = dispatch<ShapesFn>(h, (long long)h->ny, &h->shapes);
+    if (e != cudaSuccess) { free_all(h); delete h; return cuda_fail(e, "launch shapes"); }
+    h->shape = h->shapes.automatic;
     // physical constants (Sec. 2-4), lattice units, c^2 = 1/3, c_p = 1
     const lbm_params *p = params;
     Phys<double> &P = h->P;
@@ -626,14 +664,6 @@ int lbm_run_to_steady(lbm_handle *h, double tol, int64_t max_steps, int64_t *ste
 
 }  // extern "C"
 
-template <typename R, typename S, int QF, int QT> struct AutoSegFn {
-    static cudaError_t run(const lbm_handle *h, int *rows)
-    {
-        *rows = auto_segment<R, S, QF, QT>(h->nx, h->ny);
-        return cudaGetLastError();
-    }
-};
-
 template <typename R, typename S, int QF, int QT> struct GetFn {
     static cudaError_t run(const lbm_handle *h, double *stage, int lattice, int Q, int toStore)
     {
@@ -814,7 +844,7 @@ int lbm_load(lbm_handle *h, const char *path)
 int lbm_set_segment(lbm_handle *h, int32_t rows)
 {
     if (!h || rows < 0) return LBM_EINVAL;
-    h->seg_rows = rows;
+    h->shape = rows > 0 ? StepShape{rows, 0, 0} : h->shapes.automatic;
     return LBM_OK;
 }
 
@@ -828,24 +858,24 @@ int lbm_test_stall_copies(lbm_handle *h, int32_t on)
 int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows)
 {
     if (!h || reps < 1) return LBM_EINVAL;
-    // candidates: the automatic choice (whole waves), then fixed segment lengths up to the
-    // channel height
-    int cand[16], nc = 0;
-    int autoseg = 0;
-    CK(dispatch<AutoSegFn>(h, &autoseg));
-    cand[nc++] = autoseg;
+    // candidates: tiles, marching strips with the automatic segment length (whole waves), then
+    // fixed segment lengths up to the channel height
+    StepShape cand[16];
+    int nc = 0;
+    cand[nc++] = h->shapes.tile;
+    cand[nc++] = h->shapes.march;
     const int fixed[] = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256};
     for (int f : fixed)
-        if (f < h->ny && f != autoseg && nc < 16) cand[nc++] = f;
+        if (f < h->ny && f != h->shapes.march.rows && nc < 16) cand[nc++] = StepShape{f, 0, 0};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    const int saved = h->seg_rows;
+    const StepShape saved = h->shape;
     float best_ms = 1e30f;
-    int best = 0;
+    StepShape best = saved;
     int rc = LBM_OK;
     for (int k = 0; k < nc && rc == LBM_OK; ++k) {
-        h->seg_rows = cand[k];
+        h->shape = cand[k];
         // the kernel reads buffer cur and writes the other one; launching it again from
         // the same buffer leaves the state and the step count untouched
         cudaError_t e = dispatch<StepFn>(h, h->cur, (double *)nullptr);      // warm-up
@@ -860,8 +890,8 @@ int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows)
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    h->seg_rows = rc == LBM_OK ? best : saved;
-    if (rows) *rows = h->seg_rows;
+    h->shape = rc == LBM_OK ? best : saved;
+    if (rows) *rows = h->shape.rows > 0 ? h->shape.rows : h->shape.ty;
     return rc;
 }
 
@@ -901,7 +931,9 @@ struct lbm_batch {
     void *d_args[2] = {nullptr, nullptr};   // StepArgs per case, source buffer 0 / 1, no macros
     void *d_args_m[2] = {nullptr, nullptr}; // same, writing the macroscopic fields
     int4 *d_ctas = nullptr;
-    int n_ctas = 0, seg = 32;
+    int n_ctas = 0;
+    Shapes shapes;
+    StepShape shape;
     int *d_active = nullptr;
     std::vector<int> active;
     double *d_results = nullptr;       // [n][4] reduction results of the last check, then the fault word
@@ -938,12 +970,13 @@ template <typename R, typename S, int QF, int QT> struct BatchArgsFn {
 };
 
 template <typename R, typename S, int QF, int QT> struct BatchTableFn {
-    static cudaError_t run(const lbm_handle *, lbm_batch *b, int seg)
+    static cudaError_t run(const lbm_handle *, lbm_batch *b, StepShape shape)
     {
-        const int TX = step_strip_width<R, S, QF, QT>();
+        const int w = shape.rows > 0 ? step_strip_width<R, S, QF, QT>() : shape.tx;
+        const int t_rows = shape.rows > 0 ? shape.rows : shape.ty;
         std::vector<int4> t;
         for (int c = 0; c < b->n; ++c) {
-            const int strips = (b->h[c]->nx + TX - 1) / TX, segs = (b->h[c]->ny + seg - 1) / seg;
+            const int strips = (b->h[c]->nx + w - 1) / w, segs = (b->h[c]->ny + t_rows - 1) / t_rows;
             for (int by = 0; by < segs; ++by)
                 for (int bx = 0; bx < strips; ++bx) t.push_back(make_int4(c, bx, by, 0));
         }
@@ -952,7 +985,7 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
         cudaError_t e = cudaMalloc((void **)&b->d_ctas, t.size() * sizeof(int4));
         if (e != cudaSuccess) return e;
         b->n_ctas = (int)t.size();
-        b->seg = seg;
+        b->shape = shape;
         return cudaMemcpy(b->d_ctas, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice);
     }
 };
@@ -961,15 +994,10 @@ template <typename R, typename S, int QF, int QT> struct BatchStepFn {
     static cudaError_t run(const lbm_handle *, lbm_batch *b, int par, int macro)
     {
         const StepArgs<R, S> *args = (const StepArgs<R, S> *)(macro ? b->d_args_m[par] : b->d_args[par]);
-        return launch_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->seg, b->stream);
-    }
-};
-
-template <typename R, typename S, int QF, int QT> struct BatchSlotsFn {
-    static cudaError_t run(const lbm_handle *, int *slots)
-    {
-        *slots = resident_ctas<R, S, QF, QT>();
-        return cudaSuccess;
+        if (b->shape.rows > 0)
+            return launch_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape.rows, b->stream);
+        return launch_tile_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape.tx, b->shape.ty,
+                                               b->stream);
     }
 };
 
@@ -1058,9 +1086,18 @@ int lbm_batch_create(int32_t n, const lbm_domain *domains, const lbm_params *par
     cudaError_t e = cudaMemcpy(b->d_active, b->active.data(), n * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_results, 0, (4 * (size_t)n + 1) * sizeof(double));
     if (e == cudaSuccess) e = dispatch<BatchArgsFn>(b->h[0], b);
-    int slots = 0;
-    if (e == cudaSuccess) e = dispatch<BatchSlotsFn>(b->h[0], &slots);
-    if (e == cudaSuccess) e = dispatch<BatchTableFn>(b->h[0], b, 32);
+    // the shapes for as many rows of the widest channel as the batch has nodes; marching segments of
+    // 32 rows until tuned
+    const lbm_handle *widest = b->h[0];
+    long long nodes = 0;
+    for (const lbm_handle *h : b->h) {
+        nodes += (long long)h->nx * h->ny;
+        if (h->nx > widest->nx) widest = h;
+    }
+    if (e == cudaSuccess) e = dispatch<ShapesFn>(widest, (nodes + widest->nx - 1) / widest->nx, &b->shapes);
+    b->shapes.march.rows = 32;
+    if (b->shapes.automatic.rows > 0) b->shapes.automatic = b->shapes.march;
+    if (e == cudaSuccess) e = dispatch<BatchTableFn>(b->h[0], b, b->shapes.automatic);
     if (e != cudaSuccess) { int rc = cuda_fail(e, "lbm_batch_create"); lbm_batch_destroy(b); return rc; }
     *out = b;
     return LBM_OK;
@@ -1079,15 +1116,18 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
     if (!b || reps < 1) return LBM_EINVAL;
     int maxny = 0;
     for (lbm_handle *h : b->h) maxny = h->ny > maxny ? h->ny : maxny;
-    const int cand[] = {8, 12, 16, 24, 32, 48, 64, 96, 128};
+    const int fixed[] = {8, 12, 16, 24, 32, 48, 64, 96, 128};
+    std::vector<StepShape> cand = {b->shapes.tile};
+    for (int seg : fixed)
+        if (seg <= maxny || seg == fixed[0]) cand.push_back(StepShape{seg, 0, 0});
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     float best_ms = 1e30f;
-    int best = b->seg, rc = LBM_OK;
-    for (int seg : cand) {
-        if (seg > maxny && seg != cand[0]) continue;
-        cudaError_t e = dispatch<BatchTableFn>(b->h[0], b, seg);
+    StepShape best = b->shape;
+    int rc = LBM_OK;
+    for (const StepShape &shape : cand) {
+        cudaError_t e = dispatch<BatchTableFn>(b->h[0], b, shape);
         // launches from buffer 0 into buffer 1 leave the state (in buffer 0) untouched
         if (e == cudaSuccess) e = dispatch<BatchStepFn>(b->h[0], b, 0, 0);
         if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
@@ -1097,7 +1137,7 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
         float ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
         if (e != cudaSuccess) { rc = cuda_fail(e, "lbm_batch_autotune"); break; }
-        if (ms < best_ms) { best_ms = ms; best = seg; }
+        if (ms < best_ms) { best_ms = ms; best = shape; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1106,7 +1146,7 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
         if (e != cudaSuccess) rc = cuda_fail(e, "lbm_batch_autotune");
     }
     b->graph_valid = false;
-    if (rows) *rows = b->seg;
+    if (rows) *rows = b->shape.rows > 0 ? b->shape.rows : b->shape.ty;
     return rc;
 }
 
@@ -1203,7 +1243,7 @@ int lbm_batch_size(const lbm_batch *b, int32_t *n, int32_t *ctas, int32_t *rows)
     if (!b) return LBM_EINVAL;
     if (n) *n = b->n;
     if (ctas) *ctas = b->n_ctas;
-    if (rows) *rows = b->seg;
+    if (rows) *rows = b->shape.rows > 0 ? b->shape.rows : b->shape.ty;
     return LBM_OK;
 }
 

@@ -56,7 +56,7 @@ template <typename Real> struct Phys {
     Real g2min;       // |grad phi|^2 below which n = 0
 };
 
-template <typename Real, typename Store> struct StepArgs {
+template <typename Real, typename Store> struct alignas(16) StepArgs {
     int nx, ny, pitch;
     long long plane;                // ny * pitch elements per population plane
     const Store *f_in;
@@ -97,14 +97,20 @@ enum { RT_PHI0 = 0, RT_DR = 1, RT_GREF = 2, RT_TH0 = 3, RT_C01 = 4, RT_DRLO = 5,
 // dR of the mirrored row y + 3 (high, low), d_y phi0(y + 1), unused
 enum { RX_PHI0 = 0, RX_TH0 = 1, RX_C01 = 2, RX_GREF = 3, RX_DR3 = 4, RX_DR3LO = 5, RX_GREF1 = 6, RX_N = 8 };
 
-// ---- storage conversion ----
+// Programmatic dependent launch: let the next launch of the stream start; wait for the complete
+// end of the previous one (no-ops in a launch without the attribute).
+__device__ __forceinline__ void pdl_launch_next_() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---- storage conversion (plain loads, which stay behind pdl_wait_: the populations are
+// written by the launch before) ----
 template <typename Real, typename Store>
 __device__ __forceinline__ Real ld_(const Store *p)
 {
     if constexpr (std::is_same<Store, __half>::value)
-        return Real(__half2float(__ldg(p)));
+        return Real(__half2float(*p));
     else
-        return Real(__ldg(p));
+        return Real(*p);
 }
 template <typename Real, typename Store>
 __device__ __forceinline__ void st_(Store *p, Real v)
@@ -177,6 +183,10 @@ __device__ __forceinline__ Real rcp_(Real x)
     }
 }
 
+// |g|^2 with the contraction written out: two kernels that form it in different surroundings
+// (from the same gradient) get the same bits
+template <typename Real> __device__ __forceinline__ Real norm2_(Real gx, Real gy) { return fma(gx, gx, gy * gy); }
+
 // The unit normal n = grad phi / |grad phi| as (n_x, n_y - 1).  For an interface close to
 // the flat reference n_y is close to 1, so n_y - 1 = -g_x^2 / (|g| (|g| + g_y)) is formed
 // without cancellation; the stencils of div n take its differences.  n = 0 (n_y - 1 = -1)
@@ -184,7 +194,7 @@ __device__ __forceinline__ Real rcp_(Real x)
 template <typename Real>
 __device__ __forceinline__ void unit_normal_dev_(Real gx, Real gy, Real g2min, Real &nx, Real &my)
 {
-    const Real g2 = gx * gx + gy * gy;
+    const Real g2 = norm2_(gx, gy);
     if (g2 > g2min) {
         Real m, im;
         if constexpr (std::is_same<Real, double>::value) {

@@ -8,20 +8,46 @@
 
 namespace lbm {
 
-// One time step from A's input buffers to its output buffers.  seg_rows > 0 sets the
-// number of rows each CTA marches through; 0 picks it from the occupancy (whole waves).
-template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_step(const StepArgs<Real, Store> &A, cudaStream_t s, int seg_rows);
+// A launch that may start while the previous launch of its stream drains (the kernel calls
+// pdl_wait_ before it touches what that one wrote).
+struct PdlLaunch {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    PdlLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t s)
+    {
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = s;
+        cfg.attrs = at, cfg.numAttrs = 1;
+    }
+};
 
-// Many cases in one launch (see batch_kernel): ctas[i] = (case, strip, segment, 0).
+// How a step is launched: rows > 0: row-marching strips, each CTA walking that many rows; else
+// 2-D tiles of tx x ty nodes.
+struct StepShape {
+    int rows, tx, ty;
+};
+
+// One time step from A's input buffers to its output buffers.
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int rows);
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, int tx, int ty);
+
+// Many cases in one launch (see batch_kernel, tile_batch_kernel): ctas[i] = (case, strip, segment, 0)
+// or (case, tile column, tile row, 0).
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active, int seg,
                          cudaStream_t s);
-// Columns per strip of the step kernel, and CTAs of the batch kernel resident on the device.
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active,
+                              int tx, int ty, cudaStream_t s);
+// Columns per strip of the march.
 template <typename Real, typename Store, int QF, int QT> int step_strip_width();
-template <typename Real, typename Store, int QF, int QT> int resident_ctas();
-// Rows per segment the step kernel picks when none is set (whole waves of resident CTAs).
+// Rows per segment of the march when none is set (whole waves of resident CTAs).
 template <typename Real, typename Store, int QF, int QT> int auto_segment(int nx, int ny);
+// Tile shape for a channel on a device with `sms` SMs.
+template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx, long long ny, int sms, int *tx, int *ty);
 
 // Initialisation: macro [5][ny][nx] (phi, u, v, T, dp) holds the fields; entries whose
 // bit in `defaults` (1 phi, 2 u, 4 v, 8 T, 16 dp) is set are filled with the defaults

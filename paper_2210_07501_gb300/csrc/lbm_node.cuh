@@ -1,0 +1,248 @@
+// lbm_node.cuh -- what the step kernels share: the loads of the pull with the wall rules, the
+// stencils on rows in shared memory and the update of one node (forces, macros, the three
+// collisions, the stores), in one order of operations, so that every kernel gives the
+// same bits.
+#pragma once
+
+#include "lbm_device.cuh"
+
+namespace lbm {
+
+template <typename Real> struct Vec2;
+template <> struct Vec2<float> { using T = float2; };
+template <> struct Vec2<double> { using T = double2; };
+
+// The RX_N reference values of a staged row (16-byte aligned) in registers: two or four
+// 16-byte loads instead of one load per value.
+template <typename Real>
+__device__ __forceinline__ void load_rowref_(const Real *rx, Real *v)
+{
+    if constexpr (std::is_same<Real, float>::value) {
+        const float4 a = reinterpret_cast<const float4 *>(rx)[0], b = reinterpret_cast<const float4 *>(rx)[1];
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < RX_N / 2; ++i) {
+            const double2 d = reinterpret_cast<const double2 *>(rx)[i];
+            v[2 * i] = d.x, v[2 * i + 1] = d.y;
+        }
+    }
+}
+static_assert(RX_N == 8, "load_rowref_ reads eight values");
+
+template <typename Real>
+__device__ __forceinline__ void grad3_(const Real *rm, const Real *r0, const Real *rp, int c, Real &gx, Real &gy)
+{
+    const Real c1 = Real(1.0 / 3.0), c2 = Real(1.0 / 12.0);
+    if constexpr (std::is_same<Real, float>::value) {
+        // diagonal terms from (NE, NW) +- (SE, SW): (NE + SE) - (NW + SW) and
+        // (NE - SE) + (NW - SW), both halves of a pair in one packed instruction
+        const float2 P = f2_(rp[c + 1], rp[c - 1]), Q = f2_(rm[c + 1], rm[c - 1]);
+        const float2 S = add2_(P, Q), D = sub2_(P, Q);
+        const float2 G = fma2_(bc2_(c1), f2_(r0[c + 1] - r0[c - 1], rp[c] - rm[c]),
+                               mul2_(bc2_(c2), f2_(S.x - S.y, D.x + D.y)));
+        gx = G.x, gy = G.y;
+        return;
+    }
+    const Real ne = rp[c + 1], nw = rp[c - 1], se = rm[c + 1], sw = rm[c - 1];
+    gx = c1 * (r0[c + 1] - r0[c - 1]) + c2 * ((ne - nw) + (se - sw));
+    gy = c1 * (rp[c] - rm[c]) + c2 * ((ne - se) + (nw - sw));
+}
+
+// Loads of one node for the pull: populations of one lattice (plane base pointers `pl`,
+// wall rule KIND) at row y and column x, with the wall rules of Sec. 5.1.  Offsets are
+// 32-bit element indices.  WALLS = false: no link of the row crosses a wall.
+//   KIND 0: phase field, specular reflection (free slip, no flux through the wall)
+//   KIND 1: flow, halfway bounce-back (no slip)
+//   KIND 2: energy, anti-bounce-back to the wall temperature where the link crosses the wall
+// Values come out in stored units (for FP16 storage: times its scale; wscale multiplies
+// the anti-bounce-back wall term accordingly).
+template <int KIND, int Q, bool WALLS = true, typename Real, typename Store>
+__device__ __forceinline__ void pull_row_(const Store *const *pl, int pitch, int ny, int nx, int y, int x, int xm,
+                                          int xp, Real wscale, const Real *__restrict__ twall, Real dTcold, Real *out)
+{
+    const int r0 = y * pitch;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const int ex = ex_(a), ey = ey_(a);
+        const int xs = ex > 0 ? xm : (ex < 0 ? xp : x);
+        const bool wall = WALLS && ((ey > 0 && y == 0) || (ey < 0 && y == ny - 1));
+        Real v;
+        if (!wall) {
+            const int rs = ey > 0 ? r0 - pitch : (ey < 0 ? r0 + pitch : r0);
+            v = ld_<Real, Store>(pl[a] + (rs + xs));
+        } else if (KIND == 0) {
+            v = ld_<Real, Store>(pl[mir_(a)] + (r0 + xs));
+        } else {
+            v = ld_<Real, Store>(pl[opp_(a)] + (r0 + x));
+        }
+        if (KIND == 2 && wall) {
+            const Real tw = ey > 0 ? twall[(1 - ex) * nx + x] : dTcold;
+            Real t = Real(2.0 * w_<Q>(a)) * tw;
+            if constexpr (scaled_<Store>()) t *= wscale;
+            v = -v + t;
+        }
+        out[a] = v;
+    }
+}
+
+// Pulled populations of one lattice -> what the step keeps of them, in one order of
+// operations for every kernel (FP16 storage: the sums are rescaled, not each value).
+// phi - phi0 of a row from the pulled deviations and that row's dR (high and low parts)
+template <int QF, typename Real, typename Store>
+__device__ __forceinline__ Real phi_dev_(const StepArgs<Real, Store> &A, const Real *f, Real dr, Real drlo)
+{
+    Real dphi = f[0];
+#pragma unroll
+    for (int a = 1; a < QF; ++a) dphi += f[a];
+    if constexpr (scaled_<Store>()) dphi *= A.isf;
+    if constexpr (std::is_same<Real, double>::value) return dphi + dr;
+    else return (dphi + drlo) + dr;
+}
+// T - T_ref
+template <int QT, typename Real, typename Store>
+__device__ __forceinline__ Real temp_dev_(const StepArgs<Real, Store> &A, const Real *h)
+{
+    Real dT = h[0];
+#pragma unroll
+    for (int a = 1; a < QT; ++a) dT += h[a];
+    if constexpr (scaled_<Store>()) dT *= A.ish;
+    return dT;
+}
+// (sigma - sigma0, p - p0) of row r at column x from dT of the pulled populations (of row r
+// itself, or of the row next to the wall for the ghost rows r = -1 and r = ny)
+template <typename Real, typename Store>
+__device__ __forceinline__ typename Vec2<Real>::T sig_p_(const StepArgs<Real, Store> &A, int r, int x, Real dT, Real dp)
+{
+    Real dTs = dT;
+    if (r == -1) dTs = Real(2) * A.twall[A.nx + x] - dT;   // T_ghost = 2 T_w - T_adjacent
+    else if (r == A.ny) dTs = Real(2) * A.P.dTcold - dT;
+    typename Vec2<Real>::T v;
+    v.x = dTs * (A.P.sigma1 + A.P.sigma2 * dTs);
+    v.y = dp;
+    return v;
+}
+// first raw moments of f, and (T - T_ref, first raw moments) of h
+template <int QF, typename Real, typename Store>
+__device__ __forceinline__ void keep_f_(const StepArgs<Real, Store> &A, const Real *f, Real *m)
+{
+    raw_first_<QF>(f, m[0], m[1]);
+    if constexpr (scaled_<Store>()) m[0] *= A.isf, m[1] *= A.isf;
+}
+template <int QT, typename Real, typename Store>
+__device__ __forceinline__ void keep_h_(const StepArgs<Real, Store> &A, const Real *h, Real dT, Real *m)
+{
+    m[0] = dT;
+    raw_first_<QT>(h, m[1], m[2]);
+    if constexpr (scaled_<Store>()) m[1] *= A.ish, m[2] *= A.ish;
+}
+// grad phi = grad (phi - phi0) + (0, d_y phi0) at column c of the phi - phi0 rows rm, r0, rp
+template <typename Real>
+__device__ __forceinline__ void grad_phi_(const Real *rm, const Real *r0, const Real *rp, int c, Real gref, Real &gx,
+                                          Real &gy)
+{
+    grad3_(rm, r0, rp, c, gx, gy);
+    gy += gref;
+}
+// the unit normal of a gradient as (n_x, n_y - 1)
+template <typename Real, typename R2 = typename Vec2<Real>::T>
+__device__ __forceinline__ R2 normal_(Real gx, Real gy, Real g2min)
+{
+    R2 n;
+    unit_normal_dev_(gx, gy, g2min, n.x, n.y);
+    return n;
+}
+
+// Row y, column x of the step: from phi - phi0 = dphi and grad phi = (gpx, gpy) of the node, the
+// unit normal (n_x, n_y - 1) and (sigma - sigma0, p - p0) around it (rows m, 0, p at column s),
+// what the collisions keep of the pulled populations (fm: first raw moments of f; hm: T - T_ref
+// and first raw moments of h; g: the nine flow populations) and the row's reference values,
+// the post-collision populations, the stored pressure and, if asked for, the fields.
+template <typename Real, typename Store, int QF, int QT, typename R2 = typename Vec2<Real>::T>
+__device__ __forceinline__ void node_step_(const StepArgs<Real, Store> &A, int x, int y, Real dphi, Real gpx, Real gpy,
+                                           int s, const R2 *nm, const R2 *n0, const R2 *np, const R2 *qm, const R2 *q0,
+                                           const R2 *qp, const Real *fm, const Real *hm, Real *g, Real phi_ref, Real th0,
+                                           Real c01)
+{
+    const Phys<Real> &P = A.P;
+    const Real c2 = Real(1.0 / 3.0), hf = Real(0.5);
+    constexpr bool SCALED = scaled_<Store>();
+    const Real phi = phi_ref + dphi;
+    const Real g2 = norm2_(gpx, gpy);
+    const R2 nC = n0[s], nE = n0[s + 1], nW = n0[s - 1], nN = np[s], nS = nm[s];
+    const R2 nNE = np[s + 1], nNW = np[s - 1], nSE = nm[s + 1], nSW = nm[s - 1];
+    const Real c1 = Real(1.0 / 3.0), cd = Real(1.0 / 12.0);
+    const R2 qE = q0[s + 1], qW = q0[s - 1], qN = qp[s], qS = qm[s];
+    const R2 qNE = qp[s + 1], qNW = qp[s - 1], qSE = qm[s + 1], qSW = qm[s - 1];
+    Real divn, dsx, dsy, dpx, dpy;
+    if constexpr (std::is_same<Real, float>::value) {
+        // the same stencils with the (n_x, n_y) and (sigma, p) halves paired; the
+        // diagonal terms of div n summed as (NE - SW) +- (SE - NW)
+        const float2 T1 = sub2_(nNE, nSW), T2 = sub2_(nSE, nNW);
+        divn = c1 * ((nE.x - nW.x) + (nN.y - nS.y)) + cd * ((T1.x + T2.x) + (T1.y - T2.y));
+        const float2 X = fma2_(bc2_(c1), sub2_(qE, qW), mul2_(bc2_(cd), add2_(sub2_(qNE, qNW), sub2_(qSE, qSW))));
+        const float2 Y = fma2_(bc2_(c1), sub2_(qN, qS), mul2_(bc2_(cd), add2_(sub2_(qNE, qSE), sub2_(qNW, qSW))));
+        dsx = X.x, dpx = X.y, dsy = Y.x, dpy = Y.y;
+    } else {
+        divn = c1 * (nE.x - nW.x) + cd * ((nNE.x - nNW.x) + (nSE.x - nSW.x)) + c1 * (nN.y - nS.y) +
+               cd * ((nNE.y - nSE.y) + (nNW.y - nSW.y));
+        dsx = c1 * (qE.x - qW.x) + cd * ((qNE.x - qNW.x) + (qSE.x - qSW.x));
+        dsy = c1 * (qN.x - qS.x) + cd * ((qNE.x - qSE.x) + (qNW.x - qSW.x));
+        dpx = c1 * (qE.y - qW.y) + cd * ((qNE.y - qNW.y) + (qSE.y - qSW.y));
+        dpy = c1 * (qN.y - qS.y) + cd * ((qNE.y - qSE.y) + (qNW.y - qSW.y));
+    }
+    const Real nxv = nC.x, nyv = Real(1) + nC.y;
+    const Real dT = hm[0];
+    const Real sigma = P.sigma0 + dT * (P.sigma1 + P.sigma2 * dT);
+    const Real Fsx = P.csf * (-sigma * g2 * divn * nxv + g2 * ((Real(1) - nxv * nxv) * dsx - nxv * nyv * dsy));
+    const Real Fsy = P.csf * (-sigma * g2 * divn * nyv + g2 * ((Real(1) - nyv * nyv) * dsy - nxv * nyv * dsx));
+    const Real Ftx = Fsx + P.Fx, Fty = Fsy + P.Fy;
+    const Real Fpx = -dpx + c2 * P.drho * gpx, Fpy = -dpy + c2 * P.drho * gpy;
+    const Real rho = P.rhoA + phi * P.drho;
+    const Real irho = rcp_(rho);
+    Real s0, sx, sy, r20, r02, r11;
+    flow_raw_moments_(g, s0, sx, sy, r20, r02, r11);
+    if constexpr (SCALED) s0 *= A.isg, sx *= A.isg, sy *= A.isg, r20 *= A.isg, r02 *= A.isg, r11 *= A.isg;
+    const Real irc2 = Real(3) * irho;
+    const Real ux = (sx + hf * c2 * Ftx) * irc2;
+    const Real uy = (sy + hf * c2 * Fty) * irc2;
+    const Real dp = s0 + hf * (Fpx * ux + Fpy * uy);
+    const Real om_nu = rcp_(Real(3) * (P.muA + phi * P.dmu) * irho + hf);
+    const Real om_T = rcp_(Real(3) * (P.kA + phi * P.dk) * irho + hf);
+    // theta(phi) - theta(phi0) = (4 / W) dphi (1 - 2 phi0 - dphi)
+    const Real dth = P.W4 * dphi * (Real(1) - Real(2) * phi_ref - dphi);
+    Real fo[QF], ho[QT];
+    // (FP16 storage: the results come out in stored units)
+    collide_phase_dev_<QF, Real, SCALED>(fo, fm[0], fm[1], dphi, phi, ux, uy, nxv, nC.y, th0, dth, c01,
+                                         P.Mphi, P.omega_phi, A.sf);
+    collide_flow_<Real, SCALED>(g, rho, dp, ux, uy, Fpx, Fpy, Ftx, Fty, om_nu, s0, sx, sy, r20, r02, r11, A.sg);
+    collide_energy_<QT, Real, SCALED>(ho, hm[1], hm[2], dT, ux, uy, P.T_ref, om_T, A.sh);
+    const int o = y * A.pitch + x;
+    // one unsigned 32-bit byte offset from every plane's base (measured 2 % faster than
+    // plane base + element index)
+    const uint32_t ob = uint32_t(o) * uint32_t(sizeof(Store));
+    auto at = [&](Store *base) { return reinterpret_cast<Store *>(reinterpret_cast<char *>(base) + ob); };
+#pragma unroll
+    for (int a = 0; a < QF; ++a) {
+        st_(at(A.fo[a]), fo[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        st_(at(A.go[a]), g[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < QT; ++a) {
+        st_(at(A.ho[a]), ho[a]);
+    }
+    A.dp_out[o] = dp;
+    if (A.macro) {
+        const long long N = (long long)A.nx * A.ny, m = (long long)y * A.nx + x;
+        A.macro[m] = A.phi0[y] + double(dphi);
+        A.macro[N + m] = double(ux);
+        A.macro[2 * N + m] = double(uy);
+        A.macro[3 * N + m] = double(P.T_ref) + double(dT);
+        A.macro[4 * N + m] = double(dp);
+    }
+}
+
+}  // namespace lbm

@@ -12,8 +12,8 @@
 // post-collision populations and p to the other buffer.
 // Populations live in SoA planes [Q][ny][pitch], x fastest: every pull of a warp is a
 // contiguous (shifted) row segment.  No tensor cores: the step is a bandwidth-bound stencil.
-#include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_node.cuh"
 
 namespace lbm {
 
@@ -29,84 +29,6 @@ namespace lbm {
 // in shared memory filled by bulk copies D - 1 rows ahead (below); the first rows of a
 // segment are loaded directly.  Every thread works on the same row, so wall tests and row
 // addresses are uniform across the CTA; only 4 halo columns per strip are recomputed.
-template <typename Real> struct Vec2;
-template <> struct Vec2<float> { using T = float2; };
-template <> struct Vec2<double> { using T = double2; };
-
-// The RX_N reference values of a staged row (16-byte aligned) in registers: two or four
-// 16-byte loads instead of one load per value.
-template <typename Real>
-__device__ __forceinline__ void load_rowref_(const Real *rx, Real *v)
-{
-    if constexpr (std::is_same<Real, float>::value) {
-        const float4 a = reinterpret_cast<const float4 *>(rx)[0], b = reinterpret_cast<const float4 *>(rx)[1];
-        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
-    } else {
-#pragma unroll
-        for (int i = 0; i < RX_N / 2; ++i) {
-            const double2 d = reinterpret_cast<const double2 *>(rx)[i];
-            v[2 * i] = d.x, v[2 * i + 1] = d.y;
-        }
-    }
-}
-static_assert(RX_N == 8, "load_rowref_ reads eight values");
-
-template <typename Real>
-__device__ __forceinline__ void grad3_(const Real *rm, const Real *r0, const Real *rp, int c, Real &gx, Real &gy)
-{
-    const Real c1 = Real(1.0 / 3.0), c2 = Real(1.0 / 12.0);
-    if constexpr (std::is_same<Real, float>::value) {
-        // diagonal terms from (NE, NW) +- (SE, SW): (NE + SE) - (NW + SW) and
-        // (NE - SE) + (NW - SW), both halves of a pair in one packed instruction
-        const float2 P = f2_(rp[c + 1], rp[c - 1]), Q = f2_(rm[c + 1], rm[c - 1]);
-        const float2 S = add2_(P, Q), D = sub2_(P, Q);
-        const float2 G = fma2_(bc2_(c1), f2_(r0[c + 1] - r0[c - 1], rp[c] - rm[c]),
-                               mul2_(bc2_(c2), f2_(S.x - S.y, D.x + D.y)));
-        gx = G.x, gy = G.y;
-        return;
-    }
-    const Real ne = rp[c + 1], nw = rp[c - 1], se = rm[c + 1], sw = rm[c - 1];
-    gx = c1 * (r0[c + 1] - r0[c - 1]) + c2 * ((ne - nw) + (se - sw));
-    gy = c1 * (rp[c] - rm[c]) + c2 * ((ne - se) + (nw - sw));
-}
-
-// Loads of one row for the pull: populations of one lattice (plane base pointers `pl`,
-// wall rule KIND) at row y and column x, with the wall rules of Sec. 5.1.  Offsets are
-// 32-bit element indices; the row part is CTA-uniform.
-//   KIND 0: phase field, specular reflection (free slip, no flux through the wall)
-//   KIND 1: flow, halfway bounce-back (no slip)
-//   KIND 2: energy, anti-bounce-back to the wall temperature where the link crosses the wall
-// Values come out in stored units (for FP16 storage: times its scale; wscale multiplies
-// the anti-bounce-back wall term accordingly).
-template <int KIND, int Q, typename Real, typename Store>
-__device__ __forceinline__ void pull_row_(const Store *const *pl, int pitch, int ny, int nx, int y, int x, int xm,
-                                          int xp, Real wscale, const Real *__restrict__ twall, Real dTcold, Real *out)
-{
-    const int r0 = y * pitch;
-#pragma unroll
-    for (int a = 0; a < Q; ++a) {
-        const int ex = ex_(a), ey = ey_(a);
-        const int xs = ex > 0 ? xm : (ex < 0 ? xp : x);
-        const bool wall = (ey > 0 && y == 0) || (ey < 0 && y == ny - 1);
-        Real v;
-        if (!wall) {
-            const int rs = ey > 0 ? r0 - pitch : (ey < 0 ? r0 + pitch : r0);
-            v = ld_<Real, Store>(pl[a] + (rs + xs));
-        } else if (KIND == 0) {
-            v = ld_<Real, Store>(pl[mir_(a)] + (r0 + xs));
-        } else {
-            v = ld_<Real, Store>(pl[opp_(a)] + (r0 + x));
-        }
-        if (KIND == 2 && wall) {
-            const Real tw = ey > 0 ? twall[(1 - ex) * nx + x] : dTcold;
-            Real t = Real(2.0 * w_<Q>(a)) * tw;
-            if constexpr (scaled_<Store>()) t *= wscale;
-            v = -v + t;
-        }
-        out[a] = v;
-    }
-}
-
 // ---- asynchronous row staging ----------------------------------------------------------
 // The population rows a CTA pulls from are copied into shared memory by the bulk-copy (TMA)
 // engine, D - 1 output rows ahead of the row being collided: the loads hold no registers
@@ -334,8 +256,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         }
     };
     // Pulled values of a completed stage at the thread's columns (wall rules of Sec. 5.1), in
-    // stored units: with FP16 storage the sums and moments formed from them are rescaled
-    // (put_phi_dr, put_sig, keep_f, keep_h, the flow's moments), not each value.
+    // stored units (lbm_node.cuh rescales the sums and moments formed from FP16 values).
     constexpr bool SCALED = scaled_<Store>();
     auto read_f = [&](int sl, Real *f) {
         const Store *st = stage_pop(sl) + HS + cf;
@@ -385,16 +306,9 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         pull_row_<2, QT>(A.hi, pitch, ny, nx, gy, xh, xhm, xhp, A.sh, A.twall, P.dTcold, h);
         dp = A.dp_in[gy * pitch + xh];
     };
-    // phi - phi0 of row r (ghost rows: of the mirrored row) from the pulled deviations and
-    // that row's dR (high and low parts)
+    // rows into the rings (ghost rows of phi: of the mirrored row)
     auto put_phi_dr = [&](int r, const Real *f, Real dr, Real drlo) {
-        Real dphi = f[0];
-#pragma unroll
-        for (int a = 1; a < QF; ++a) dphi += f[a];
-        if constexpr (SCALED) dphi *= A.isf;
-        if constexpr (std::is_same<Real, double>::value) dphi += dr;
-        else dphi = (dphi + drlo) + dr;
-        s_phi[r & 7][cf + 2] = dphi;
+        s_phi[r & 7][cf + 2] = phi_dev_<QF>(A, f, dr, drlo);
     };
     auto put_phi = [&](int r, const Real *f) {
         const int gy = mirror_row_(r, ny);
@@ -402,37 +316,16 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
     };
     // returns T - T_ref of the pulled populations (of row r itself, not the ghost value)
     auto put_sig = [&](int r, const Real *h, Real dp) -> Real {
-        Real dT = h[0];
-#pragma unroll
-        for (int a = 1; a < QT; ++a) dT += h[a];
-        if constexpr (SCALED) dT *= A.ish;
-        Real dTs = dT;
-        if (r == -1) dTs = Real(2) * A.twall[nx + xh] - dT;   // T_ghost = 2 T_w - T_adjacent
-        else if (r == ny) dTs = Real(2) * P.dTcold - dT;
-        R2 v;
-        v.x = dTs * (P.sigma1 + P.sigma2 * dTs);
-        v.y = dp;
-        s_sp[r & 3][ch + 1] = v;
+        const Real dT = temp_dev_<QT>(A, h);
+        s_sp[r & 3][ch + 1] = sig_p_(A, r, xh, dT, dp);
         return dT;
     };
-    // what the collisions keep of pulled populations: first raw moments of f, and
-    // (T - T_ref, first raw moments) of h
-    auto keep_f = [&](const Real *f, Real *m) {
-        raw_first_<QF>(f, m[0], m[1]);
-        if constexpr (SCALED) m[0] *= A.isf, m[1] *= A.isf;
-    };
-    auto keep_h = [&](const Real *h, Real dT, Real *m) {
-        m[0] = dT;
-        raw_first_<QT>(h, m[1], m[2]);
-        if constexpr (SCALED) m[1] *= A.ish, m[2] *= A.ish;
-    };
-    // grad phi = grad (phi - phi0) + (0, d_y phi0); the normal as (n_x, n_y - 1)
+    auto keep_f = [&](const Real *f, Real *m) { keep_f_<QF>(A, f, m); };
+    auto keep_h = [&](const Real *h, Real dT, Real *m) { keep_h_<QT>(A, h, dT, m); };
     auto put_n_g = [&](int r, Real gref) {
         Real gx, gy;
-        R2 n;
-        grad3_(s_phi[(r - 1) & 7], s_phi[r & 7], s_phi[(r + 1) & 7], ch + 2, gx, gy);
-        unit_normal_dev_(gx, gy + gref, P.g2min, n.x, n.y);
-        s_n[r & 3][ch + 1] = n;
+        grad_phi_(&s_phi[(r - 1) & 7][0], &s_phi[r & 7][0], &s_phi[(r + 1) & 7][0], ch + 2, gref, gx, gy);
+        s_n[r & 3][ch + 1] = normal_(gx, gy, P.g2min);
     };
     auto put_n = [&](int r) { put_n_g(r, __ldg(t_gref + r)); };
     // After a wait gave up: flag the fault, let the copies this CTA started land, return.
@@ -457,6 +350,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         s_abort = 0;
         mbar_init_fence_();
     }
+    pdl_wait_();
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < D - 1; ++k) issue(y0 + k, k);
@@ -492,7 +386,6 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         put_n(y0);
     }
 
-    const Real c2 = Real(1.0 / 3.0), hf = Real(0.5);
     int sl = 0;          // slot of the stage of row y
     uint32_t par = 0;    // its mbarrier phase parity
     // One barrier per row: before it, phi of row y + 3, sigma and p of row y + 1 and the
@@ -540,90 +433,11 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
             return;
         }
         if (xin) {
-            const int c = tid + 2, s = tid + 1;
-            const Real *pm = s_phi[(y - 1) & 7], *p0 = s_phi[y & 7], *pp = s_phi[(y + 1) & 7];
-            const Real dphi = p0[c];
-            const Real phi = phi_ref + dphi;
             Real gpx, gpy;
-            grad3_(pm, p0, pp, c, gpx, gpy);
-            gpy += gref;
-            const Real g2 = gpx * gpx + gpy * gpy;
-            const R2 *nm = s_n[(y - 1) & 3], *n0 = s_n[y & 3], *np = s_n[(y + 1) & 3];
-            const R2 *qm = s_sp[(y - 1) & 3], *q0 = s_sp[y & 3], *qp = s_sp[(y + 1) & 3];
-            const R2 nC = n0[s], nE = n0[s + 1], nW = n0[s - 1], nN = np[s], nS = nm[s];
-            const R2 nNE = np[s + 1], nNW = np[s - 1], nSE = nm[s + 1], nSW = nm[s - 1];
-            const Real c1 = Real(1.0 / 3.0), cd = Real(1.0 / 12.0);
-            const R2 qE = q0[s + 1], qW = q0[s - 1], qN = qp[s], qS = qm[s];
-            const R2 qNE = qp[s + 1], qNW = qp[s - 1], qSE = qm[s + 1], qSW = qm[s - 1];
-            Real divn, dsx, dsy, dpx, dpy;
-            if constexpr (std::is_same<Real, float>::value) {
-                // the same stencils with the (n_x, n_y) and (sigma, p) halves paired; the
-                // diagonal terms of div n summed as (NE - SW) +- (SE - NW)
-                const float2 T1 = sub2_(nNE, nSW), T2 = sub2_(nSE, nNW);
-                divn = c1 * ((nE.x - nW.x) + (nN.y - nS.y)) + cd * ((T1.x + T2.x) + (T1.y - T2.y));
-                const float2 X = fma2_(bc2_(c1), sub2_(qE, qW), mul2_(bc2_(cd), add2_(sub2_(qNE, qNW), sub2_(qSE, qSW))));
-                const float2 Y = fma2_(bc2_(c1), sub2_(qN, qS), mul2_(bc2_(cd), add2_(sub2_(qNE, qSE), sub2_(qNW, qSW))));
-                dsx = X.x, dpx = X.y, dsy = Y.x, dpy = Y.y;
-            } else {
-                divn = c1 * (nE.x - nW.x) + cd * ((nNE.x - nNW.x) + (nSE.x - nSW.x)) + c1 * (nN.y - nS.y) +
-                       cd * ((nNE.y - nSE.y) + (nNW.y - nSW.y));
-                dsx = c1 * (qE.x - qW.x) + cd * ((qNE.x - qNW.x) + (qSE.x - qSW.x));
-                dsy = c1 * (qN.x - qS.x) + cd * ((qNE.x - qSE.x) + (qNW.x - qSW.x));
-                dpx = c1 * (qE.y - qW.y) + cd * ((qNE.y - qNW.y) + (qSE.y - qSW.y));
-                dpy = c1 * (qN.y - qS.y) + cd * ((qNE.y - qSE.y) + (qNW.y - qSW.y));
-            }
-            const Real nxv = nC.x, nyv = Real(1) + nC.y;
-            const Real dT = hm0[0];
-            const Real sigma = P.sigma0 + dT * (P.sigma1 + P.sigma2 * dT);
-            const Real Fsx = P.csf * (-sigma * g2 * divn * nxv + g2 * ((Real(1) - nxv * nxv) * dsx - nxv * nyv * dsy));
-            const Real Fsy = P.csf * (-sigma * g2 * divn * nyv + g2 * ((Real(1) - nyv * nyv) * dsy - nxv * nyv * dsx));
-            const Real Ftx = Fsx + P.Fx, Fty = Fsy + P.Fy;
-            const Real Fpx = -dpx + c2 * P.drho * gpx, Fpy = -dpy + c2 * P.drho * gpy;
-            const Real rho = P.rhoA + phi * P.drho;
-            const Real irho = rcp_(rho);
-            Real s0, sx, sy, r20, r02, r11;
-            flow_raw_moments_(g, s0, sx, sy, r20, r02, r11);
-            if constexpr (SCALED) s0 *= A.isg, sx *= A.isg, sy *= A.isg, r20 *= A.isg, r02 *= A.isg, r11 *= A.isg;
-            const Real irc2 = Real(3) * irho;
-            const Real ux = (sx + hf * c2 * Ftx) * irc2;
-            const Real uy = (sy + hf * c2 * Fty) * irc2;
-            const Real dp = s0 + hf * (Fpx * ux + Fpy * uy);
-            const Real om_nu = rcp_(Real(3) * (P.muA + phi * P.dmu) * irho + hf);
-            const Real om_T = rcp_(Real(3) * (P.kA + phi * P.dk) * irho + hf);
-            // theta(phi) - theta(phi0) = (4 / W) dphi (1 - 2 phi0 - dphi)
-            const Real dth = P.W4 * dphi * (Real(1) - Real(2) * phi_ref - dphi);
-            Real fo[QF], ho[QT];
-            // (FP16 storage: the results come out in stored units)
-            collide_phase_dev_<QF, Real, SCALED>(fo, fm0[0], fm0[1], dphi, phi, ux, uy, nxv, nC.y, th0, dth, c01,
-                                                 P.Mphi, P.omega_phi, A.sf);
-            collide_flow_<Real, SCALED>(g, rho, dp, ux, uy, Fpx, Fpy, Ftx, Fty, om_nu, s0, sx, sy, r20, r02, r11, A.sg);
-            collide_energy_<QT, Real, SCALED>(ho, hm0[1], hm0[2], dT, ux, uy, P.T_ref, om_T, A.sh);
-            const int o = y * pitch + x;
-            // one unsigned 32-bit byte offset from every plane's base (measured 2 % faster than
-            // plane base + element index)
-            const uint32_t ob = uint32_t(o) * uint32_t(sizeof(Store));
-            auto at = [&](Store *base) { return reinterpret_cast<Store *>(reinterpret_cast<char *>(base) + ob); };
-#pragma unroll
-            for (int a = 0; a < QF; ++a) {
-                st_(at(A.fo[a]), fo[a]);
-            }
-#pragma unroll
-            for (int a = 0; a < 9; ++a) {
-                st_(at(A.go[a]), g[a]);
-            }
-#pragma unroll
-            for (int a = 0; a < QT; ++a) {
-                st_(at(A.ho[a]), ho[a]);
-            }
-            A.dp_out[o] = dp;
-            if (A.macro) {
-                const long long N = (long long)nx * ny, m = (long long)y * nx + x;
-                A.macro[m] = A.phi0[y] + double(dphi);
-                A.macro[N + m] = double(ux);
-                A.macro[2 * N + m] = double(uy);
-                A.macro[3 * N + m] = double(P.T_ref) + double(dT);
-                A.macro[4 * N + m] = double(dp);
-            }
+            grad_phi_(&s_phi[(y - 1) & 7][0], &s_phi[y & 7][0], &s_phi[(y + 1) & 7][0], tid + 2, gref, gpx, gpy);
+            node_step_<Real, Store, QF, QT>(A, x, y, s_phi[y & 7][tid + 2], gpx, gpy, tid + 1, s_n[(y - 1) & 3],
+                                            s_n[y & 3], s_n[(y + 1) & 3], s_sp[(y - 1) & 3], s_sp[y & 3],
+                                            s_sp[(y + 1) & 3], fm0, hm0, g, phi_ref, th0, c01);
         }
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
@@ -637,8 +451,9 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
 }
 
 template <typename Real, typename Store, int QF, int QT, int TX>
-__global__ void __launch_bounds__(TX + 32, march_ctas<Real, Store>()) march_kernel(const StepArgs<Real, Store> A, int seg)
+__global__ void __launch_bounds__(TX + 32, march_ctas<Real, Store>()) march_kernel(const __grid_constant__ StepArgs<Real, Store> A, int seg)
 {
+    pdl_launch_next_();
     march_body<Real, Store, QF, QT, TX>(A, seg, blockIdx.x, blockIdx.y);
 }
 
@@ -650,8 +465,12 @@ __global__ void __launch_bounds__(TX + 32, batch_ctas<Real>()) batch_kernel(cons
                                                        const int4 *__restrict__ ctas, const int *__restrict__ active,
                                                        int seg)
 {
+    pdl_launch_next_();
     const int4 t = ctas[blockIdx.x];
-    if (!active[t.x]) return;
+    if (!active[t.x]) {
+        pdl_wait_();   // every CTA: the launch must end after the one before it
+        return;
+    }
     march_body<Real, Store, QF, QT, TX>(cases[t.x], seg, t.y, t.z);
 }
 
@@ -687,21 +506,8 @@ cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, i
                          cudaStream_t s)
 {
     constexpr int TX = march_width<Real>();
-    const int dyn = prepare_kernels<Real, Store, QF, QT>();
-    batch_kernel<Real, Store, QF, QT, TX><<<n_ctas, TX + 32, dyn, s>>>(cases, ctas, active, seg);
-    return cudaGetLastError();
-}
-
-template <typename Real, typename Store, int QF, int QT>
-int resident_ctas()
-{
-    constexpr int TX = march_width<Real>();
-    const int dyn = prepare_kernels<Real, Store, QF, QT>();
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<Real, Store, QF, QT, TX>, TX + 32, dyn);
-    return sms * (per_sm > 0 ? per_sm : 1);
+    PdlLaunch l(dim3(n_ctas), dim3(TX + 32), prepare_kernels<Real, Store, QF, QT>(), s);
+    return cudaLaunchKernelEx(&l.cfg, batch_kernel<Real, Store, QF, QT, TX>, cases, ctas, active, seg);
 }
 
 // Segment length: the one that minimises the estimated step time, waves of resident CTAs
@@ -751,23 +557,21 @@ int auto_segment(int nx, int ny)
 }
 
 template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_step(const StepArgs<Real, Store> &A, cudaStream_t s, int seg_rows)
+cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int rows)
 {
     constexpr int TX = march_width<Real>();
-    const int dyn = prepare_kernels<Real, Store, QF, QT>();
-    const int seg = seg_rows > 0 ? (seg_rows < A.ny ? seg_rows : A.ny) : auto_segment<Real, Store, QF, QT>(A.nx, A.ny);
-    dim3 grid((A.nx + TX - 1) / TX, (A.ny + seg - 1) / seg);
-    march_kernel<Real, Store, QF, QT, TX><<<grid, TX + 32, dyn, s>>>(A, seg);
-    return cudaGetLastError();
+    const int seg = rows < A.ny ? rows : A.ny;
+    PdlLaunch l(dim3((A.nx + TX - 1) / TX, (A.ny + seg - 1) / seg), dim3(TX + 32),
+                prepare_kernels<Real, Store, QF, QT>(), s);
+    return cudaLaunchKernelEx(&l.cfg, march_kernel<Real, Store, QF, QT, TX>, A, seg);
 }
 
 #define LBM_INST(R, S, QF, QT)                                                                              \
-    template cudaError_t launch_step<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, int);             \
+    template cudaError_t launch_march<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, int);            \
     template cudaError_t launch_batch<R, S, QF, QT>(const StepArgs<R, S> *, const int4 *, int, const int *, \
                                                     int, cudaStream_t);                                   \
     template int step_strip_width<R, S, QF, QT>();                                                         \
-    template int auto_segment<R, S, QF, QT>(int, int);                                                     \
-    template int resident_ctas<R, S, QF, QT>();
+    template int auto_segment<R, S, QF, QT>(int, int);
 LBM_INST(double, double, 5, 5)
 LBM_INST(double, double, 5, 9)
 LBM_INST(double, double, 9, 5)
