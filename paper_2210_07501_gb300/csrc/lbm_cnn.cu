@@ -18,14 +18,12 @@
 #include <vector>
 
 #include "../../include/lbm_gb300.h"
+#include "lbm_pdl.h"
 
 namespace {
 
 constexpr int NL = 6;
 constexpr int CH[NL + 1] = {12, 32, 32, 32, 32, 32, 4};
-constexpr int TILE = 16;       // 16 x 16 output pixels per CTA
-constexpr int CCH = 8;         // input channels staged per pass
-
 template <typename A> __device__ __forceinline__ float to_f(A v)
 {
     if constexpr (std::is_same<A, __nv_bfloat16>::value) return __bfloat162float(v);
@@ -36,6 +34,18 @@ template <typename A> __device__ __forceinline__ A from_f(float v)
     if constexpr (std::is_same<A, __nv_bfloat16>::value) return __float2bfloat16_rn(v);
     else return v;
 }
+// an input value as the activation type holds it; a result as the output holds it (rounded
+// to the activation type also where it is handed out in float)
+template <typename A, typename In> __device__ __forceinline__ float load_as(In v)
+{
+    if constexpr (std::is_same<In, A>::value) return to_f(v);
+    else return to_f(from_f<A>(v));
+}
+template <typename A, typename Out> __device__ __forceinline__ Out store_as(float v)
+{
+    if constexpr (std::is_same<Out, A>::value) return from_f<A>(v);
+    else return to_f(from_f<A>(v));
+}
 __device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
 __device__ __forceinline__ float dsilu(float z)
 {
@@ -43,164 +53,280 @@ __device__ __forceinline__ float dsilu(float z)
     return s * (1.0f + z * (1.0f - s));
 }
 
-// y[b][co][h][w] = bias[co] + sum_{ci, dy, dx} w[co][ci][dy][dx] * a[b][ci][h+dy-1][w+dx-1],
-// a = x (layer 0) or silu(x) (later layers).
-template <int CIN, int COUT, typename A>
-__global__ void __launch_bounds__(TILE *TILE) conv_fwd(const A *__restrict__ x, const float *__restrict__ wgt,
-                                                       const float *__restrict__ bias, A *__restrict__ y, int H, int W,
-                                                       int act_in)
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// ---- 3x3 convolutions on the FP32 pipes ----------------------------------------------------
+// Forward (BWD = false): y[b][co][h][w] = bias[co] + sum_{ci, dy, dx} w[co][ci][dy][dx] a[b][ci][h+dy-1][w+dx-1],
+// a = x (first layer) or silu(x).  Data gradient (BWD = true): the same sum over the layer's output
+// channels with the kernel flipped, times silu'(z) of the pixel.
+//
+// Bound: FP32 multiply-adds (2.4 G per 32 -> 32 layer at batch 16 of 256 x 64: 62 us at 80 TFLOP/s).  The
+// weights are kept in FP32 and the sums in FP32 in one order (per input channel the nine taps in
+// sequence, then the channel's sum onto the accumulator), which the matrix units cannot give.
+// The weights come laid out as they are read: [input][tap][output], for the data gradient flipped and
+// with the layer's channels swapped (weight_place, kept by set_params and the Adam step).
+// A thread holds 4 pixels of a row x COG output channels: per weight quad from shared memory (one
+// 16-byte broadcast) 8 packed FMAs (two channels each), per input channel 18 input values for 36 taps.
+// 124 us a 32 -> 32 layer (304 us with one pixel a thread and one scalar FMA per weight read), half of
+// the FP32 peak; the rest is staging (silu and its division on every input, 1.3 times with the
+// halo) that the four CTAs per SM overlap only in part.  Tiles of 16 rows: 141 us.
+constexpr int CCH = 8;         // input channels staged per pass
+template <int CO, int COG_, int TWQ_, int TH_> struct Tile {
+    static constexpr int COG = COG_, TWQ = TWQ_, TH = TH_;   // channels a thread, pixel quads a row, rows
+    static constexpr int NC = TWQ * TH * (CO / COG);         // threads that compute
+    static constexpr int NT = NC < 128 ? 128 : NC;           // threads (all stage)
+};
+
+// The rows iy < ROWS (image rows h0 - 1 + iy, zero outside) and columns ix < COLS + 2 (image columns
+// w0 - 1 + ix, wrapped; columns past the wrapped one are zero, they are not used) of nc planes of x,
+// through f, into dst[c * PLANE + iy * PW + ix].  NT threads: COLS by row, then the two edge
+// columns; U loads of a thread in flight (one at a time left the kernels waiting for memory two
+// thirds of their time).
+template <int NT, int COLS, int ROWS, int PW, int PLANE, int U, typename In, typename F>
+__device__ __forceinline__ void stage_planes(const In *x, int nc, int h0, int w0, int H, int W, float *dst, F f)
 {
-    __shared__ float s_x[CCH][TILE + 2][TILE + 2];
-    __shared__ float s_w[COUT][CCH][9];
-    const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;
-    const int w0 = blockIdx.x * TILE, h0 = blockIdx.y * TILE, b = blockIdx.z;
-    const int wo = w0 + tx, ho = h0 + ty;
-    float acc[COUT];
+    constexpr int RG = NT / COLS;
+    const int col = threadIdx.x % COLS, ww0 = w0 + col, rows = nc * ROWS;
+    const int wc = ww0 < W ? ww0 : (ww0 == W ? 0 : -1);
+    for (int r0 = threadIdx.x / COLS; r0 < rows; r0 += RG * U) {
+        In v[U];
+        bool in[U];
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = bias[co];
-    for (int c0 = 0; c0 < CIN; c0 += CCH) {
-        const int nc = CIN - c0 < CCH ? CIN - c0 : CCH;
-        for (int e = threadIdx.x; e < CCH * (TILE + 2) * (TILE + 2); e += TILE * TILE) {
-            const int c = e / ((TILE + 2) * (TILE + 2)), r = e % ((TILE + 2) * (TILE + 2));
-            const int iy = r / (TILE + 2), ix = r % (TILE + 2);
-            const int hh = h0 + iy - 1, ww = (w0 + ix - 1 + W) % W;
-            float v = 0.0f;
-            if (c < nc && hh >= 0 && hh < H) {
-                v = to_f(x[(((long long)b * CIN + c0 + c) * H + hh) * W + ww]);
-                if (act_in) v = silu(v);
-            }
-            s_x[c][iy][ix] = v;
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * RG, c = r / ROWS, hh = h0 + r - c * ROWS - 1;
+            in[u] = r < rows && hh >= 0 && hh < H && wc >= 0;
+            if (in[u]) v[u] = x[((long long)c * H + hh) * W + wc];
         }
-        for (int e = threadIdx.x; e < COUT * CCH * 9; e += TILE * TILE) {
-            const int co = e / (CCH * 9), r = e % (CCH * 9), c = r / 9, k = r % 9;
-            s_w[co][c][k] = c < nc ? wgt[((co * CIN) + c0 + c) * 9 + k] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * RG, c = r / ROWS;
+            if (r < rows) dst[c * PLANE + (r - c * ROWS) * PW + col + 1] = in[u] ? f(v[u]) : 0.f;
         }
-        __syncthreads();
-        for (int c = 0; c < nc; ++c) {
-            float xv[9];
-#pragma unroll
-            for (int k = 0; k < 9; ++k) xv[k] = s_x[c][ty + k / 3][tx + k % 3];
-#pragma unroll
-            for (int co = 0; co < COUT; ++co) {
-                float s = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) s += s_w[co][c][k] * xv[k];
-                acc[co] += s;
-            }
-        }
-        __syncthreads();
     }
-    if (ho < H && wo < W)
+    for (int e = threadIdx.x; e < 2 * rows; e += NT) {
+        const int r = e >> 1, c = r / ROWS, hh = h0 + r - c * ROWS - 1, ix = e & 1 ? COLS + 1 : 0;
+        int ww = w0 - 1 + ix;
+        ww = ww < 0 ? W - 1 : (ww < W ? ww : (ww == W ? 0 : -1));
+        const bool in = hh >= 0 && hh < H && ww >= 0;
+        dst[c * PLANE + (r - c * ROWS) * PW + ix] = in ? f(x[((long long)c * H + hh) * W + ww]) : 0.f;
+    }
+}
+// 16-byte aligned words of global memory into shared memory (cp.async; stage_wait before use)
+template <int NT> __device__ __forceinline__ void stage_words(const float *src, int n4, float *dst)
+{
+    for (int e = threadIdx.x; e < n4; e += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + 4 * e)),
+                     "l"(src + 4 * e)
+                     : "memory");
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+template <int CI, int CO, typename T, bool BWD, bool ACT, typename In, typename A, typename Out>
+__global__ void __launch_bounds__(T::NT, 512 / T::NT)
+conv3x3(const In *x, const float *wgt, const float *bias, const A *zin, Out *y, int H, int W)
+{
+    constexpr int COG = T::COG, TWQ = T::TWQ, TH = T::TH, NT = T::NT;
+    constexpr int PW = TWQ * 4 + 4, PLANE = (TH + 2) * PW;
+    __shared__ __align__(16) float s_x[CCH * PLANE];
+    __shared__ __align__(16) float s_w[CCH * 9 * CO];
+    const int q = threadIdx.x % TWQ, row = threadIdx.x / TWQ % TH, cg = threadIdx.x / (TWQ * TH);
+    const bool on = T::NC == NT || threadIdx.x < T::NC;
+    const int w0 = blockIdx.x * (TWQ * 4), h0 = blockIdx.y * TH, b = blockIdx.z;
+    lbm::pdl_wait_();   // (no __restrict__: nothing may be read before the wait)
+    float2 acc[4][COG / 2];
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) y[(((long long)b * COUT + co) * H + ho) * W + wo] = from_f<A>(acc[co]);
+    for (int j = 0; j < COG / 2; ++j) {
+        const float2 v = BWD || !on ? f2(0.f, 0.f) : f2(bias[cg * COG + 2 * j], bias[cg * COG + 2 * j + 1]);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) acc[p][j] = v;
+    }
+    for (int c0 = 0; c0 < CI; c0 += CCH) {
+        const int nc = CI - c0 < CCH ? CI - c0 : CCH;
+        if (c0) __syncthreads();
+        stage_words<NT>(wgt + c0 * 9 * CO, nc * 9 * CO / 4, s_w);
+        stage_planes<NT, TWQ * 4, TH + 2, PW, PLANE, (TWQ > 4 ? 10 : 5)>(
+            x + ((long long)b * CI + c0) * H * W, nc, h0, w0, H, W, s_x, [](In v) {
+                const float u = BWD ? to_f(v) : load_as<A>(v);
+                return ACT ? silu(u) : u;
+            });
+        stage_wait();
+        __syncthreads();
+        if (!on) continue;
+#pragma unroll 1
+        for (int c = 0; c < nc; ++c) {
+            const float *xs = s_x + c * PLANE + row * PW + 4 * q;
+            float xv[3][6];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 u = *reinterpret_cast<const float4 *>(xs + i * PW);
+                const float2 v = *reinterpret_cast<const float2 *>(xs + i * PW + 4);
+                xv[i][0] = u.x, xv[i][1] = u.y, xv[i][2] = u.z, xv[i][3] = u.w, xv[i][4] = v.x, xv[i][5] = v.y;
+            }
+            const float *ws = s_w + c * 9 * CO + cg * COG;
+#pragma unroll
+            for (int j = 0; j < COG / 2; j += 2) {
+                float2 sa[4], sb[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) sa[p] = sb[p] = f2(0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float4 u = *reinterpret_cast<const float4 *>(ws + k * CO + 2 * j);
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const float v = xv[k / 3][k % 3 + p];
+                        sa[p] = fma2(f2(u.x, u.y), f2(v, v), sa[p]);
+                        sb[p] = fma2(f2(u.z, u.w), f2(v, v), sb[p]);
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    acc[p][j] = __fadd2_rn(acc[p][j], sa[p]);
+                    acc[p][j + 1] = __fadd2_rn(acc[p][j + 1], sb[p]);
+                }
+            }
+        }
+    }
+    lbm::pdl_launch_next_();
+    const int ho = h0 + row, wo = w0 + 4 * q;
+    if (!on || ho >= H) return;
+#pragma unroll
+    for (int j = 0; j < COG; ++j) {
+        const long long o = (((long long)b * CO + cg * COG + j) * H + ho) * W + wo;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            if (wo + p < W) {
+                const float v = j & 1 ? acc[p][j / 2].y : acc[p][j / 2].x;
+                if constexpr (BWD) y[o + p] = v * dsilu(to_f(zin[o + p]));
+                else y[o + p] = store_as<A, Out>(v);
+            }
+    }
 }
 
-// da[b][ci][h][w] = sum_{co, dy, dx} w[co][ci][dy][dx] * dz[b][co][h-dy+1][w-dx+1]; then, for
-// layers after the first, dz_in = da * silu'(z_in).
-template <int CIN, int COUT, typename A>
-__global__ void __launch_bounds__(TILE *TILE) conv_bwd_data(const float *__restrict__ dz, const float *__restrict__ wgt,
-                                                            const A *__restrict__ zin, float *__restrict__ dzin, int H,
-                                                            int W)
+// ---- weight and bias gradients -------------------------------------------------------------
+// dw[co][ci][k] = sum_p a[ci][p + k] dz[co][p], db[co] = sum_p dz[co][p], over all pixels.  A contraction
+// over the pixels with 32 x 288 results: a thread holds 4 output channels x 1 input channel x 9 taps, each as
+// the packed sums of its even and odd columns (72 registers); per four pixels 72 packed FMAs on 3 + 4
+// 16-byte shared loads (the inputs by lane, the dz by broadcast).  A CTA walks over tiles of 8 x 32
+// pixels: the sums of a tile (128 terms each) are added to the CTA's, so no chain is longer than before
+// (256), and only gridDim partial sums reach memory (before: one per 16 x 16 tile, reduced by one
+// strided thread per result, 154 us a layer).  158 us a 32 -> 32 layer, 718 us with one FMA per two
+// shared loads.
+constexpr int GW = 32, GH = 8, GT = 256;
+constexpr int GP = GW + 4, GPLANE = (GH + 2) * GP + 4;   // plane stride = 4 x odd words: no bank conflicts
+static_assert(GPLANE % 32 % 8 == 4, "16-byte loads of 8 lanes must hit distinct banks");
+constexpr int GD = GH * GW;
+template <int CI, int CO> constexpr int grad_groups() { return GT / (CI * CO / 4) < GH ? GT / (CI * CO / 4) : GH; }
+template <int CI, int CO> constexpr size_t grad_smem() { return (CI * GPLANE + CO * GD) * sizeof(float); }
+
+template <int CI, int CO, bool ACT, typename In, typename A>
+__global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz, float *part, int H, int W, int B)
 {
-    __shared__ float s_d[CCH][TILE + 2][TILE + 2];
-    __shared__ float s_w[CIN][CCH][9];
-    const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;
-    const int w0 = blockIdx.x * TILE, h0 = blockIdx.y * TILE, b = blockIdx.z;
-    const int wo = w0 + tx, ho = h0 + ty;
-    float acc[CIN];
+    constexpr int NG = grad_groups<CI, CO>(), PER = CI * CO / 4, NW = CO * CI * 9;
+    constexpr int BL = GT / CO;   // threads per bias sum
+    extern __shared__ __align__(16) float s_a[];   // [CI][GPLANE], then dz [CO][GH][GW]
+    float *s_d = s_a + CI * GPLANE;
+    const int t = threadIdx.x, ci = t % CI, cog = t / CI % (CO / 4), grp = t / PER;
+    const bool on = grp < NG;
+    float tot[4][9], db = 0.f;
 #pragma unroll
-    for (int ci = 0; ci < CIN; ++ci) acc[ci] = 0.0f;
-    for (int c0 = 0; c0 < COUT; c0 += CCH) {
-        const int nc = COUT - c0 < CCH ? COUT - c0 : CCH;
-        for (int e = threadIdx.x; e < CCH * (TILE + 2) * (TILE + 2); e += TILE * TILE) {
-            const int c = e / ((TILE + 2) * (TILE + 2)), r = e % ((TILE + 2) * (TILE + 2));
-            const int iy = r / (TILE + 2), ix = r % (TILE + 2);
-            const int hh = h0 + iy - 1, ww = (w0 + ix - 1 + W) % W;
-            float v = 0.0f;
-            if (c < nc && hh >= 0 && hh < H) v = dz[(((long long)b * COUT + c0 + c) * H + hh) * W + ww];
-            s_d[c][iy][ix] = v;
-        }
-        for (int e = threadIdx.x; e < CIN * CCH * 9; e += TILE * TILE) {
-            const int ci = e / (CCH * 9), r = e % (CCH * 9), c = r / 9, k = r % 9;
-            s_w[ci][c][k] = c < nc ? wgt[(((c0 + c) * CIN) + ci) * 9 + (8 - k)] : 0.0f;   // flipped kernel
-        }
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) tot[i][k] = 0.f;
+    const int tw = (W + GW - 1) / GW, th = (H + GH - 1) / GH, tiles = tw * th * B;
+    lbm::pdl_wait_();
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int b = tile / (tw * th), r0 = tile - b * (tw * th), h0 = r0 / tw * GH, w0 = r0 % tw * GW;
         __syncthreads();
-        for (int c = 0; c < nc; ++c) {
-            float dv[9];
+        stage_planes<GT, GW, GH + 2, GP, GPLANE, 10>(x + (long long)b * CI * H * W, CI, h0, w0, H, W, s_a, [](In v) {
+            const float u = load_as<A>(v);
+            return ACT ? silu(u) : u;
+        });
+        for (int e = t; e < CO * GD; e += GT) {   // dz, zero outside: element-wise asynchronous copies
+            const int c = e / GD, r = e - c * GD, hh = h0 + r / GW, ww = w0 + r % GW;
+            const bool in = hh < H && ww < W;
+            const float *src = dz + (((long long)b * CO + c) * H + (in ? hh : 0)) * W + (in ? ww : 0);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(s_d + e)),
+                         "l"(src), "r"(in ? 4 : 0)
+                         : "memory");
+        }
+        stage_wait();
+        __syncthreads();
+        {
+            float s = 0.f;   // the thread's share of a bias sum: columns t % BL, + BL, ..
+            const float *d = s_d + t / BL * GD;
+            for (int p = t % BL; p < GD; p += BL) s += d[p];
+            db += s;
+        }
+        if (!on) continue;
+        float2 acc[4][9];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) dv[k] = s_d[c][ty + k / 3][tx + k % 3];
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int ci = 0; ci < CIN; ++ci) {
-                float s = 0.0f;
+            for (int k = 0; k < 9; ++k) acc[i][k] = f2(0.f, 0.f);
+#pragma unroll 1
+        for (int y = grp; y < GH; y += NG) {
+            const float *as = s_a + ci * GPLANE + y * GP, *ds = s_d + 4 * cog * GD + y * GW;
+            float4 cur[3];
 #pragma unroll
-                for (int k = 0; k < 9; ++k) s += s_w[ci][c][k] * dv[k];
-                acc[ci] += s;
+            for (int i = 0; i < 3; ++i) cur[i] = *reinterpret_cast<const float4 *>(as + i * GP);
+#pragma unroll 2
+            for (int c = 0; c < GW; c += 4) {
+                float4 d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) d[i] = *reinterpret_cast<const float4 *>(ds + i * GD + c);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const float4 u = cur[i], n = *reinterpret_cast<const float4 *>(as + i * GP + c + 4);
+                    const float2 p0[3] = {f2(u.x, u.y), f2(u.y, u.z), f2(u.z, u.w)};
+                    const float2 p1[3] = {f2(u.z, u.w), f2(u.w, n.x), f2(n.x, n.y)};
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            acc[o][3 * i + k] = fma2(p0[k], f2(d[o].x, d[o].y), acc[o][3 * i + k]);
+                            acc[o][3 * i + k] = fma2(p1[k], f2(d[o].z, d[o].w), acc[o][3 * i + k]);
+                        }
+                    cur[i] = n;
+                }
             }
         }
-        __syncthreads();
-    }
-    if (ho < H && wo < W)
 #pragma unroll
-        for (int ci = 0; ci < CIN; ++ci) {
-            const long long o = (((long long)b * CIN + ci) * H + ho) * W + wo;
-            dzin[o] = acc[ci] * dsilu(to_f(zin[o]));
-        }
-}
-
-// Partial weight and bias gradients of one 16 x 16 tile of one sample:
-// part[tile][co][ci][k] = sum_p a[ci][p + k] dz[co][p],  part_b[tile][co] = sum_p dz[co][p].
-template <int CIN, int COUT, typename A>
-__global__ void __launch_bounds__(TILE *TILE) conv_bwd_weight(const A *__restrict__ x, const float *__restrict__ dz,
-                                                              float *__restrict__ part, int H, int W, int act_in)
-{
-    extern __shared__ float smem[];
-    float *s_x = smem;                                        // [CIN][TILE+2][TILE+2]
-    float *s_d = smem + CIN * (TILE + 2) * (TILE + 2);        // [COUT][TILE][TILE]
-    const int w0 = blockIdx.x * TILE, h0 = blockIdx.y * TILE, b = blockIdx.z;
-    for (int e = threadIdx.x; e < CIN * (TILE + 2) * (TILE + 2); e += TILE * TILE) {
-        const int c = e / ((TILE + 2) * (TILE + 2)), r = e % ((TILE + 2) * (TILE + 2));
-        const int iy = r / (TILE + 2), ix = r % (TILE + 2);
-        const int hh = h0 + iy - 1, ww = (w0 + ix - 1 + W) % W;
-        float v = 0.0f;
-        if (hh >= 0 && hh < H) {
-            v = to_f(x[(((long long)b * CIN + c) * H + hh) * W + ww]);
-            if (act_in) v = silu(v);
-        }
-        s_x[e] = v;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) tot[i][k] += acc[i][k].x + acc[i][k].y;
     }
-    for (int e = threadIdx.x; e < COUT * TILE * TILE; e += TILE * TILE) {
-        const int c = e / (TILE * TILE), r = e % (TILE * TILE), iy = r / TILE, ix = r % TILE;
-        const int hh = h0 + iy, ww = w0 + ix;
-        s_d[e] = (hh < H && ww < W) ? dz[(((long long)b * COUT + c) * H + hh) * W + ww] : 0.0f;
+    lbm::pdl_launch_next_();
+    // the pixel groups' sums onto the first group's, in sequence, through shared memory
+    if constexpr (NG > 1) {
+        static_assert((NG - 1) * PER * 36 * sizeof(float) <= grad_smem<CI, CO>(), "the groups' sums fit the tile's memory");
+        __syncthreads();
+        if (on && grp > 0)
+#pragma unroll
+            for (int i = 0; i < 36; ++i) s_a[((grp - 1) * 36 + i) * PER + t % PER] = tot[i / 9][i % 9];
+        __syncthreads();
+        if (grp == 0)
+            for (int g = 0; g < NG - 1; ++g)
+#pragma unroll
+                for (int i = 0; i < 36; ++i) tot[i / 9][i % 9] += s_a[(g * 36 + i) * PER + t];
     }
+    float *out = part + (long long)blockIdx.x * (NW + CO);
+    if (grp == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) out[((4 * cog + i) * CI + ci) * 9 + k] = tot[i][k];
+#pragma unroll
+    for (int o = BL / 2 < 16 ? BL / 2 : 16; o > 0; o >>= 1) db += __shfl_down_sync(0xffffffffu, db, o);
+    constexpr int PB = BL > 32 ? BL / 32 : 1;   // warps per bias sum
     __syncthreads();
-    const int nw = COUT * CIN * 9, tiles = gridDim.x * gridDim.y * gridDim.z;
-    const int tile = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    for (int j = threadIdx.x; j < nw + COUT; j += TILE * TILE) {
-        float s = 0.0f;
-        if (j < nw) {
-            const int co = j / (CIN * 9), r = j % (CIN * 9), ci = r / 9, k = r % 9, ky = k / 3, kx = k % 3;
-            const float *xs = s_x + ci * (TILE + 2) * (TILE + 2);
-            const float *ds = s_d + co * TILE * TILE;
-            for (int py = 0; py < TILE; ++py)
-#pragma unroll 4
-                for (int px = 0; px < TILE; ++px) s += xs[(py + ky) * (TILE + 2) + px + kx] * ds[py * TILE + px];
-        } else {
-            const float *ds = s_d + (j - nw) * TILE * TILE;
-            for (int p = 0; p < TILE * TILE; ++p) s += ds[p];
-        }
-        part[(long long)j * tiles + tile] = s;
+    if (t % 32 % BL == 0) s_a[t / (BL < 32 ? BL : 32)] = db;
+    __syncthreads();
+    if (t < CO) {
+        float v = s_a[t * PB];
+        for (int i = 1; i < PB; ++i) v += s_a[t * PB + i];
+        out[NW + t] = v;
     }
-}
-
-// grad[j] = sum over tiles of part[j][tile], in tile order.
-__global__ void reduce_parts(const float *__restrict__ part, int tiles, int n, float *__restrict__ grad)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double s = 0.0;
-    for (int t = 0; t < tiles; ++t) s += part[(long long)j * tiles + t];
-    grad[j] = (float)s;
 }
 
 // MSE loss on the last layer: dz = 2 (y - t) / N; per-block partial sums of (y - t)^2.
@@ -224,31 +350,78 @@ __global__ void mse_grad(const A *__restrict__ y, const float *__restrict__ t, l
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void adam_step(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                          float *__restrict__ v, int n, float lr, float b1, float b2, float eps, float c1, float c2)
+// Where parameter i = weight [co][ci][k] of its layer goes in the two layouts the convolutions read;
+// false for a bias.
+struct Layers {
+    int n, off_w[NL], off_b[NL];
+};
+__device__ __forceinline__ bool weight_place(const Layers &L, int i, int &fwd, int &bwd)
+{
+    constexpr int ch[NL + 1] = {12, 32, 32, 32, 32, 32, 4};
+    int l = 0;
+    while (l + 1 < NL && i >= L.off_w[l + 1]) ++l;
+    if (i >= L.off_b[l]) return false;
+    const int r = i - L.off_w[l], co = r / (ch[l] * 9), ci = r / 9 % ch[l], k = r % 9;
+    fwd = L.off_w[l] + (ci * 9 + k) * ch[l + 1] + co;
+    bwd = L.off_w[l] + (co * 9 + 8 - k) * ch[l] + ci;
+    return true;
+}
+
+// grad[j] = sum over the n_part partial sums of its layer (layer l's lie at part + n_part off_w[l],
+// [n_part][parameters of the layer]), in a fixed order: 8 threads per result, each every 8th
+// partial sum, then the 8 in sequence.  The threads' sums carry their rounding errors along (two-sum:
+// as good as FP64, whose one pipe per SM alone would take 20 us for the 12.7 M terms of the largest
+// batch); the last eight are added in FP64.
+__global__ void __launch_bounds__(256) reduce_parts(const float *part, int n_part, Layers L, float *grad)
+{
+    __shared__ double sh[8][32];
+    const int lane = threadIdx.x % 32, g = threadIdx.x / 32, j = blockIdx.x * 32 + lane;
+    int l = 0;
+    while (l + 1 < NL && j >= L.off_w[l + 1]) ++l;
+    const int n = (l + 1 < NL ? L.off_w[l + 1] : L.n) - L.off_w[l];
+    const float *p0 = part + (long long)n_part * L.off_w[l] + (j - L.off_w[l]);
+    lbm::pdl_wait_();
+    float s = 0.f, c = 0.f;
+    if (j < L.n) {
+#pragma unroll 8
+        for (int p = g; p < n_part; p += 8) {
+            const float x = p0[(long long)p * n], t = s + x, z = t - s;
+            c += (s - (t - z)) + (x - z);
+            s = t;
+        }
+    }
+    sh[g][lane] = (double)s + (double)c;
+    __syncthreads();
+    if (g == 0 && j < L.n) {
+        double d = sh[0][lane];
+        for (int i = 1; i < 8; ++i) d += sh[i][lane];
+        grad[j] = (float)d;
+    }
+}
+
+__global__ void lay_out(const float *__restrict__ p, float *__restrict__ pf, float *__restrict__ pb, Layers L)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    int f, b;
+    if (i < L.n && weight_place(L, i, f, b)) pf[f] = p[i], pb[b] = p[i];
+}
+
+__global__ void adam_step(float *__restrict__ p, float *__restrict__ pf, float *__restrict__ pb,
+                          const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v, Layers L, float lr,
+                          float b1, float b2, float eps, float c1, float c2)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n) return;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+    int f, b;
+    if (weight_place(L, i, f, b)) pf[f] = pi, pb[b] = pi;
 }
-
-template <typename A> __global__ void to_act(const float *__restrict__ x, A *__restrict__ y, long long n)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = from_f<A>(x[i]);
-}
-template <typename A> __global__ void from_act(const A *__restrict__ x, float *__restrict__ y, long long n)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = to_f(x[i]);
-}
-
-int nparams_of_layer(int l) { return CH[l + 1] * CH[l] * 9 + CH[l + 1]; }
 
 }  // namespace
 
@@ -256,77 +429,97 @@ struct lbm_cnn {
     int H = 0, W = 0, Bmax = 0, bf16 = 1;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    int n_params = 0;
-    int off_w[NL], off_b[NL];
+    int n_params = 0, sms = 0;
+    Layers L;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;   // params, grads, Adam state
-    void *act[NL + 1] = {nullptr};    // act[0] = input, act[l+1] = pre-activation output of layer l
+    float *pf = nullptr, *pb = nullptr;   // the weights as the convolutions read them (weight_place)
+    void *act[NL + 1] = {nullptr};    // act[l+1] = pre-activation output of layer l (act[0]: the caller's input)
     float *dz[2] = {nullptr, nullptr};
-    float *part = nullptr;
-    long long part_cap = 0;
+    float *part = nullptr;            // partial weight gradients
     double *loss_part = nullptr, *loss_host = nullptr;
     int64_t t = 0;                    // Adam step
 };
 
 static thread_local char g_cnn_err[160] = "";
 
-template <typename A> static cudaError_t cnn_forward_impl(lbm_cnn *c, int B)
+template <typename K, typename... Args>
+static cudaError_t go(lbm_cnn *c, K kernel, dim3 grid, int block, size_t smem, Args... args)
 {
-    const dim3 grid((c->W + TILE - 1) / TILE, (c->H + TILE - 1) / TILE, B), blk(TILE * TILE);
-    for (int l = 0; l < NL; ++l) {
-        const A *x = (const A *)c->act[l];
-        A *y = (A *)c->act[l + 1];
-        const float *w = c->p + c->off_w[l], *bias = c->p + c->off_b[l];
-        const int act_in = l > 0;
-        if (l == 0) conv_fwd<CH[0], 32, A><<<grid, blk, 0, c->stream>>>(x, w, bias, y, c->H, c->W, act_in);
-        else if (CH[l + 1] == 32) conv_fwd<32, 32, A><<<grid, blk, 0, c->stream>>>(x, w, bias, y, c->H, c->W, act_in);
-        else conv_fwd<32, 4, A><<<grid, blk, 0, c->stream>>>(x, w, bias, y, c->H, c->W, act_in);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    lbm::PdlLaunch l(grid, dim3(block), smem, c->stream);
+    return cudaLaunchKernelEx(&l.cfg, kernel, args...);
 }
 
-template <int CIN, int COUT, typename A>
-static cudaError_t bwd_weight_launch(lbm_cnn *c, int l, int B, const float *dz)
+// One convolution.  Tiles of 32 x 8 pixels (16 channels a thread) where they fill the GPU, else of
+// 16 x 8 (8 channels a thread: half the pixels per CTA, 1.25 times the time per pixel).
+template <int CI, int CO, bool BWD, bool ACT, typename In, typename A, typename Out>
+static cudaError_t conv(lbm_cnn *c, int B, const In *x, const float *w, const float *bias, const A *zin, Out *y)
 {
-    const dim3 grid((c->W + TILE - 1) / TILE, (c->H + TILE - 1) / TILE, B), blk(TILE * TILE);
-    const size_t sm = (CIN * (TILE + 2) * (TILE + 2) + COUT * TILE * TILE) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(conv_bwd_weight<CIN, COUT, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    conv_bwd_weight<CIN, COUT, A><<<grid, blk, sm, c->stream>>>((const A *)c->act[l], dz, c->part, c->H, c->W, l > 0);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int n = nparams_of_layer(l), tiles = grid.x * grid.y * grid.z;
-    // weights then biases: the layer's parameters are contiguous (w, then b)
-    reduce_parts<<<(n + 255) / 256, 256, 0, c->stream>>>(c->part, tiles, n, c->g + c->off_w[l]);
-    return cudaGetLastError();
+    using Big = Tile<CO, CO < 16 ? CO : 16, 8, 8>;
+    using Small = Tile<CO, CO < 8 ? CO : 8, 4, 8>;
+    const dim3 gb((c->W + 31) / 32, (c->H + 7) / 8, B), gs((c->W + 15) / 16, (c->H + 7) / 8, B);
+    const long long nb = (long long)gb.x * gb.y * gb.z, ns = (long long)gs.x * gs.y * gs.z;
+    const double tb = 2.0 * ((nb + 4 * c->sms - 1) / (4 * c->sms)), ts = 1.25 * ((ns + 4 * c->sms - 1) / (4 * c->sms));
+    if (tb <= ts)
+        return go(c, conv3x3<CI, CO, Big, BWD, ACT, In, A, Out>, gb, Big::NT, 0, x, w, bias, zin, y, c->H, c->W);
+    return go(c, conv3x3<CI, CO, Small, BWD, ACT, In, A, Out>, gs, Small::NT, 0, x, w, bias, zin, y, c->H, c->W);
 }
 
-template <typename A> static cudaError_t cnn_backward_impl(lbm_cnn *c, int B, const float *target, double *loss)
+// Forward pass; the last layer's output goes to y (its activation type, or float).
+template <typename A, typename Out> static cudaError_t cnn_forward_impl(lbm_cnn *c, const float *x, int B, Out *y)
+{
+    const A *none = nullptr;
+    const float *w = c->pf, *p = c->p;
+    const int *ow = c->L.off_w, *ob = c->L.off_b;
+    cudaError_t e = conv<CH[0], 32, false, false>(c, B, x, w + ow[0], p + ob[0], none, (A *)c->act[1]);
+    for (int l = 1; l < NL - 1 && e == cudaSuccess; ++l)
+        e = conv<32, 32, false, true>(c, B, (const A *)c->act[l], w + ow[l], p + ob[l], none, (A *)c->act[l + 1]);
+    if (e == cudaSuccess)
+        e = conv<32, 4, false, true>(c, B, (const A *)c->act[NL - 1], w + ow[NL - 1], p + ob[NL - 1], none, y);
+    return e;
+}
+
+// Two CTAs per SM walk over the tiles (fewer where there are fewer tiles).
+static int grad_ctas(const lbm_cnn *c, int B)
+{
+    const long long tiles = (long long)((c->W + GW - 1) / GW) * ((c->H + GH - 1) / GH) * B;
+    return (int)(tiles < 2 * c->sms ? tiles : 2 * c->sms);
+}
+
+template <int CI, int CO, bool ACT, typename In, typename A>
+static cudaError_t conv_gradient(lbm_cnn *c, int l, int B, const In *x, const float *dz)
+{
+    constexpr size_t sm = grad_smem<CI, CO>();
+    auto *kernel = conv_grad<CI, CO, ACT, In, A>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const int ctas = grad_ctas(c, B);
+    if (e == cudaSuccess)
+        e = go(c, kernel, dim3(ctas), GT, sm, x, dz, c->part + (size_t)ctas * c->L.off_w[l], c->H, c->W, B);
+    return e;
+}
+
+template <typename A>
+static cudaError_t cnn_backward_impl(lbm_cnn *c, const float *x, int B, const float *target, double *loss)
 {
     const long long nout = (long long)B * CH[NL] * c->H * c->W;
     const int lb = 512;
     mse_grad<A><<<lb, 256, 0, c->stream>>>((const A *)c->act[NL], target, nout, c->dz[0], c->loss_part);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const dim3 grid((c->W + TILE - 1) / TILE, (c->H + TILE - 1) / TILE, B), blk(TILE * TILE);
-    int cur = 0;
-    for (int l = NL - 1; l >= 0; --l) {
-        const float *dz = c->dz[cur];
-        if (l == 0) e = bwd_weight_launch<CH[0], 32, A>(c, l, B, dz);
-        else if (CH[l + 1] == 32) e = bwd_weight_launch<32, 32, A>(c, l, B, dz);
-        else e = bwd_weight_launch<32, 4, A>(c, l, B, dz);
-        if (e != cudaSuccess) return e;
-        if (l > 0) {
-            float *dzin = c->dz[1 - cur];
-            const A *zin = (const A *)c->act[l];
-            if (CH[l + 1] == 32) conv_bwd_data<32, 32, A><<<grid, blk, 0, c->stream>>>(dz, c->p + c->off_w[l], zin, dzin, c->H, c->W);
-            else conv_bwd_data<32, 4, A><<<grid, blk, 0, c->stream>>>(dz, c->p + c->off_w[l], zin, dzin, c->H, c->W);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            cur = 1 - cur;
-        }
+    const float *w = c->pb, *none = nullptr;
+    const int *ow = c->L.off_w;
+    const A *in = (const A *)c->act[NL - 1];
+    if (e == cudaSuccess) e = conv_gradient<32, 4, true, A, A>(c, NL - 1, B, in, c->dz[0]);
+    if (e == cudaSuccess) e = conv<4, 32, true, false>(c, B, (const float *)c->dz[0], w + ow[NL - 1], none, in, c->dz[1]);
+    int cur = 1;
+    for (int l = NL - 2; l > 0 && e == cudaSuccess; --l, cur = 1 - cur) {
+        in = (const A *)c->act[l];
+        e = conv_gradient<32, 32, true, A, A>(c, l, B, in, c->dz[cur]);
+        if (e == cudaSuccess)
+            e = conv<32, 32, true, false>(c, B, (const float *)c->dz[cur], w + ow[l], none, in, c->dz[1 - cur]);
     }
+    if (e == cudaSuccess) e = conv_gradient<CH[0], 32, false, float, A>(c, 0, B, x, c->dz[cur]);
+    if (e == cudaSuccess)
+        e = go(c, reduce_parts, dim3((c->n_params + 31) / 32), 256, 0, (const float *)c->part, grad_ctas(c, B), c->L, c->g);
+    if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(c->loss_host, c->loss_part, lb * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return e;
     e = cudaStreamSynchronize(c->stream);
@@ -337,18 +530,16 @@ template <typename A> static cudaError_t cnn_backward_impl(lbm_cnn *c, int B, co
     return cudaSuccess;
 }
 
+static cudaError_t lay_out_weights(lbm_cnn *c)
+{
+    lay_out<<<(c->n_params + 255) / 256, 256, 0, c->stream>>>(c->p, c->pf, c->pb, c->L);
+    return cudaGetLastError();
+}
+
 static int cnn_fail(cudaError_t e, const char *what)
 {
     snprintf(g_cnn_err, sizeof(g_cnn_err), "%s: %s", what, cudaGetErrorString(e));
     return LBM_ECUDA;
-}
-
-static cudaError_t cnn_load_input(lbm_cnn *c, const float *x, int B)
-{
-    const long long n = (long long)B * CH[0] * c->H * c->W;
-    if (c->bf16) to_act<__nv_bfloat16><<<1024, 256, 0, c->stream>>>(x, (__nv_bfloat16 *)c->act[0], n);
-    else to_act<float><<<1024, 256, 0, c->stream>>>(x, (float *)c->act[0], n);
-    return cudaGetLastError();
 }
 
 extern "C" {
@@ -357,7 +548,7 @@ void lbm_cnn_destroy(lbm_cnn *c)
 {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    float *fs[] = {c->p, c->g, c->m, c->v, c->dz[0], c->dz[1], c->part};
+    float *fs[] = {c->p, c->pf, c->pb, c->g, c->m, c->v, c->dz[0], c->dz[1], c->part};
     for (float *f : fs)
         if (f) cudaFree(f);
     for (int l = 0; l <= NL; ++l)
@@ -386,21 +577,23 @@ int lbm_cnn_create(int32_t H, int32_t W, int32_t batch_max, int32_t bf16_activat
     }
     int off = 0;
     for (int l = 0; l < NL; ++l) {
-        c->off_w[l] = off;
+        c->L.off_w[l] = off;
         off += CH[l + 1] * CH[l] * 9;
-        c->off_b[l] = off;
+        c->L.off_b[l] = off;
         off += CH[l + 1];
     }
-    c->n_params = off;
+    c->n_params = c->L.n = off;
     const size_t asz = c->bf16 ? 2 : 4;
     const long long plane = (long long)H * W;
     bool ok = true;
-    for (float **f : {&c->p, &c->g, &c->m, &c->v}) ok = ok && cudaMalloc((void **)f, off * sizeof(float)) == cudaSuccess;
-    for (int l = 0; l <= NL && ok; ++l) ok = cudaMalloc(&c->act[l], (size_t)batch_max * CH[l] * plane * asz) == cudaSuccess;
+    for (float **f : {&c->p, &c->pf, &c->pb, &c->g, &c->m, &c->v}) ok = ok && cudaMalloc((void **)f, off * sizeof(float)) == cudaSuccess;
+    for (int l = 1; l <= NL && ok; ++l) ok = cudaMalloc(&c->act[l], (size_t)batch_max * CH[l] * plane * asz) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k) ok = cudaMalloc((void **)&c->dz[k], (size_t)batch_max * 32 * plane * sizeof(float)) == cudaSuccess;
-    const long long tiles = (long long)((W + TILE - 1) / TILE) * ((H + TILE - 1) / TILE) * batch_max;
-    c->part_cap = tiles * (32 * 32 * 9 + 32);
-    ok = ok && cudaMalloc((void **)&c->part, (size_t)c->part_cap * sizeof(float)) == cudaSuccess;
+    int dev = 0;
+    ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+    const size_t part_floats = (size_t)grad_ctas(c, batch_max) * off;
+    ok = ok && cudaMalloc((void **)&c->part, part_floats * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&c->loss_part, 512 * sizeof(double)) == cudaSuccess;
     ok = ok && cudaMallocHost((void **)&c->loss_host, 512 * sizeof(double)) == cudaSuccess;
     if (!ok) { cudaGetLastError(); lbm_cnn_destroy(c); return LBM_ENOMEM; }
@@ -412,12 +605,13 @@ int lbm_cnn_create(int32_t H, int32_t W, int32_t batch_max, int32_t bf16_activat
         for (int i = 0; i < CH[l + 1] * CH[l] * 9; ++i) {
             s = s * 6364136223846793005ULL + 1442695040888963407ULL;
             const double u01 = (double)(s >> 11) / 9007199254740992.0;
-            h[c->off_w[l] + i] = (float)((2.0 * u01 - 1.0) * a);
+            h[c->L.off_w[l] + i] = (float)((2.0 * u01 - 1.0) * a);
         }
     }
     cudaError_t e = cudaMemcpy(c->p, h.data(), off * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->m, 0, off * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(c->v, 0, off * sizeof(float));
+    if (e == cudaSuccess) e = lay_out_weights(c);
     if (e != cudaSuccess) { lbm_cnn_destroy(c); return LBM_ECUDA; }
     *out = c;
     return LBM_OK;
@@ -444,6 +638,7 @@ int lbm_cnn_set_params(lbm_cnn *c, const float *host)
     cudaError_t e = cudaMemcpyAsync(c->p, host, c->n_params * sizeof(float), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->m, 0, c->n_params * sizeof(float), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->v, 0, c->n_params * sizeof(float), c->stream);
+    if (e == cudaSuccess) e = lay_out_weights(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     c->t = 0;
     return e == cudaSuccess ? LBM_OK : cnn_fail(e, "lbm_cnn_set_params");
@@ -452,24 +647,18 @@ int lbm_cnn_set_params(lbm_cnn *c, const float *host)
 int lbm_cnn_forward(lbm_cnn *c, const float *x, int32_t B, float *y)
 {
     if (!c || !x || !y || B < 1 || B > c->Bmax) return LBM_EINVAL;
-    cudaError_t e = cnn_load_input(c, x, B);
-    if (e == cudaSuccess) e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, B) : cnn_forward_impl<float>(c, B);
-    const long long n = (long long)B * CH[NL] * c->H * c->W;
-    if (e == cudaSuccess) {
-        if (c->bf16) from_act<__nv_bfloat16><<<1024, 256, 0, c->stream>>>((const __nv_bfloat16 *)c->act[NL], y, n);
-        else from_act<float><<<1024, 256, 0, c->stream>>>((const float *)c->act[NL], y, n);
-        e = cudaGetLastError();
-    }
+    const cudaError_t e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, x, B, y) : cnn_forward_impl<float>(c, x, B, y);
     return e == cudaSuccess ? LBM_OK : cnn_fail(e, "lbm_cnn_forward");
 }
 
 int lbm_cnn_gradients(lbm_cnn *c, const float *x, const float *target, int32_t B, float *grad_host, double *loss)
 {
     if (!c || !x || !target || B < 1 || B > c->Bmax) return LBM_EINVAL;
-    cudaError_t e = cnn_load_input(c, x, B);
-    if (e == cudaSuccess) e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, B) : cnn_forward_impl<float>(c, B);
+    cudaError_t e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, x, B, (__nv_bfloat16 *)c->act[NL])
+                            : cnn_forward_impl<float>(c, x, B, (float *)c->act[NL]);
     if (e == cudaSuccess)
-        e = c->bf16 ? cnn_backward_impl<__nv_bfloat16>(c, B, target, loss) : cnn_backward_impl<float>(c, B, target, loss);
+        e = c->bf16 ? cnn_backward_impl<__nv_bfloat16>(c, x, B, target, loss)
+                    : cnn_backward_impl<float>(c, x, B, target, loss);
     if (e == cudaSuccess && grad_host) {
         e = cudaMemcpyAsync(grad_host, c->g, c->n_params * sizeof(float), cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -484,7 +673,8 @@ int lbm_cnn_train_step(lbm_cnn *c, const float *x, const float *target, int32_t 
     c->t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)c->t), c2 = 1.0f - powf(b2, (float)c->t);
-    adam_step<<<(c->n_params + 255) / 256, 256, 0, c->stream>>>(c->p, c->g, c->m, c->v, c->n_params, lr, b1, b2, 1e-8f, c1, c2);
+    adam_step<<<(c->n_params + 255) / 256, 256, 0, c->stream>>>(c->p, c->pf, c->pb, c->g, c->m, c->v, c->L, lr, b1,
+                                                                b2, 1e-8f, c1, c2);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? LBM_OK : cnn_fail(e, "lbm_cnn_train_step");
 }

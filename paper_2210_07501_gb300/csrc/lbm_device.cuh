@@ -24,6 +24,8 @@
 
 #include <type_traits>
 
+#include "lbm_pdl.h"
+
 namespace lbm {
 
 // ---- D2Q9 velocities (Sec. 4.1; velocity 8 is (+1,-1) as in App. B's P) ----
@@ -96,11 +98,6 @@ enum { RT_PHI0 = 0, RT_DR = 1, RT_GREF = 2, RT_TH0 = 3, RT_C01 = 4, RT_DRLO = 5,
 // fields of StepArgs::rowx for output row y: phi0(y), theta(phi0(y)), c01(y), d_y phi0(y),
 // dR of the mirrored row y + 3 (high, low), d_y phi0(y + 1), unused
 enum { RX_PHI0 = 0, RX_TH0 = 1, RX_C01 = 2, RX_GREF = 3, RX_DR3 = 4, RX_DR3LO = 5, RX_GREF1 = 6, RX_N = 8 };
-
-// Programmatic dependent launch: let the next launch of the stream start; wait for the complete
-// end of the previous one (no-ops in a launch without the attribute).
-__device__ __forceinline__ void pdl_launch_next_() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait_() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- storage conversion (plain loads, which stay behind pdl_wait_: the populations are
 // written by the launch before) ----

@@ -5,22 +5,9 @@
 #include <cuda_runtime.h>
 
 #include "lbm_device.cuh"
+#include "lbm_pdl.h"
 
 namespace lbm {
-
-// A launch that may start while the previous launch of its stream drains (the kernel calls
-// pdl_wait_ before it touches what that one wrote).
-struct PdlLaunch {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    PdlLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t s)
-    {
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = s;
-        cfg.attrs = at, cfg.numAttrs = 1;
-    }
-};
 
 // How a step is launched: rows > 0: row-marching strips, each CTA walking that many rows; else
 // 2-D tiles of tx x ty nodes.

@@ -62,3 +62,33 @@ def test_training_reduces_loss(pkg):
         last = net.train_step(x, t, 1e-3)
     assert last < 0.3 * first, (first, last)
     net.close()
+
+
+@pytest.mark.parametrize("B,H,W", [(1, 1, 3), (2, 9, 33), (3, 8, 17), (12, 33, 250)])
+def test_tiles_of_every_size_against_oracle(pkg, B, H, W):
+    """Outputs and gradients at the edges of the pixel tiles (16 x 8 and 32 x 8, ragged in both
+    directions), on the smallest image and on one whose tiles outnumber the CTAs, FP32 activations.
+    Bar: six layers of 288-term FP32 sums, 6 x 6e-8 x sqrt(288) = 6e-6, rounded up to 1e-5."""
+    from oracle import cnn as C
+    rng = np.random.default_rng(B * H + W)
+    net = pkg.Cnn(H, W, batch_max=B, bf16=False, seed=1)
+    p = rng.normal(scale=0.08, size=net.n_params).astype(np.float32)
+    net.set_params(p)
+    x = rng.normal(size=(B, 12, H, W)).astype(np.float32)
+    t = rng.normal(size=(B, 4, H, W)).astype(np.float32)
+    xd, td = torch.tensor(x, device="cuda"), torch.tensor(t, device="cuda")
+    yd = torch.empty((B, 4, H, W), dtype=torch.float32, device="cuda")
+    net.forward(xd, yd)
+    torch.cuda.synchronize()
+    L, g, y = C.loss_and_grad(p.astype(np.float64), x.astype(np.float64), t.astype(np.float64))
+    gg, loss = net.gradients(xd, td)
+    ef, eg = rel(yd.cpu().numpy(), y), rel(gg.astype(np.float64), g)
+    print(f"{B}x{H}x{W}: forward rel {ef:.2e}, gradient rel {eg:.2e}")
+    assert ef <= 1e-5 and eg <= 1e-5 and abs(loss - L) <= 1e-5 * abs(L)
+    # a step from these gradients moves the weights that the next forward pass reads
+    net.train_step(xd, td, 1e-2)
+    net.forward(xd, yd)
+    torch.cuda.synchronize()
+    _, _, y2 = C.loss_and_grad(net.get_params().astype(np.float64), x.astype(np.float64), t.astype(np.float64))
+    assert rel(yd.cpu().numpy(), y2) <= 1e-5
+    net.close()
