@@ -77,6 +77,7 @@ template <typename Real> static Phys<Real> cast_phys(const Phys<double> &d)
     Phys<Real> p;
     p.W4 = Real(d.W4);
     p.csf = Real(d.csf);
+    p.csf12 = Real(d.csf12);
     p.sigma0 = Real(d.sigma0);
     p.sigma1 = Real(d.sigma1);
     p.sigma2 = Real(d.sigma2);
@@ -88,6 +89,15 @@ template <typename Real> static Phys<Real> cast_phys(const Phys<double> &d)
     p.dmu = Real(d.dmu);
     p.kA = Real(d.kA);
     p.dk = Real(d.dk);
+    p.mu3A = Real(d.mu3A);
+    p.dmu3 = Real(d.dmu3);
+    p.k3A = Real(d.k3A);
+    p.dk3 = Real(d.dk3);
+    p.c2drho = Real(d.c2drho);
+    p.irhoA = Real(d.irhoA);
+    p.omnuA = Real(d.omnuA);
+    p.omTA = Real(d.omTA);
+    p.constant = d.constant;
     p.omega_phi = Real(d.omega_phi);
     p.Mphi = Real(d.Mphi);
     p.Fx = Real(d.Fx);
@@ -172,7 +182,8 @@ template <typename R, typename S, int QF, int QT> struct StepFn {
 // The march reads no row twice and reaches the copy bandwidth once its strips fill the GPU for
 // several waves; the tiles win while they do not.  Measured (us a step, march / tiles): FP32 20.6 / 9.6
 // at 1024 x 256, 74 / 70 at 2048 x 1024, 136 / 135 at 4096 x 1024, 486 / 513 at 8192 x 2048.
-// FP16 storage is never bandwidth bound: 31 / 12 at 1024 x 256, 628 / 529 at 8192 x 2048.
+// FP16 storage is never bandwidth bound: 31 / 12 at 1024 x 256, 628 / 529 at 8192 x 2048.  FP64 (FP64 pipe):
+// 298 tiles at 1000 x 500 (1.68 nodes/ns), the march 1216 at 2048 x 1024 (1.72 nodes/ns, no halo of normals).
 static long long tile_nodes_max(int prec)
 {
     return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 1LL << 22 : 1LL << 19);
@@ -369,6 +380,7 @@ static int build_phase_reference(lbm_handle *h)
         o[RX_DR3] = T(RT_DR, mirror(j + 3));
         o[RX_DR3LO] = T(RT_DRLO, mirror(j + 3));
         o[RX_GREF1] = T(RT_GREF, j + 1);
+        o[RX_P1] = 1.0 - 2.0 * T(RT_PHI0, j);
     }
     cudaError_t e;
     if (h->rsize == 8) {
@@ -482,6 +494,7 @@ int lbm_create(const lbm_domain *domain, const lbm_params *params, void *stream,
     Phys<double> &P = h->P;
     P.W4 = 4.0 / domain->W;
     P.csf = 1.5 * domain->W;
+    P.csf12 = P.csf / 12.0;
     P.sigma0 = p->sigma0;
     P.sigma1 = p->sigma1;
     P.sigma2 = p->sigma2;
@@ -494,6 +507,15 @@ int lbm_create(const lbm_domain *domain, const lbm_params *params, void *stream,
     P.dmu = (p->visc_ratio - 1.0) * P.muA;
     P.kA = p->rho_bottom * alphaA;
     P.dk = (p->cond_ratio - 1.0) * P.kA;
+    P.mu3A = 3.0 * P.muA;
+    P.dmu3 = 3.0 * P.dmu;
+    P.k3A = 3.0 * P.kA;
+    P.dk3 = 3.0 * P.dk;
+    P.c2drho = P.drho / 3.0;
+    P.irhoA = 1.0 / P.rhoA;
+    P.omnuA = 1.0 / fma(P.mu3A, P.irhoA, 0.5);
+    P.omTA = 1.0 / fma(P.k3A, P.irhoA, 0.5);
+    P.constant = P.drho != 0.0 ? 0 : 1 | (P.dmu3 == 0.0 ? 2 : 0) | (P.dk3 == 0.0 ? 4 : 0);
     P.omega_phi = 1.0 / p->tau_phi;
     P.Mphi = (1.0 / P.omega_phi - 0.5) / 3.0;
     P.Fx = p->Fx_ext;

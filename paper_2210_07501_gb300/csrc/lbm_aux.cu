@@ -60,10 +60,10 @@ __global__ void init_pop_kernel(const StepArgs<Real, Store> A)
             const double mx = double(P.Mphi) * theta * nxv, my = double(P.Mphi) * theta * nyv, c2p = phi_d / 3.0;
             if constexpr (QF == 9) {
                 const double k[9] = {phi_d, mx, my, c2p, c2p, 0.0, 0.0, 0.0, phi_d / 9.0};
-                central_to_pop9_(k, k, uxd, uyd, f);
+                central_to_pop9_(k, uxd, uyd, f);
             } else {
                 const double k[5] = {phi_d, mx, my, c2p, c2p};
-                central_to_pop5_(k, k, uxd, uyd, f);
+                central_to_pop5_(k, uxd, uyd, f);
             }
 #pragma unroll
             for (int a = 0; a < QF; ++a) {
@@ -80,7 +80,7 @@ __global__ void init_pop_kernel(const StepArgs<Real, Store> A)
             const Real k[9] = {dp, ux * d, uy * d, dp * ax - rc2 * ux2, dp * ay - rc2 * uy2, -uxy * d, ax * uy * d,
                                ay * ux * d, dp * ax * ay - rc2 * (c2 * (ux2 + uy2) + ux2 * uy2)};
             Real g[9];
-            central_to_pop9_(k, k, ux, uy, g);
+            central_to_pop9_(k, ux, uy, g);
 #pragma unroll
             for (int a = 0; a < 9; ++a) {
                 Real v = g[a];
@@ -96,10 +96,10 @@ __global__ void init_pop_kernel(const StepArgs<Real, Store> A)
                 const Real k[9] = {dT, Tr * ux, Tr * uy, c2 * dT - Tr * ux2, c2 * dT - Tr * uy2, -Tr * ux * uy,
                                    Tr * (c2 + ux2) * uy, Tr * (c2 + uy2) * ux,
                                    Real(1.0 / 9.0) * dT - Tr * (c2 * (ux2 + uy2) + ux2 * uy2)};
-                central_to_pop9_(k, k, ux, uy, h);
+                central_to_pop9_(k, ux, uy, h);
             } else {
                 const Real k[5] = {dT, Tr * ux, Tr * uy, c2 * dT - Tr * ux2, c2 * dT - Tr * uy2};
-                central_to_pop5_(k, k, ux, uy, h);
+                central_to_pop5_(k, ux, uy, h);
             }
 #pragma unroll
             for (int a = 0; a < QT; ++a) {

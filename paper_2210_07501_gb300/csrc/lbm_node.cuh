@@ -30,23 +30,26 @@ __device__ __forceinline__ void load_rowref_(const Real *rx, Real *v)
 }
 static_assert(RX_N == 8, "load_rowref_ reads eight values");
 
-template <typename Real>
-__device__ __forceinline__ void grad3_(const Real *rm, const Real *r0, const Real *rp, int c, Real &gx, Real &gy)
+// grad phi = grad (phi - phi0) + (0, d_y phi0), isotropic, at column c of the phi - phi0 rows rm, r0, rp.
+__device__ __forceinline__ void grad_ref_(const float *rm, const float *r0, const float *rp, int c, float gref, float &gx,
+                                          float &gy)
 {
-    const Real c1 = Real(1.0 / 3.0), c2 = Real(1.0 / 12.0);
-    if constexpr (std::is_same<Real, float>::value) {
-        // diagonal terms from (NE, NW) +- (SE, SW): (NE + SE) - (NW + SW) and
-        // (NE - SE) + (NW - SW), both halves of a pair in one packed instruction
-        const float2 P = f2_(rp[c + 1], rp[c - 1]), Q = f2_(rm[c + 1], rm[c - 1]);
-        const float2 S = add2_(P, Q), D = sub2_(P, Q);
-        const float2 G = fma2_(bc2_(c1), f2_(r0[c + 1] - r0[c - 1], rp[c] - rm[c]),
-                               mul2_(bc2_(c2), f2_(S.x - S.y, D.x + D.y)));
-        gx = G.x, gy = G.y;
-        return;
-    }
-    const Real ne = rp[c + 1], nw = rp[c - 1], se = rm[c + 1], sw = rm[c - 1];
-    gx = c1 * (r0[c + 1] - r0[c - 1]) + c2 * ((ne - nw) + (se - sw));
-    gy = c1 * (rp[c] - rm[c]) + c2 * ((ne - se) + (nw - sw));
+    // diagonal terms from (NE, NW) +- (SE, SW): (NE + SE) - (NW + SW) and (NE - SE) + (NW - SW), both
+    // halves of a pair in one packed instruction
+    const float c1 = float(1.0 / 3.0), c2 = float(1.0 / 12.0);
+    const float2 P = f2_(rp[c + 1], rp[c - 1]), Q = f2_(rm[c + 1], rm[c - 1]);
+    const float2 S = add2_(P, Q), D = sub2_(P, Q);
+    const float2 G = fma2_(bc2_(c1), f2_(r0[c + 1] - r0[c - 1], rp[c] - rm[c]),
+                           mul2_(bc2_(c2), f2_(S.x - S.y, D.x + D.y)));
+    gx = G.x, gy = G.y + gref;
+}
+// FP64: (4 (E - W) + (NE - SW) + (SE - NW)) / 12, (4 (N - S) + (NE - SW) - (SE - NW)) / 12
+__device__ __forceinline__ void grad_ref_(const double *rm, const double *r0, const double *rp, int c, double gref,
+                                          double &gx, double &gy)
+{
+    const double a = rp[c + 1] - rm[c - 1], b = rm[c + 1] - rp[c - 1], d = 1.0 / 12.0;
+    gx = fma(4.0, r0[c + 1] - r0[c - 1], a + b) * d;
+    gy = fma(d, fma(4.0, rp[c] - rm[c], a - b), gref);
 }
 
 // Loads of one node for the pull: populations of one lattice (plane base pointers `pl`,
@@ -136,14 +139,6 @@ __device__ __forceinline__ void keep_h_(const StepArgs<Real, Store> &A, const Re
     raw_first_<QT>(h, m[1], m[2]);
     if constexpr (scaled_<Store>()) m[1] *= A.ish, m[2] *= A.ish;
 }
-// grad phi = grad (phi - phi0) + (0, d_y phi0) at column c of the phi - phi0 rows rm, r0, rp
-template <typename Real>
-__device__ __forceinline__ void grad_phi_(const Real *rm, const Real *r0, const Real *rp, int c, Real gref, Real &gx,
-                                          Real &gy)
-{
-    grad3_(rm, r0, rp, c, gx, gy);
-    gy += gref;
-}
 // the unit normal of a gradient as (n_x, n_y - 1)
 template <typename Real, typename R2 = typename Vec2<Real>::T>
 __device__ __forceinline__ R2 normal_(Real gx, Real gy, Real g2min)
@@ -162,61 +157,79 @@ template <typename Real, typename Store, int QF, int QT, typename R2 = typename 
 __device__ __forceinline__ void node_step_(const StepArgs<Real, Store> &A, int x, int y, Real dphi, Real gpx, Real gpy,
                                            int s, const R2 *nm, const R2 *n0, const R2 *np, const R2 *qm, const R2 *q0,
                                            const R2 *qp, const Real *fm, const Real *hm, Real *g, Real phi_ref, Real th0,
-                                           Real c01)
+                                           Real c01, Real p1)
 {
     const Phys<Real> &P = A.P;
     const Real c2 = Real(1.0 / 3.0), hf = Real(0.5);
     constexpr bool SCALED = scaled_<Store>();
     const Real phi = phi_ref + dphi;
-    const Real g2 = norm2_(gpx, gpy);
     const R2 nC = n0[s], nE = n0[s + 1], nW = n0[s - 1], nN = np[s], nS = nm[s];
     const R2 nNE = np[s + 1], nNW = np[s - 1], nSE = nm[s + 1], nSW = nm[s - 1];
-    const Real c1 = Real(1.0 / 3.0), cd = Real(1.0 / 12.0);
     const R2 qE = q0[s + 1], qW = q0[s - 1], qN = qp[s], qS = qm[s];
     const R2 qNE = qp[s + 1], qNW = qp[s - 1], qSE = qm[s + 1], qSW = qm[s - 1];
-    Real divn, dsx, dsy, dpx, dpy;
+    const Real g2 = norm2_(gpx, gpy), dT = hm[0];
+    const Real nxv = nC.x, nyv = Real(1) + nC.y;
+    Real fo[QF], ho[QT], ux, uy, dp;
     if constexpr (std::is_same<Real, float>::value) {
-        // the same stencils with the (n_x, n_y) and (sigma, p) halves paired; the
-        // diagonal terms of div n summed as (NE - SW) +- (SE - NW)
+        // the stencils with the (n_x, n_y) and (sigma, p) halves paired; the diagonal terms of
+        // div n summed as (NE - SW) +- (SE - NW)
+        const Real c1 = Real(1.0 / 3.0), cd = Real(1.0 / 12.0);
         const float2 T1 = sub2_(nNE, nSW), T2 = sub2_(nSE, nNW);
-        divn = c1 * ((nE.x - nW.x) + (nN.y - nS.y)) + cd * ((T1.x + T2.x) + (T1.y - T2.y));
+        const Real divn = c1 * ((nE.x - nW.x) + (nN.y - nS.y)) + cd * ((T1.x + T2.x) + (T1.y - T2.y));
         const float2 X = fma2_(bc2_(c1), sub2_(qE, qW), mul2_(bc2_(cd), add2_(sub2_(qNE, qNW), sub2_(qSE, qSW))));
         const float2 Y = fma2_(bc2_(c1), sub2_(qN, qS), mul2_(bc2_(cd), add2_(sub2_(qNE, qSE), sub2_(qNW, qSW))));
-        dsx = X.x, dpx = X.y, dsy = Y.x, dpy = Y.y;
+        const Real dsx = X.x, dpx = X.y, dsy = Y.x, dpy = Y.y;
+        const Real sigma = P.sigma0 + dT * (P.sigma1 + P.sigma2 * dT);
+        const Real Fsx = P.csf * (-sigma * g2 * divn * nxv + g2 * ((Real(1) - nxv * nxv) * dsx - nxv * nyv * dsy));
+        const Real Fsy = P.csf * (-sigma * g2 * divn * nyv + g2 * ((Real(1) - nyv * nyv) * dsy - nxv * nyv * dsx));
+        const Real Ftx = Fsx + P.Fx, Fty = Fsy + P.Fy;
+        const Real Fpx = -dpx + c2 * P.drho * gpx, Fpy = -dpy + c2 * P.drho * gpy;
+        const Real rho = P.rhoA + phi * P.drho;
+        const Real irho = rcp_(rho);
+        Real s0, sx, sy, r20, r02, r11;
+        flow_raw_moments_(g, s0, sx, sy, r20, r02, r11);
+        if constexpr (SCALED) s0 *= A.isg, sx *= A.isg, sy *= A.isg, r20 *= A.isg, r02 *= A.isg, r11 *= A.isg;
+        const Real irc2 = Real(3) * irho;
+        ux = (sx + hf * c2 * Ftx) * irc2;
+        uy = (sy + hf * c2 * Fty) * irc2;
+        dp = s0 + hf * (Fpx * ux + Fpy * uy);
+        const Real om_nu = rcp_(Real(3) * (P.muA + phi * P.dmu) * irho + hf);
+        const Real om_T = rcp_(Real(3) * (P.kA + phi * P.dk) * irho + hf);
+        // theta(phi) - theta(phi0) = (4 / W) dphi (1 - 2 phi0 - dphi)
+        const Real dth = P.W4 * dphi * (Real(1) - Real(2) * phi_ref - dphi);
+        // (FP16 storage: the results come out in stored units)
+        collide_phase_dev_<QF, SCALED>(fo, fm[0], fm[1], dphi, phi, ux, uy, nxv, nC.y, th0, dth, c01, P.Mphi,
+                                       P.omega_phi, A.sf);
+        collide_flow_<SCALED>(g, rho, dp, ux, uy, Fpx, Fpy, Ftx, Fty, om_nu, s0, sx, sy, r20, r02, r11, A.sg);
+        collide_energy_<QT, SCALED>(ho, hm[1], hm[2], dT, ux, uy, P.T_ref, om_T, A.sh);
     } else {
-        divn = c1 * (nE.x - nW.x) + cd * ((nNE.x - nNW.x) + (nSE.x - nSW.x)) + c1 * (nN.y - nS.y) +
-               cd * ((nNE.y - nSE.y) + (nNW.y - nSW.y));
-        dsx = c1 * (qE.x - qW.x) + cd * ((qNE.x - qNW.x) + (qSE.x - qSW.x));
-        dsy = c1 * (qN.x - qS.x) + cd * ((qNE.x - qSE.x) + (qNW.x - qSW.x));
-        dpx = c1 * (qE.y - qW.y) + cd * ((qNE.y - qNW.y) + (qSE.y - qSW.y));
-        dpy = c1 * (qN.y - qS.y) + cd * ((qNE.y - qSE.y) + (qNW.y - qSW.y));
+        // the same with as few FP64 instructions as it takes: stencils times 12 (the factor goes into
+        // constants), F_s = delta_s (grad sigma - (sigma div n + n . grad sigma) n), no division
+        // where a property is constant
+        const Real divn = fma(Real(4), (nE.x - nW.x) + (nN.y - nS.y),
+                              ((nNE.x - nSW.x) + (nSE.x - nNW.x)) + ((nNE.y - nSW.y) - (nSE.y - nNW.y)));
+        const Real a = qNE.x - qSW.x, b = qSE.x - qNW.x, u = qNE.y - qSW.y, v = qSE.y - qNW.y;
+        const Real dsx = fma(Real(4), qE.x - qW.x, a + b), dsy = fma(Real(4), qN.x - qS.x, a - b);
+        const Real dpx = fma(Real(4), qE.y - qW.y, u + v), dpy = fma(Real(4), qN.y - qS.y, u - v);
+        const Real csf = P.csf12 * g2, nf = -fma(P.sigma0 + q0[s].x, divn, fma(nxv, dsx, nyv * dsy));
+        const Real Ftx = fma(csf, fma(nxv, nf, dsx), P.Fx), Fty = fma(csf, fma(nyv, nf, dsy), P.Fy);
+        const Real Fpx = fma(P.c2drho, gpx, Real(-1.0 / 12.0) * dpx), Fpy = fma(P.c2drho, gpy, Real(-1.0 / 12.0) * dpy);
+        const Real rho = fma(phi, P.drho, P.rhoA);
+        const Real irho = P.constant & 1 ? P.irhoA : rcp_(rho);
+        const Real om_nu = P.constant & 2 ? P.omnuA : rcp_(fma(fma(phi, P.dmu3, P.mu3A), irho, hf));
+        const Real om_T = P.constant & 4 ? P.omTA : rcp_(fma(fma(phi, P.dk3, P.k3A), irho, hf));
+        Real s0, sx, sy, d2, r11;
+        flow_raw_moments_(g, s0, sx, sy, d2, r11);
+        const Real irc2 = Real(3) * irho;
+        ux = fma(hf * c2, Ftx, sx) * irc2;
+        uy = fma(hf * c2, Fty, sy) * irc2;
+        const Real Gh = hf * fma(Fpx, ux, Fpy * uy);
+        dp = s0 + Gh;
+        const Real dth = (P.W4 * dphi) * (p1 - dphi);   // p1 = 1 - 2 phi0
+        collide_phase_raw_<QF>(fo, fm[0], fm[1], dphi, phi, ux, uy, nxv, nC.y, th0, dth, c01, P.Mphi, P.omega_phi);
+        collide_flow_raw_(g, rho, dp, ux, uy, Fpx, Fpy, Ftx, Fty, Gh, om_nu, sx, sy, d2, r11);
+        collide_energy_raw_<QT>(ho, hm[1], hm[2], dT, ux, uy, P.T_ref, om_T);
     }
-    const Real nxv = nC.x, nyv = Real(1) + nC.y;
-    const Real dT = hm[0];
-    const Real sigma = P.sigma0 + dT * (P.sigma1 + P.sigma2 * dT);
-    const Real Fsx = P.csf * (-sigma * g2 * divn * nxv + g2 * ((Real(1) - nxv * nxv) * dsx - nxv * nyv * dsy));
-    const Real Fsy = P.csf * (-sigma * g2 * divn * nyv + g2 * ((Real(1) - nyv * nyv) * dsy - nxv * nyv * dsx));
-    const Real Ftx = Fsx + P.Fx, Fty = Fsy + P.Fy;
-    const Real Fpx = -dpx + c2 * P.drho * gpx, Fpy = -dpy + c2 * P.drho * gpy;
-    const Real rho = P.rhoA + phi * P.drho;
-    const Real irho = rcp_(rho);
-    Real s0, sx, sy, r20, r02, r11;
-    flow_raw_moments_(g, s0, sx, sy, r20, r02, r11);
-    if constexpr (SCALED) s0 *= A.isg, sx *= A.isg, sy *= A.isg, r20 *= A.isg, r02 *= A.isg, r11 *= A.isg;
-    const Real irc2 = Real(3) * irho;
-    const Real ux = (sx + hf * c2 * Ftx) * irc2;
-    const Real uy = (sy + hf * c2 * Fty) * irc2;
-    const Real dp = s0 + hf * (Fpx * ux + Fpy * uy);
-    const Real om_nu = rcp_(Real(3) * (P.muA + phi * P.dmu) * irho + hf);
-    const Real om_T = rcp_(Real(3) * (P.kA + phi * P.dk) * irho + hf);
-    // theta(phi) - theta(phi0) = (4 / W) dphi (1 - 2 phi0 - dphi)
-    const Real dth = P.W4 * dphi * (Real(1) - Real(2) * phi_ref - dphi);
-    Real fo[QF], ho[QT];
-    // (FP16 storage: the results come out in stored units)
-    collide_phase_dev_<QF, Real, SCALED>(fo, fm[0], fm[1], dphi, phi, ux, uy, nxv, nC.y, th0, dth, c01,
-                                         P.Mphi, P.omega_phi, A.sf);
-    collide_flow_<Real, SCALED>(g, rho, dp, ux, uy, Fpx, Fpy, Ftx, Fty, om_nu, s0, sx, sy, r20, r02, r11, A.sg);
-    collide_energy_<QT, Real, SCALED>(ho, hm[1], hm[2], dT, ux, uy, P.T_ref, om_T, A.sh);
     const int o = y * A.pitch + x;
     // one unsigned 32-bit byte offset from every plane's base (measured 2 % faster than
     // plane base + element index)

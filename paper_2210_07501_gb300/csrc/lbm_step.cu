@@ -324,7 +324,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
     auto keep_h = [&](const Real *h, Real dT, Real *m) { keep_h_<QT>(A, h, dT, m); };
     auto put_n_g = [&](int r, Real gref) {
         Real gx, gy;
-        grad_phi_(&s_phi[(r - 1) & 7][0], &s_phi[r & 7][0], &s_phi[(r + 1) & 7][0], ch + 2, gref, gx, gy);
+        grad_ref_(&s_phi[(r - 1) & 7][0], &s_phi[r & 7][0], &s_phi[(r + 1) & 7][0], ch + 2, gref, gx, gy);
         s_n[r & 3][ch + 1] = normal_(gx, gy, P.g2min);
     };
     auto put_n = [&](int r) { put_n_g(r, __ldg(t_gref + r)); };
@@ -420,7 +420,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
             }
             if (colt) read_g(std::true_type(), sl, y, g);
         }
-        const Real phi_ref = rx[RX_PHI0], th0 = rx[RX_TH0], c01 = rx[RX_C01], gref = rx[RX_GREF];
+        const Real phi_ref = rx[RX_PHI0], th0 = rx[RX_TH0], c01 = rx[RX_C01], gref = rx[RX_GREF], p1 = rx[RX_P1];
         // refill the slot read one row ago (every thread is past its reads) with row y + D - 1
         issue(y + D - 1, sl == 0 ? D - 1 : sl - 1);
         if (++sl == D) {
@@ -434,10 +434,10 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         }
         if (xin) {
             Real gpx, gpy;
-            grad_phi_(&s_phi[(y - 1) & 7][0], &s_phi[y & 7][0], &s_phi[(y + 1) & 7][0], tid + 2, gref, gpx, gpy);
+            grad_ref_(&s_phi[(y - 1) & 7][0], &s_phi[y & 7][0], &s_phi[(y + 1) & 7][0], tid + 2, gref, gpx, gpy);
             node_step_<Real, Store, QF, QT>(A, x, y, s_phi[y & 7][tid + 2], gpx, gpy, tid + 1, s_n[(y - 1) & 3],
                                             s_n[y & 3], s_n[(y + 1) & 3], s_sp[(y - 1) & 3], s_sp[y & 3],
-                                            s_sp[(y + 1) & 3], fm0, hm0, g, phi_ref, th0, c01);
+                                            s_sp[(y + 1) & 3], fm0, hm0, g, phi_ref, th0, c01, p1);
         }
 #pragma unroll
         for (int a = 0; a < 2; ++a) {

@@ -95,7 +95,7 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
     __syncthreads();
     auto put_n = [&](int hx, int hy, Real &gx, Real &gy) {
         const Real *r = s_phi + (hy + 2) * PX;
-        grad_phi_(r - PX, r, r + PX, hx + 2, t_gref[y0 + hy], gx, gy);
+        grad_ref_(r - PX, r, r + PX, hx + 2, t_gref[y0 + hy], gx, gy);
         s_n[(hy + 1) * SX + hx + 1] = normal_(gx, gy, A.P.g2min);
     };
     Real gpx, gpy;   // grad phi of the thread's own node
@@ -111,7 +111,7 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
         load_rowref_(A.rowx + (long long)y * RX_N, rx);
         const R2 *n = s_n + (ly + 1) * SX, *q = s_sp + (ly + 1) * SX;
         node_step_<Real, Store, QF, QT>(A, x, y, dphi, gpx, gpy, lx + 1, n - SX, n, n + SX, q - SX, q, q + SX, fm, hm,
-                                        g, rx[RX_PHI0], rx[RX_TH0], rx[RX_C01]);
+                                        g, rx[RX_PHI0], rx[RX_TH0], rx[RX_C01], rx[RX_P1]);
     }
 }
 
@@ -186,14 +186,14 @@ cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ct
 
 // Tile shape.  FP32 arithmetic: 32 x 8.  FP64 is bound by the SM's one FP64 pipe (16 cycles a warp
 // instruction), so what counts is the FP64 instructions of the SM with the most tiles: warps of
-// nodes, the inner ring's normals, the outer ring's phi, and a start-up of ~200 (the shapes this
+// nodes, the inner ring's normals, the outer ring's phi, and a start-up of ~150 (the shapes this
 // ranks first are within 3 % of the best measured at 200 x 100, 160 x 320 and 1024 x 256).
 template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx, long long ny, int sms, int *tx, int *ty)
 {
     using G = TileGeo<Real, Store>;
     *tx = G::TX, *ty = G::NT / G::TX;
     if (G::FIXED) return;
-    const double node = 330.0 + 19.0 * (QF + QT - 10), normal = 55.0, pull = 15.0, start = 200.0;
+    const double node = 260.0 + 14.0 * (QF + QT - 10), normal = 36.0, pull = 13.0, start = 150.0;
     auto warps = [](int n) { return double((n + 31) / 32); };
     double best = -1.0;
     for (int a = (nx + 63) / 64; a <= (nx + 7) / 8; ++a)
