@@ -583,7 +583,7 @@ int lbm_init_fields(lbm_handle *h, const double *phi, const double *u, const dou
 static int run_check(lbm_handle *h)
 {
     const long long N = (long long)h->nx * h->ny;
-    CK(launch_reduce(h->macro, h->uprev, N, 1, h->partials, reduce_blocks(), h->result, h->stream));
+    CK(launch_reduce(h->macro, h->uprev, N, 1, h->partials, h->result, h->stream));
     h->prev_check_step = h->last_check_step;
     h->have_prev_check = h->have_check;
     h->last_check_step = h->step;
@@ -628,8 +628,7 @@ int lbm_fields_device(lbm_handle *h, void *phi, void *u, void *v, void *T, void 
     if (!h || (dtype != LBM_DTYPE_F64 && dtype != LBM_DTYPE_F32)) return LBM_EINVAL;
     const long long N = (long long)h->nx * h->ny;
     void *dst[5] = {phi, u, v, T, dp};
-    for (int k = 0; k < 5; ++k)
-        if (dst[k]) CK(launch_export(h->macro + k * N, dst[k], N, dtype == LBM_DTYPE_F32, h->stream));
+    CK(launch_export(h->macro, dst, N, dtype == LBM_DTYPE_F32, h->stream));
     return LBM_OK;
 }
 
@@ -637,10 +636,9 @@ int lbm_diag(lbm_handle *h, double *mass, double *residual, int64_t *step)
 {
     if (!h) return LBM_EINVAL;
     const long long N = (long long)h->nx * h->ny;
-    // residual terms of the last check, then a fresh mass / finiteness reduction
-    CK(cudaMemcpyAsync(h->host_result, h->result, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(launch_reduce(h->macro, h->uprev, N, 0, h->partials, reduce_blocks(), h->result + 4, h->stream));
-    CK(cudaMemcpyAsync(h->host_result + 4, h->result + 4, 5 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    // residual terms of the last check, a fresh mass / finiteness reduction, the fault word
+    CK(launch_reduce(h->macro, h->uprev, N, 0, h->partials, h->result + 4, h->stream));
+    CK(cudaMemcpyAsync(h->host_result, h->result, 9 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     const double *r = h->host_result;
     if (*(const unsigned int *)(r + 8)) return LBM_EDEVICE;
@@ -959,6 +957,7 @@ struct lbm_batch {
     int *d_active = nullptr;
     std::vector<int> active;
     double *d_results = nullptr;       // [n][4] reduction results of the last check, then the fault word
+    ReduceCase *d_reduce = nullptr;
     double *h_results = nullptr;       // pinned copy
     std::vector<int64_t> steps;        // steps taken per case
     std::vector<double> residual;      // last residual per case (-1 before two checks)
@@ -1035,11 +1034,7 @@ static int batch_capture(lbm_batch *b)
     cudaError_t e = cudaSuccess;
     for (int64_t k = 0; k < b->K && e == cudaSuccess; ++k)
         e = dispatch<BatchStepFn>(b->h[0], b, (int)(k & 1), (int)(k == b->K - 1));
-    for (int c = 0; c < b->n && e == cudaSuccess; ++c) {
-        lbm_handle *h = b->h[c];
-        e = launch_reduce(h->macro, h->uprev, (long long)h->nx * h->ny, 1, h->partials, reduce_blocks(),
-                          b->d_results + 4 * c, b->stream);
-    }
+    if (e == cudaSuccess) e = launch_reduce_batch(b->d_reduce, b->d_active, b->n, b->d_results, b->stream);
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess) { if (g) cudaGraphDestroy(g); return cuda_fail(e, "batch capture"); }
     if (e2 != cudaSuccess) return cuda_fail(e2, "cudaStreamEndCapture");
@@ -1064,6 +1059,7 @@ void lbm_batch_destroy(lbm_batch *b)
     if (b->d_ctas) cudaFree(b->d_ctas);
     if (b->d_active) cudaFree(b->d_active);
     if (b->d_results) cudaFree(b->d_results);
+    if (b->d_reduce) cudaFree(b->d_reduce);
     if (b->h_results) cudaFreeHost(b->h_results);
     for (lbm_handle *h : b->h) lbm_destroy(h);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -1103,10 +1099,16 @@ int lbm_batch_create(int32_t n, const lbm_domain *domains, const lbm_params *par
     b->checks.assign(n, 0);
     bool ok = cudaMalloc((void **)&b->d_active, n * sizeof(int)) == cudaSuccess &&
               cudaMalloc((void **)&b->d_results, (4 * (size_t)n + 1) * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void **)&b->d_reduce, (size_t)n * sizeof(ReduceCase)) == cudaSuccess &&
               cudaMallocHost((void **)&b->h_results, (4 * (size_t)n + 1) * sizeof(double)) == cudaSuccess;
     if (!ok) { cudaGetLastError(); lbm_batch_destroy(b); return LBM_ENOMEM; }
     cudaError_t e = cudaMemcpy(b->d_active, b->active.data(), n * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_results, 0, (4 * (size_t)n + 1) * sizeof(double));
+    std::vector<ReduceCase> rc_cases;
+    for (const lbm_handle *h : b->h)
+        rc_cases.push_back(ReduceCase{h->macro, h->uprev, h->partials, (long long)h->nx * h->ny});
+    if (e == cudaSuccess)
+        e = cudaMemcpy(b->d_reduce, rc_cases.data(), n * sizeof(ReduceCase), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = dispatch<BatchArgsFn>(b->h[0], b);
     // the shapes for as many rows of the widest channel as the batch has nodes; marching segments of
     // 32 rows until tuned

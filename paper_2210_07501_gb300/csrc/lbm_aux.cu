@@ -3,6 +3,7 @@
 #include <math.h>
 
 #include "lbm_internal.h"
+#include "lbm_reduce.cuh"
 
 namespace lbm {
 
@@ -127,72 +128,66 @@ cudaError_t launch_init(const StepArgs<Real, Store> &A, double b, double W, int 
     return cudaGetLastError();
 }
 
-// ---- reductions: fixed launch shape and fixed-order final pass (deterministic) ----
-constexpr int RED_THREADS = 256;
-constexpr int RED_BLOCKS = 304;   // 2 x 152 SMs
+// ---- reductions: fixed launch shape and order (lbm_reduce.cuh) ----
 int reduce_blocks() { return RED_BLOCKS; }
 
-__device__ __forceinline__ double warp_sum_(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 __global__ void __launch_bounds__(RED_THREADS)
-reduce_partial_kernel(const double *__restrict__ macro, double *__restrict__ uprev, long long N, int update,
-                      double *__restrict__ partials)
+reduce_partial_kernel(const double *macro, double *uprev, long long N, int update, double *partials)
 {
-    double m = 0.0, du2 = 0.0, u2 = 0.0, bad = 0.0;
-    for (long long i = blockIdx.x * (long long)RED_THREADS + threadIdx.x; i < N; i += (long long)gridDim.x * RED_THREADS) {
-        const double phi = macro[i], u = macro[N + i], v = macro[2 * N + i], T = macro[3 * N + i];
-        const double up = uprev[i], vp = uprev[N + i];
-        m += phi;
-        du2 += (u - up) * (u - up) + (v - vp) * (v - vp);
-        u2 += u * u + v * v;
-        if (!isfinite(phi) || !isfinite(u) || !isfinite(v) || !isfinite(T)) bad += 1.0;
-        if (update) {
-            uprev[i] = u;
-            uprev[N + i] = v;
-        }
-    }
-    __shared__ double sh[4][RED_THREADS / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    m = warp_sum_(m);
-    du2 = warp_sum_(du2);
-    u2 = warp_sum_(u2);
-    bad = warp_sum_(bad);
-    if (lane == 0) {
-        sh[0][wid] = m;
-        sh[1][wid] = du2;
-        sh[2][wid] = u2;
-        sh[3][wid] = bad;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) t += sh[threadIdx.x][w];
-        partials[blockIdx.x * 4 + threadIdx.x] = t;
-    }
+    pdl_launch_next_();
+    pdl_wait_();
+    reduce_block_(macro, macro + N, macro + 2 * N, macro + 3 * N, uprev, uprev + N, N, blockIdx.x, update != 0,
+                  partials + 4 * blockIdx.x);
 }
 
-__global__ void reduce_final_kernel(const double *__restrict__ partials, int nblk, double *__restrict__ result)
+__global__ void __launch_bounds__(128) reduce_final_kernel(const double *partials, double *result)
 {
-    if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int b = 0; b < nblk; ++b) t += partials[b * 4 + threadIdx.x];
-        result[threadIdx.x] = t;
-    }
+    pdl_launch_next_();
+    pdl_wait_();
+    reduce_blocks_(partials, result);
 }
 
-cudaError_t launch_reduce(const double *macro, double *uprev, long long N, int update, double *partials, int nblk,
-                          double *result, cudaStream_t s)
+cudaError_t launch_reduce(const double *macro, double *uprev, long long N, int update, double *partials, double *result,
+                          cudaStream_t s)
 {
-    reduce_partial_kernel<<<nblk, RED_THREADS, 0, s>>>(macro, uprev, N, update, partials);
-    cudaError_t e = cudaGetLastError();
+    PdlLaunch l(dim3(RED_BLOCKS), dim3(RED_THREADS), 0, s), f(dim3(1), dim3(128), 0, s);
+    cudaError_t e = cudaLaunchKernelEx(&l.cfg, reduce_partial_kernel, macro, uprev, N, update, partials);
     if (e != cudaSuccess) return e;
-    reduce_final_kernel<<<1, 32, 0, s>>>(partials, nblk, result);
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&f.cfg, reduce_final_kernel, (const double *)partials, result);
+}
+
+// The same for every active channel of a batch in two launches (one pair a channel before: 64 launches
+// and 0.8 ms a check on 32 channels).
+__global__ void __launch_bounds__(RED_THREADS) reduce_batch_kernel(const ReduceCase *cases, const int *active)
+{
+    pdl_launch_next_();
+    const ReduceCase c = cases[blockIdx.y];
+    pdl_wait_();
+    if (active[blockIdx.y])
+        reduce_block_(c.macro, c.macro + c.N, c.macro + 2 * c.N, c.macro + 3 * c.N, c.uprev, c.uprev + c.N, c.N,
+                      blockIdx.x, true, c.partials + 4 * blockIdx.x);
+}
+
+__global__ void __launch_bounds__(128) reduce_batch_final_kernel(const ReduceCase *cases, const int *active,
+                                                                 double *results)
+{
+    pdl_launch_next_();
+    pdl_wait_();
+    if (active[blockIdx.x]) reduce_blocks_(cases[blockIdx.x].partials, results + 4 * blockIdx.x);
+}
+
+cudaError_t launch_reduce_batch(const ReduceCase *cases, const int *active, int n, double *results, cudaStream_t s)
+{
+    // grid.y is limited to 65535 channels
+    for (int c = 0; c < n; c += 65535) {
+        const int k = n - c < 65535 ? n - c : 65535;
+        PdlLaunch l(dim3(RED_BLOCKS, k), dim3(RED_THREADS), 0, s), f(dim3(k), dim3(128), 0, s);
+        cudaError_t e = cudaLaunchKernelEx(&l.cfg, reduce_batch_kernel, cases + c, active + c);
+        if (e != cudaSuccess) return e;
+        e = cudaLaunchKernelEx(&f.cfg, reduce_batch_final_kernel, cases + c, active + c, results + 4 * (size_t)c);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // ---- conversions (ref: optional [Q][ny] values subtracted before storing, in FP64) ----
@@ -241,18 +236,29 @@ cudaError_t launch_from_store(const Store *src, double *dst, int Q, int nx, int 
     return cudaGetLastError();
 }
 
-__global__ void export_kernel(const double *__restrict__ src, void *dst, long long N, int to_float)
+// The requested fields in one launch (blockIdx.y: which; five launches before, 10 us of a
+// 200 us pass at 128 x 32).
+struct ExportPtrs {
+    void *dst[5];
+};
+__global__ void __launch_bounds__(256) export_kernel(const double *macro, ExportPtrs p, long long N, int to_float)
 {
+    pdl_launch_next_();
+    void *dst = p.dst[blockIdx.y];
+    const double *src = macro + blockIdx.y * N;
+    pdl_wait_();
+    if (!dst) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
         if (to_float) ((float *)dst)[i] = float(src[i]);
         else ((double *)dst)[i] = src[i];
     }
 }
-cudaError_t launch_export(const double *src, void *dst, long long N, int to_float, cudaStream_t s)
+cudaError_t launch_export(const double *macro, void *const dst[5], long long N, int to_float, cudaStream_t s)
 {
-    const int blocks = int((N + 255) / 256 < 8192 ? (N + 255) / 256 : 8192);
-    export_kernel<<<blocks, 256, 0, s>>>(src, dst, N, to_float);
-    return cudaGetLastError();
+    ExportPtrs p;
+    for (int k = 0; k < 5; ++k) p.dst[k] = dst[k];
+    PdlLaunch l(dim3((unsigned)((N + 255) / 256 < 8192 ? (N + 255) / 256 : 8192), 5), dim3(256), 0, s);
+    return cudaLaunchKernelEx(&l.cfg, export_kernel, macro, p, N, to_float);
 }
 
 #define LBM_INST_INIT(R, S, QF, QT) \

@@ -42,10 +42,17 @@ template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_init(const StepArgs<Real, Store> &A, double b, double W, int defaults, cudaStream_t s);
 
-// Reductions over the macro fields: partials[nblk][4] then result[4] =
+// Reductions over the macro fields: partials[reduce_blocks()][4] then result[4] =
 // (sum phi, sum |u - u_prev|^2, sum |u|^2, non-finite count); u_prev <- u if update.
-cudaError_t launch_reduce(const double *macro, double *uprev, long long N, int update, double *partials,
-                          int nblk, double *result, cudaStream_t s);
+cudaError_t launch_reduce(const double *macro, double *uprev, long long N, int update, double *partials, double *result,
+                          cudaStream_t s);
+// The same (update = 1) for the active ones of n channels, into results[n][4].
+struct ReduceCase {
+    const double *macro;
+    double *uprev, *partials;
+    long long N;
+};
+cudaError_t launch_reduce_batch(const ReduceCase *cases, const int *active, int n, double *results, cudaStream_t s);
 int reduce_blocks();
 
 // [Q][ny][nx] doubles <-> [Q][ny][pitch] storage ((value - ref[q][y]) * scale stored; ref
@@ -56,7 +63,7 @@ cudaError_t launch_to_store(const double *src, Store *dst, int Q, int nx, int ny
 template <typename Real, typename Store>
 cudaError_t launch_from_store(const Store *src, double *dst, int Q, int nx, int ny, int pitch, Real iscale,
                               const double *ref, cudaStream_t s);
-// macro plane -> device array of float or double
-cudaError_t launch_export(const double *src, void *dst, long long N, int to_float, cudaStream_t s);
+// macro planes -> device arrays of float or double (NULL: not wanted)
+cudaError_t launch_export(const double *macro, void *const dst[5], long long N, int to_float, cudaStream_t s);
 
 }  // namespace lbm
