@@ -7,6 +7,7 @@
 // the last step of each lbm_step call (and at every residual check), the previous
 // velocity for the residual, and the reduction scratch.  All work is queued on one CUDA
 // stream; only the entry points that return data to the host synchronise it.
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -950,7 +951,8 @@ struct lbm_batch {
     std::vector<lbm_handle *> h;       // per-case state (allocated on the batch stream)
     void *d_args[2] = {nullptr, nullptr};   // StepArgs per case, source buffer 0 / 1, no macros
     void *d_args_m[2] = {nullptr, nullptr}; // same, writing the macroscopic fields
-    int4 *d_ctas = nullptr;
+    int4 *d_ctas = nullptr;            // CTA table (batches of more than PACK_CASES)
+    std::vector<unsigned char> pack[2][2];   // BatchPack by [source buffer][with macros] (smaller batches)
     int n_ctas = 0;
     Shapes shapes;
     StepShape shape;
@@ -970,6 +972,7 @@ struct lbm_batch {
 template <typename R, typename S, int QF, int QT> struct BatchArgsFn {
     static cudaError_t run(const lbm_handle *, lbm_batch *b)
     {
+        if (b->n <= PACK_CASES) return cudaSuccess;   // in the launches' parameters (BatchTableFn)
         const size_t sz = sizeof(StepArgs<R, S>);
         std::vector<StepArgs<R, S>> a(b->n);
         for (int par = 0; par < 2; ++par)
@@ -995,6 +998,24 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
     {
         const int w = shape.rows > 0 ? step_strip_width<R, S, QF, QT>() : shape.tx;
         const int t_rows = shape.rows > 0 ? shape.rows : shape.ty;
+        b->shape = shape;
+        if (b->n <= PACK_CASES) {
+            for (int par = 0; par < 2; ++par)
+                for (int m = 0; m < 2; ++m) {
+                    b->pack[par][m].assign(sizeof(BatchPack<R, S>), 0);
+                    BatchPack<R, S> &B = *reinterpret_cast<BatchPack<R, S> *>(b->pack[par][m].data());
+                    b->n_ctas = 0;
+                    for (int c = 0; c < PACK_CASES; ++c) {
+                        B.start[c] = c < b->n ? b->n_ctas : INT_MAX;
+                        if (c >= b->n) continue;
+                        B.cols[c] = (b->h[c]->nx + w - 1) / w;
+                        b->n_ctas += B.cols[c] * ((b->h[c]->ny + t_rows - 1) / t_rows);
+                        B.a[c] = make_args<R, S>(b->h[c], par, m ? b->h[c]->macro : nullptr);
+                        B.a[c].fault = (unsigned int *)(b->d_results + 4 * (size_t)b->n);   // one word per batch
+                    }
+                }
+            return cudaSuccess;
+        }
         std::vector<int4> t;
         for (int c = 0; c < b->n; ++c) {
             const int strips = (b->h[c]->nx + w - 1) / w, segs = (b->h[c]->ny + t_rows - 1) / t_rows;
@@ -1006,7 +1027,6 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
         cudaError_t e = cudaMalloc((void **)&b->d_ctas, t.size() * sizeof(int4));
         if (e != cudaSuccess) return e;
         b->n_ctas = (int)t.size();
-        b->shape = shape;
         return cudaMemcpy(b->d_ctas, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice);
     }
 };
@@ -1014,6 +1034,12 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
 template <typename R, typename S, int QF, int QT> struct BatchStepFn {
     static cudaError_t run(const lbm_handle *, lbm_batch *b, int par, int macro)
     {
+        if (b->n <= PACK_CASES) {
+            const BatchPack<R, S> &B = *reinterpret_cast<const BatchPack<R, S> *>(b->pack[par][macro].data());
+            if (b->shape.rows > 0)
+                return launch_march_pack<R, S, QF, QT>(B, b->n_ctas, b->d_active, b->shape.rows, b->stream);
+            return launch_tile_pack<R, S, QF, QT>(B, b->n_ctas, b->d_active, b->shape.tx, b->shape.ty, b->stream);
+        }
         const StepArgs<R, S> *args = (const StepArgs<R, S> *)(macro ? b->d_args_m[par] : b->d_args[par]);
         if (b->shape.rows > 0)
             return launch_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape.rows, b->stream);

@@ -21,14 +21,36 @@ cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int row
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, int tx, int ty);
 
-// Many cases in one launch (see batch_kernel, tile_batch_kernel): ctas[i] = (case, strip, segment, 0)
-// or (case, tile column, tile row, 0).
+// Many cases in one launch.  Up to PACK_CASES of them travel in the launch's parameters: their arguments
+// are then uniform values in constant memory, as those of a single channel are (fetched through
+// a pointer they cost ~160 instructions a node more and two dependent loads a CTA).  start[c]: first CTA
+// of case c (INT_MAX beyond the last case), cols[c]: its strips or tiles per row.
+constexpr int PACK_CASES = 32;
+template <typename Real, typename Store> struct BatchPack {
+    int start[PACK_CASES], cols[PACK_CASES];
+    StepArgs<Real, Store> a[PACK_CASES];
+};
+// The case of a CTA: the last one that starts at or before it.
+template <typename Real, typename Store> __device__ __forceinline__ int pack_case_(const BatchPack<Real, Store> &B, int cta)
+{
+    int c = 0;
+#pragma unroll
+    for (int s = PACK_CASES / 2; s > 0; s >>= 1)
+        if (cta >= B.start[c + s]) c += s;
+    return c;
+}
+// Larger batches: ctas[i] = (case, strip or tile column, segment or tile row, 0), arguments in device memory.
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active, int seg,
                          cudaStream_t s);
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active,
                               int tx, int ty, cudaStream_t s);
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_march_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int seg, cudaStream_t s);
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int tx, int ty,
+                             cudaStream_t s);
 // Columns per strip of the march.
 template <typename Real, typename Store, int QF, int QT> int step_strip_width();
 // Rows per segment of the march when none is set (whole waves of resident CTAs).

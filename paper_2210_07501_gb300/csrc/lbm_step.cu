@@ -475,6 +475,21 @@ __global__ void __launch_bounds__(TX + 32, batch_ctas<Real>()) batch_kernel(cons
 }
 
 
+// The same with up to PACK_CASES channels' arguments in the launch's parameters: the registers and
+// CTAs per SM of the single-channel kernel.
+template <typename Real, typename Store, int QF, int QT, int TX>
+__global__ void __launch_bounds__(TX + 32, march_ctas<Real, Store>())
+pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *active, int seg)
+{
+    pdl_launch_next_();
+    const int c = pack_case_(B, blockIdx.x), i = blockIdx.x - B.start[c], by = i / B.cols[c], bx = i - by * B.cols[c];
+    if (!active[c]) {
+        pdl_wait_();
+        return;
+    }
+    march_body<Real, Store, QF, QT, TX>(B.a[c], seg, bx, by);
+}
+
 template <typename Real, typename Store, int QF, int QT>
 int step_strip_width()
 {
@@ -492,6 +507,8 @@ static int prepare_kernels()
     if (!done) {
         cudaFuncSetAttribute(march_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
         cudaFuncSetAttribute(batch_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        cudaFuncSetAttribute(pack_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        cudaFuncSetAttribute(pack_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaFuncSetAttribute(march_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              100);
         cudaFuncSetAttribute(batch_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -508,6 +525,14 @@ cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, i
     constexpr int TX = march_width<Real>();
     PdlLaunch l(dim3(n_ctas), dim3(TX + 32), prepare_kernels<Real, Store, QF, QT>(), s);
     return cudaLaunchKernelEx(&l.cfg, batch_kernel<Real, Store, QF, QT, TX>, cases, ctas, active, seg);
+}
+
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_march_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int seg, cudaStream_t s)
+{
+    constexpr int TX = march_width<Real>();
+    PdlLaunch l(dim3(n_ctas), dim3(TX + 32), prepare_kernels<Real, Store, QF, QT>(), s);
+    return cudaLaunchKernelEx(&l.cfg, pack_kernel<Real, Store, QF, QT, TX>, B, active, seg);
 }
 
 // Segment length: the one that minimises the estimated step time, waves of resident CTAs
@@ -570,6 +595,8 @@ cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int row
     template cudaError_t launch_march<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, int);            \
     template cudaError_t launch_batch<R, S, QF, QT>(const StepArgs<R, S> *, const int4 *, int, const int *, \
                                                     int, cudaStream_t);                                   \
+    template cudaError_t launch_march_pack<R, S, QF, QT>(const BatchPack<R, S> &, int, const int *, int,    \
+                                                         cudaStream_t);                                    \
     template int step_strip_width<R, S, QF, QT>();                                                         \
     template int auto_segment<R, S, QF, QT>(int, int);
 LBM_INST(double, double, 5, 5)

@@ -163,6 +163,19 @@ tile_batch_kernel(const StepArgs<Real, Store> *__restrict__ cases, const int4 *_
     let_next_start_late_<Real>();
 }
 
+// The same with up to PACK_CASES channels' arguments in the launch's parameters.
+template <typename Real, typename Store, int QF, int QT>
+__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store>::CTAS)
+tile_pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *active, int tx, int ty)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    let_next_start_early_<Real>();
+    const int c = pack_case_(B, blockIdx.x), i = blockIdx.x - B.start[c], by = i / B.cols[c], bx = i - by * B.cols[c];
+    pdl_wait_();
+    if (active[c]) tile_body<Real, Store, QF, QT>(B.a[c], tx, ty, bx, by, smem);
+    let_next_start_late_<Real>();
+}
+
 template <typename Real> static size_t tile_smem(int tx, int ty)
 {
     return ((size_t)(ty + 4) * (tx + 4) + 4 * (size_t)(ty + 2) * (tx + 2)) * sizeof(Real);
@@ -182,6 +195,14 @@ cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ct
 {
     PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty), s);
     return cudaLaunchKernelEx(&l.cfg, tile_batch_kernel<Real, Store, QF, QT>, cases, ctas, active, tx, ty);
+}
+
+template <typename Real, typename Store, int QF, int QT>
+cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int tx, int ty,
+                             cudaStream_t s)
+{
+    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty), s);
+    return cudaLaunchKernelEx(&l.cfg, tile_pack_kernel<Real, Store, QF, QT>, B, active, tx, ty);
 }
 
 // Tile shape.  FP32 arithmetic: 32 x 8.  FP64 is bound by the SM's one FP64 pipe (16 cycles a warp
@@ -209,6 +230,8 @@ template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx
     template cudaError_t launch_tile<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, int, int);            \
     template cudaError_t launch_tile_batch<R, S, QF, QT>(const StepArgs<R, S> *, const int4 *, int, const int *, \
                                                          int, int, cudaStream_t);                              \
+    template cudaError_t launch_tile_pack<R, S, QF, QT>(const BatchPack<R, S> &, int, const int *, int, int,    \
+                                                        cudaStream_t);                                         \
     template void choose_tile<R, S, QF, QT>(int, long long, int, int *, int *);
 LBM_INST(double, double, 5, 5)
 LBM_INST(double, double, 5, 9)

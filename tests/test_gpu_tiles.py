@@ -30,3 +30,30 @@ def test_tiles_equal_marching_strips(precision, qf, qt, nx, ny):
         g.close()
     for k in got[0]:
         assert np.array_equal(got[0][k], got[1][k]), k
+
+
+@pytest.mark.parametrize("precision,n", [("fp32", 32), ("fp32", 33), ("fp64", 1), ("fp64", 33), ("fp16", 32)])
+def test_batches_of_any_number_equal_single_channels(precision, n):
+    """Batches of up to 32 channels carry their arguments in the launch's parameters, larger ones read
+    them from device memory; on tiles (the rule's choice at these sizes) and after tuning, every
+    channel has the bits of a handle of its own."""
+    from paper_2210_07501_gb300 import Lbm, LbmBatch
+    rng = np.random.Generator(np.random.PCG64(n))
+    ws = [WL.channel(int(rng.choice([33, 64, 130])), int(rng.choice([9, 16, 25])), 5.0, W=3.0,
+                     sigma1=float(rng.uniform(-2e-4, 2e-4)), sigma2=-2e-3, visc_ratio=float(rng.uniform(0.5, 2.0)))
+          for _ in range(n)]
+    b = LbmBatch(ws, precision=precision)
+    b.lbm_batch_set_check_interval(10)
+    b.lbm_batch_step(10)
+    b.lbm_batch_autotune(1)
+    b.lbm_batch_step(20)
+    for c, w in enumerate(ws):
+        g = Lbm(w["domain"], w["params"], precision=precision)
+        g.lbm_set_check_interval(10)
+        g.lbm_step(30)
+        a, r = b.lbm_batch_fields(c), g.lbm_fields()
+        for k in a:
+            assert np.array_equal(a[k], r[k]), (c, k)
+        assert b.lbm_batch_diag(c)["residual"] == g.lbm_diag()["residual"]
+        g.close()
+    b.close()
