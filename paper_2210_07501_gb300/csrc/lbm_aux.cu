@@ -248,9 +248,20 @@ __global__ void __launch_bounds__(256) export_kernel(const double *macro, Export
     const double *src = macro + blockIdx.y * N;
     pdl_wait_();
     if (!dst) return;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        if (to_float) ((float *)dst)[i] = float(src[i]);
-        else ((double *)dst)[i] = src[i];
+    // four loads in flight (the compiler cannot tell dst from src: one at a time took 210 instead of 167 us
+    // for 8192 x 2048)
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += 4 * step) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * step < N) v[k] = src[i + k * step];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i + k * step < N) {
+                if (to_float) ((float *)dst)[i + k * step] = float(v[k]);
+                else ((double *)dst)[i + k * step] = v[k];
+            }
     }
 }
 cudaError_t launch_export(const double *macro, void *const dst[5], long long N, int to_float, cudaStream_t s)
