@@ -182,12 +182,12 @@ template <typename R, typename S, int QF, int QT> struct StepFn {
 // Channels up to this many nodes (batches: in total) step on tiles, larger ones in marching strips.
 // The march reads no row twice and reaches the copy bandwidth once its strips fill the GPU for
 // several waves; the tiles win while they do not.  Measured (us a step, march / tiles): FP32 20.6 / 9.6
-// at 1024 x 256, 74 / 70 at 2048 x 1024, 136 / 135 at 4096 x 1024, 486 / 513 at 8192 x 2048.
+// at 1024 x 256, 74 / 70 at 2048 x 1024, 126 / 134 at 4096 x 1024, 449 / 513 at 8192 x 2048.
 // FP16 storage is never bandwidth bound: 31 / 12 at 1024 x 256, 628 / 529 at 8192 x 2048.  FP64 (FP64 pipe):
 // 298 tiles at 1000 x 500 (1.68 nodes/ns), the march 1216 at 2048 x 1024 (1.72 nodes/ns, no halo of normals).
 static long long tile_nodes_max(int prec)
 {
-    return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 1LL << 22 : 1LL << 19);
+    return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 3LL << 20 : 1LL << 19);
 }
 // ny_total: the channel's rows (a batch: those of all its channels, put one on top of the other)
 template <typename R, typename S, int QF, int QT> struct ShapesFn {

@@ -163,11 +163,11 @@ __device__ __forceinline__ void node_step_(const StepArgs<Real, Store> &A, int x
     const Real c2 = Real(1.0 / 3.0), hf = Real(0.5);
     constexpr bool SCALED = scaled_<Store>();
     const Real phi = phi_ref + dphi;
+    const Real g2 = norm2_(gpx, gpy), dT = hm[0];
     const R2 nC = n0[s], nE = n0[s + 1], nW = n0[s - 1], nN = np[s], nS = nm[s];
     const R2 nNE = np[s + 1], nNW = np[s - 1], nSE = nm[s + 1], nSW = nm[s - 1];
     const R2 qE = q0[s + 1], qW = q0[s - 1], qN = qp[s], qS = qm[s];
     const R2 qNE = qp[s + 1], qNW = qp[s - 1], qSE = qm[s + 1], qSW = qm[s - 1];
-    const Real g2 = norm2_(gpx, gpy), dT = hm[0];
     const Real nxv = nC.x, nyv = Real(1) + nC.y;
     Real fo[QF], ho[QT], ux, uy, dp;
     if constexpr (std::is_same<Real, float>::value) {

@@ -12,6 +12,8 @@
 // post-collision populations and p to the other buffer.
 // Populations live in SoA planes [Q][ny][pitch], x fastest: every pull of a warp is a
 // contiguous (shifted) row segment.  No tensor cores: the step is a bandwidth-bound stencil.
+#include <math.h>
+
 #include "lbm_internal.h"
 #include "lbm_node.cuh"
 
@@ -196,7 +198,9 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
     const int bspan = bhi > blo ? bhi - blo : 0, boff = blo - sx0;
     const int dlo = max(dx0, 0), dhi = min(x0 + TX + HD, nx / CD * CD);
     const int dspan = dhi > dlo ? dhi - dlo : 0, doff = dlo - dx0;
-    const int nel_s = RS - bspan, nel_d = RD - dspan;          // element-wise columns per plane
+    // element-wise columns per plane; in the last strip nothing past the wrapped halo (copying the rest of
+    // its width too made a step at 8193 x 1024 529 us instead of 239 in segments of 48 rows)
+    const int nel_s = min(RS, nx - sx0 + HS) - bspan, nel_d = min(RD, nx - dx0 + HD) - dspan;
     const int n_edge = NP * nel_s + nel_d;
     const bool edge = n_edge > 0;                               // then every thread arrives too
     constexpr bool ASYNC = sizeof(Store) >= 4;
@@ -322,12 +326,13 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
     };
     auto keep_f = [&](const Real *f, Real *m) { keep_f_<QF>(A, f, m); };
     auto keep_h = [&](const Real *h, Real dT, Real *m) { keep_h_<QT>(A, h, dT, m); };
-    auto put_n_g = [&](int r, Real gref) {
-        Real gx, gy;
+    // the normal of row r; grad phi itself stays with the thread until the row collides (formed again there
+    // it cost 18 instructions a node)
+    auto put_n_g = [&](int r, Real gref, Real &gx, Real &gy) {
         grad_ref_(&s_phi[(r - 1) & 7][0], &s_phi[r & 7][0], &s_phi[(r + 1) & 7][0], ch + 2, gref, gx, gy);
         s_n[r & 3][ch + 1] = normal_(gx, gy, P.g2min);
     };
-    auto put_n = [&](int r) { put_n_g(r, __ldg(t_gref + r)); };
+    auto put_n = [&](int r, Real &gx, Real &gy) { put_n_g(r, __ldg(t_gref + r), gx, gy); };
     // After a wait gave up: flag the fault, let the copies this CTA started land, return.
     // (k_fail: the stage whose wait gave up; the later stages issued are waited for once
     // more, all within one further second.)  The path assumes that every issued copy, a
@@ -381,9 +386,10 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
         keep_h(t, put_sig(y0, t, dp), hm0);
     }
     __syncthreads();
+    Real gm0[2];   // grad phi of row y0
     if (doH) {
-        put_n(y0 - 1);
-        put_n(y0);
+        put_n(y0 - 1, gm0[0], gm0[1]);
+        put_n(y0, gm0[0], gm0[1]);
     }
 
     int sl = 0;          // slot of the stage of row y
@@ -393,7 +399,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
     // after it, row y collides.  The rings are deep enough that these writes never touch
     // rows the previous row's collision may still be reading.
     for (int y = y0; y < y1; ++y) {
-        Real fm3[2], hm1[3], g[9];
+        Real fm3[2], hm1[3], gm1[2], g[9];
         if (!mbar_wait_(&s_bar[sl], par)) s_abort = 1;
         Real rx[RX_N];   // this row's reference values, read before the slot is refilled
         load_rowref_(stage_rx(sl), rx);
@@ -408,7 +414,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
                 Real t[QT], dp;
                 read_h(std::false_type(), sl, y + 1, t, dp);
                 keep_h(t, put_sig(y + 1, t, dp), hm1);
-                put_n_g(y + 1, rx[RX_GREF1]);
+                put_n_g(y + 1, rx[RX_GREF1], gm1[0], gm1[1]);
             }
             if (colt) read_g(std::false_type(), sl, y, g);
         } else {
@@ -416,11 +422,11 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
                 Real t[QT], dp;
                 read_h(std::true_type(), sl, y + 1, t, dp);
                 keep_h(t, put_sig(y + 1, t, dp), hm1);
-                put_n_g(y + 1, rx[RX_GREF1]);
+                put_n_g(y + 1, rx[RX_GREF1], gm1[0], gm1[1]);
             }
             if (colt) read_g(std::true_type(), sl, y, g);
         }
-        const Real phi_ref = rx[RX_PHI0], th0 = rx[RX_TH0], c01 = rx[RX_C01], gref = rx[RX_GREF], p1 = rx[RX_P1];
+        const Real phi_ref = rx[RX_PHI0], th0 = rx[RX_TH0], c01 = rx[RX_C01], p1 = rx[RX_P1];
         // refill the slot read one row ago (every thread is past its reads) with row y + D - 1
         issue(y + D - 1, sl == 0 ? D - 1 : sl - 1);
         if (++sl == D) {
@@ -433,9 +439,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
             return;
         }
         if (xin) {
-            Real gpx, gpy;
-            grad_ref_(&s_phi[(y - 1) & 7][0], &s_phi[y & 7][0], &s_phi[(y + 1) & 7][0], tid + 2, gref, gpx, gpy);
-            node_step_<Real, Store, QF, QT>(A, x, y, s_phi[y & 7][tid + 2], gpx, gpy, tid + 1, s_n[(y - 1) & 3],
+            node_step_<Real, Store, QF, QT>(A, x, y, s_phi[y & 7][tid + 2], gm0[0], gm0[1], tid + 1, s_n[(y - 1) & 3],
                                             s_n[y & 3], s_n[(y + 1) & 3], s_sp[(y - 1) & 3], s_sp[y & 3],
                                             s_sp[(y + 1) & 3], fm0, hm0, g, phi_ref, th0, c01, p1);
         }
@@ -444,6 +448,7 @@ __device__ __forceinline__ void march_body(const StepArgs<Real, Store> &A, int s
             fm0[a] = fm1[a];
             fm1[a] = fm2[a];
             fm2[a] = fm3[a];
+            gm0[a] = gm1[a];
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a) hm0[a] = hm1[a];
@@ -535,50 +540,44 @@ cudaError_t launch_march_pack(const BatchPack<Real, Store> &B, int n_ctas, const
     return cudaLaunchKernelEx(&l.cfg, pack_kernel<Real, Store, QF, QT, TX>, B, active, seg);
 }
 
-// Segment length: the one that minimises the estimated step time, waves of resident CTAs
-// times (rows per segment + the ~6 start-up rows each segment re-derives), preferring longer
-// segments on ties.  Small grids get short segments (more CTAs in one wave); large grids
-// whole waves.  Segments are at least 8 rows.
-static int choose_segment(int strips, int ny, int slots)
+// Segment length.  FP32 arithmetic, from the waves of resident CTAs and the rows per segment plus the
+// ~6 start-up rows each segment re-derives.  Where segments of 16 rows and more make at least 2.5
+// waves, the CTAs of different age even each other out: (waves + 1/2) (rows + 6), e.g. 50 rows at
+// 8192 x 2048 (449 us with 48; 485 with the 187 rows that make one whole wave, 460 with 64).  Smaller
+// grids, and FP64 (bound by the pipe of the SM with the most CTAs: 1172 us in one whole wave of 54
+// rows at 2048 x 1024, 1231 to 2070 with 16 to 96): whole waves, preferring longer segments on ties.
+// Segments are at least 8 rows.
+static int choose_segment(int strips, int ny, int slots, bool fp64)
 {
     int best = ny;
-    long long best_cost = -1;
+    double best_cost = -1.0;
+    bool many = false;
     for (int nseg = 1; nseg <= (ny + 7) / 8; ++nseg) {
         const int seg = (ny + nseg - 1) / nseg;
         const int used = (ny + seg - 1) / seg;          // segments actually launched
-        const long long ctas = (long long)strips * used;
-        const long long waves = (ctas + slots - 1) / slots;
-        const long long cost = waves * (seg + 6);
-        if (best_cost < 0 || cost < best_cost) {
+        const double waves = double((long long)strips * used) / slots;
+        const bool m = !fp64 && waves >= 2.5 && seg >= 16;
+        if (many && !m) continue;
+        const double cost = (m ? waves + 0.5 : ceil(waves)) * (seg + 6);
+        if (best_cost < 0.0 || (m && !many) || cost < best_cost) {
             best_cost = cost;
             best = seg;
         }
+        many = m;
     }
     return best;
-}
-
-// resident CTAs of the step kernel on the device (per template instance)
-template <typename Real, typename Store, int QF, int QT>
-static int march_slots()
-{
-    constexpr int TX = march_width<Real>();
-    const int dyn = prepare_kernels<Real, Store, QF, QT>();
-    static int slots = 0;
-    if (slots == 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_kernel<Real, Store, QF, QT, TX>, TX + 32, dyn);
-        slots = sms * (per_sm > 0 ? per_sm : 1);
-    }
-    return slots;
 }
 
 template <typename Real, typename Store, int QF, int QT>
 int auto_segment(int nx, int ny)
 {
     constexpr int TX = march_width<Real>();
-    return choose_segment((nx + TX - 1) / TX, ny, march_slots<Real, Store, QF, QT>());
+    const int dyn = prepare_kernels<Real, Store, QF, QT>();
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_kernel<Real, Store, QF, QT, TX>, TX + 32, dyn);
+    return choose_segment((nx + TX - 1) / TX, ny, sms * (per_sm > 0 ? per_sm : 1), sizeof(Real) == 8);
 }
 
 template <typename Real, typename Store, int QF, int QT>
