@@ -175,19 +175,20 @@ template <typename R, typename S, int QF, int QT> struct StepFn {
         if (h->shape.rows > 0) return launch_march<R, S, QF, QT>(A, h->stream, h->shape.rows);
         // the stall hook acts on the copies that only the march has
         if (h->tx_extra) return launch_march<R, S, QF, QT>(A, h->stream, h->shapes.march.rows);
-        return launch_tile<R, S, QF, QT>(A, h->stream, h->shape.tx, h->shape.ty);
+        return launch_tile<R, S, QF, QT>(A, h->stream, h->shape);
     }
 };
 
 // Channels up to this many nodes (batches: in total) step on tiles, larger ones in marching strips.
 // The march reads no row twice and reaches the copy bandwidth once its strips fill the GPU for
-// several waves; the tiles win while they do not.  Measured (us a step, march / tiles): FP32 20.6 / 9.6
-// at 1024 x 256, 74 / 70 at 2048 x 1024, 126 / 134 at 4096 x 1024, 449 / 513 at 8192 x 2048.
-// FP16 storage is never bandwidth bound: 31 / 12 at 1024 x 256, 628 / 529 at 8192 x 2048.  FP64 (FP64 pipe):
-// 298 tiles at 1000 x 500 (1.68 nodes/ns), the march 1216 at 2048 x 1024 (1.72 nodes/ns, no halo of normals).
+// several waves; the tiles win while they do not.  Measured (us a step, march / tiles): FP32 20.6 / 8.8
+// at 1024 x 256, 74 / 66 at 2048 x 1024, 126 / 124 at 4096 x 1024, 238 / 242 at 4096 x 2048, 449 / 474 at
+// 8192 x 2048.
+// FP16 storage is never bandwidth bound: 31 / 9.9 at 1024 x 256, 310 / 222 at 8192 x 1024.  FP64 (FP64 pipe):
+// 893 / 881 at 1501 x 1001, 1175 / 1226 at 2048 x 1024 (the march forms no normal twice).
 static long long tile_nodes_max(int prec)
 {
-    return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 3LL << 20 : 1LL << 19);
+    return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 1LL << 22 : 1LL << 20);
 }
 // ny_total: the channel's rows (a batch: those of all its channels, put one on top of the other)
 template <typename R, typename S, int QF, int QT> struct ShapesFn {
@@ -197,9 +198,8 @@ template <typename R, typename S, int QF, int QT> struct ShapesFn {
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        out->tile = StepShape{0, 0, 0};
-        choose_tile<R, S, QF, QT>(h->nx, ny_total, sms, &out->tile.tx, &out->tile.ty);
-        out->march = StepShape{auto_segment<R, S, QF, QT>(h->nx, h->ny), 0, 0};
+        out->tile = choose_tile<R, S, QF, QT>(h->nx, ny_total, sms);
+        out->march = StepShape{auto_segment<R, S, QF, QT>(h->nx, h->ny), 0, 0, sms};
         out->automatic = h->nx * ny_total <= tile_nodes_max(h->prec) ? out->tile : out->march;
         return cudaGetLastError();
     }
@@ -865,7 +865,7 @@ int lbm_load(lbm_handle *h, const char *path)
 int lbm_set_segment(lbm_handle *h, int32_t rows)
 {
     if (!h || rows < 0) return LBM_EINVAL;
-    h->shape = rows > 0 ? StepShape{rows, 0, 0} : h->shapes.automatic;
+    h->shape = rows > 0 ? StepShape{rows, 0, 0, 0} : h->shapes.automatic;
     return LBM_OK;
 }
 
@@ -887,7 +887,7 @@ int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows)
     cand[nc++] = h->shapes.march;
     const int fixed[] = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256};
     for (int f : fixed)
-        if (f < h->ny && f != h->shapes.march.rows && nc < 16) cand[nc++] = StepShape{f, 0, 0};
+        if (f < h->ny && f != h->shapes.march.rows && nc < 16) cand[nc++] = StepShape{f, 0, 0, 0};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1038,13 +1038,12 @@ template <typename R, typename S, int QF, int QT> struct BatchStepFn {
             const BatchPack<R, S> &B = *reinterpret_cast<const BatchPack<R, S> *>(b->pack[par][macro].data());
             if (b->shape.rows > 0)
                 return launch_march_pack<R, S, QF, QT>(B, b->n_ctas, b->d_active, b->shape.rows, b->stream);
-            return launch_tile_pack<R, S, QF, QT>(B, b->n_ctas, b->d_active, b->shape.tx, b->shape.ty, b->stream);
+            return launch_tile_pack<R, S, QF, QT>(B, b->n_ctas, b->d_active, b->shape, b->stream);
         }
         const StepArgs<R, S> *args = (const StepArgs<R, S> *)(macro ? b->d_args_m[par] : b->d_args[par]);
         if (b->shape.rows > 0)
             return launch_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape.rows, b->stream);
-        return launch_tile_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape.tx, b->shape.ty,
-                                               b->stream);
+        return launch_tile_batch<R, S, QF, QT>(args, b->d_ctas, b->n_ctas, b->d_active, b->shape, b->stream);
     }
 };
 
@@ -1169,7 +1168,7 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
     const int fixed[] = {8, 12, 16, 24, 32, 48, 64, 96, 128};
     std::vector<StepShape> cand = {b->shapes.tile};
     for (int seg : fixed)
-        if (seg <= maxny || seg == fixed[0]) cand.push_back(StepShape{seg, 0, 0});
+        if (seg <= maxny || seg == fixed[0]) cand.push_back(StepShape{seg, 0, 0, 0});
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));

@@ -10,16 +10,16 @@
 namespace lbm {
 
 // How a step is launched: rows > 0: row-marching strips, each CTA walking that many rows; else
-// 2-D tiles of tx x ty nodes.
+// 2-D tiles of tx x ty nodes (sms: SMs of the device).
 struct StepShape {
-    int rows, tx, ty;
+    int rows, tx, ty, sms;
 };
 
 // One time step from A's input buffers to its output buffers.
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int rows);
 template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, int tx, int ty);
+cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const StepShape &shape);
 
 // Many cases in one launch.  Up to PACK_CASES of them travel in the launch's parameters: their arguments
 // are then uniform values in constant memory, as those of a single channel are (fetched through
@@ -45,18 +45,18 @@ cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, i
                          cudaStream_t s);
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active,
-                              int tx, int ty, cudaStream_t s);
+                              const StepShape &shape, cudaStream_t s);
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_march_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int seg, cudaStream_t s);
 template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int tx, int ty,
+cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, const StepShape &shape,
                              cudaStream_t s);
 // Columns per strip of the march.
 template <typename Real, typename Store, int QF, int QT> int step_strip_width();
 // Rows per segment of the march when none is set (whole waves of resident CTAs).
 template <typename Real, typename Store, int QF, int QT> int auto_segment(int nx, int ny);
 // Tile shape for a channel on a device with `sms` SMs.
-template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx, long long ny, int sms, int *tx, int *ty);
+template <typename Real, typename Store, int QF, int QT> StepShape choose_tile(int nx, long long ny, int sms);
 
 // Initialisation: macro [5][ny][nx] (phi, u, v, T, dp) holds the fields; entries whose
 // bit in `defaults` (1 phi, 2 u, 4 v, 8 T, 16 dp) is set are filled with the defaults

@@ -53,32 +53,32 @@ __device__ __forceinline__ void grad_ref_(const double *rm, const double *r0, co
 }
 
 // Loads of one node for the pull: populations of one lattice (plane base pointers `pl`,
-// wall rule KIND) at row y and column x, with the wall rules of Sec. 5.1.  Offsets are
-// 32-bit element indices.  WALLS = false: no link of the row crosses a wall.
+// wall rule KIND) at row y and column x, with the wall rules of Sec. 5.1.  WALLS = false: no link of
+// the row crosses a wall.
 //   KIND 0: phase field, specular reflection (free slip, no flux through the wall)
 //   KIND 1: flow, halfway bounce-back (no slip)
 //   KIND 2: energy, anti-bounce-back to the wall temperature where the link crosses the wall
 // Values come out in stored units (for FP16 storage: times its scale; wscale multiplies
-// the anti-bounce-back wall term accordingly).
+// the anti-bounce-back wall term accordingly).  Addresses are a plane's base plus an unsigned 32-bit
+// byte offset (base plus element index took a 64-bit multiply-add per load).
 template <int KIND, int Q, bool WALLS = true, typename Real, typename Store>
 __device__ __forceinline__ void pull_row_(const Store *const *pl, int pitch, int ny, int nx, int y, int x, int xm,
                                           int xp, Real wscale, const Real *__restrict__ twall, Real dTcold, Real *out)
 {
-    const int r0 = y * pitch;
+    const uint32_t S = sizeof(Store), r0 = uint32_t(y) * uint32_t(pitch) * S, dr = uint32_t(pitch) * S;
+    auto at = [&](const Store *base, uint32_t row, int col) {
+        return ld_<Real, Store>(
+            reinterpret_cast<const Store *>(reinterpret_cast<const char *>(base) + (row + uint32_t(col) * S)));
+    };
 #pragma unroll
     for (int a = 0; a < Q; ++a) {
         const int ex = ex_(a), ey = ey_(a);
         const int xs = ex > 0 ? xm : (ex < 0 ? xp : x);
         const bool wall = WALLS && ((ey > 0 && y == 0) || (ey < 0 && y == ny - 1));
         Real v;
-        if (!wall) {
-            const int rs = ey > 0 ? r0 - pitch : (ey < 0 ? r0 + pitch : r0);
-            v = ld_<Real, Store>(pl[a] + (rs + xs));
-        } else if (KIND == 0) {
-            v = ld_<Real, Store>(pl[mir_(a)] + (r0 + xs));
-        } else {
-            v = ld_<Real, Store>(pl[opp_(a)] + (r0 + x));
-        }
+        if (!wall) v = at(pl[a], ey > 0 ? r0 - dr : (ey < 0 ? r0 + dr : r0), xs);
+        else if (KIND == 0) v = at(pl[mir_(a)], r0, xs);
+        else v = at(pl[opp_(a)], r0, x);
         if (KIND == 2 && wall) {
             const Real tw = ey > 0 ? twall[(1 - ex) * nx + x] : dTcold;
             Real t = Real(2.0 * w_<Q>(a)) * tw;

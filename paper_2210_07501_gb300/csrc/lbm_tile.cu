@@ -1,11 +1,12 @@
 // lbm_tile.cu -- the step on 2-D tiles: one node per thread, all rows of a tile at once.
 //
 // The row-marching kernel (lbm_step.cu) walks a strip row by row, so a channel with few strips
-// pays its ~1.5 us per row in series on a few SMs: 22 us a step at 128 x 32 (4 CTAs), 21 us at
-// 1024 x 256 (256 CTAs of 8 + 6 rows).  Here every node has its thread; the two rows and columns
+// pays its ~1.5 us per row in series on a few SMs: 22 us a step at 128 x 32 (4 CTAs; 3.2 here), 21 us
+// at 1024 x 256 (256 CTAs of 8 + 6 rows; 8.8 here).  Here every node has its thread; the two rows and columns
 // around a tile are pulled again by its CTA (phi; sigma and p on the inner ring), the normals of
 // the inner ring are formed again, and the step is one latency: load, barrier, normals,
-// barrier, collide, store.  The arithmetic of a node is that of lbm_node.cuh, so the
+// barrier, collide, store.  Bound in FP32 arithmetic by instruction issue (~640 a node, half of the
+// cycles) and the latency of the two barriers, in FP64 by the FP64 pipe.  The arithmetic of a node is that of lbm_node.cuh, so the
 // results are the march's bit for bit.
 #include "lbm_internal.h"
 #include "lbm_node.cuh"
@@ -14,13 +15,14 @@ namespace lbm {
 
 // FP32 arithmetic: tiles of 32 x 8 with compile-time strides; FP64: any shape of up to 256 nodes,
 // chosen for the channel (choose_tile).
-template <typename Real, typename Store> struct TileGeo {
+template <typename Real, typename Store, int QF = 5, int QT = 5> struct TileGeo {
     static constexpr bool FIXED = sizeof(Real) == 4;
     static constexpr int NT = 256, TX = 32;
-    // FP32: four CTAs per SM (64 registers; three of 80: 14 % slower at 1024 x 256; five of 48: 10 %).
-    // FP16: five (48 registers): 529 us at 8192 x 2048 against 607 with four, the conversions
-    // and the smaller loads leave it latency bound.  FP64 takes the registers it needs.
-    static constexpr int CTAS = sizeof(Real) == 8 ? 1 : (sizeof(Store) == 2 ? 5 : 4);
+    // FP32: four CTAs per SM (64 registers; three: 9.8 us instead of 8.8 at 1024 x 256, five: 9.1, and 14.3
+    // instead of 11.8 with three D2Q9 lattices).  FP16, latency bound on its smaller loads: five (48
+    // registers; 222 us at 8192 x 1024, 240 with four), four with two D2Q9 scalar lattices, which
+    // spill at 48.  FP64 takes the registers it needs.
+    static constexpr int CTAS = sizeof(Real) == 8 ? 1 : (sizeof(Store) == 2 && QF + QT < 18 ? 5 : 4);
 };
 
 template <typename Real, typename Store, int QF, int QT>
@@ -56,16 +58,7 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
             pull_row_<1, 9, WALLS>(A.gi, pitch, ny, nx, y, x, xm, xp, A.sg, A.twall, A.P.dTcold, g);
         }
         // the two halo rows and columns around the tile: phi, and sigma and p on the inner ring
-        const int nr = 4 * (ex + 4 + ey);
-        for (int i = t; i < nr; i += NT) {
-            int hx, hy;
-            if (i < 4 * (ex + 4)) {
-                const int r = i / (ex + 4);
-                hx = i - r * (ex + 4) - 2, hy = r < 2 ? r - 2 : ey + r - 2;
-            } else {
-                const int j = i - 4 * (ex + 4), k = j & 3;
-                hx = k < 2 ? k - 2 : ex + k - 2, hy = j >> 2;
-            }
+        auto halo = [&](int hx, int hy) {
             int X = x0 + hx;
             X = X < 0 ? X + nx : (X >= nx ? X - nx : X);
             const int xm = X == 0 ? nx - 1 : X - 1, xp = X == nx - 1 ? 0 : X + 1;
@@ -79,6 +72,29 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
                 s_sp[(hy + 1) * SX + hx + 1] = sig_p_(A, r, X, temp_dev_<QT>(A, v), pv);
             }
             s_phi[(hy + 2) * PX + hx + 2] = phi_dev_<QF>(A, q, t_dR[gy], t_dRlo[gy]);
+        };
+        if constexpr (G::FIXED) {
+            // a warp per halo row (the columns of the tile), then the side columns, four a row:
+            // no division (by the ragged width) on the way to the loads
+            static_assert(G::TX == 32 && 4 * 32 + 4 * (G::NT / 32 + 4) <= G::NT, "one halo node per thread");
+            if (t < 4 * 32) {
+                const int r = t >> 5, hx = t & 31;
+                if (hx < ex) halo(hx, r < 2 ? r - 2 : ey + r - 2);
+            } else if (t < 4 * 32 + 4 * (ey + 4)) {
+                const int j = t - 4 * 32, k = j & 3;
+                halo(k < 2 ? k - 2 : ex + k - 2, (j >> 2) - 2);
+            }
+        } else {
+            const int nr = 4 * (ex + 4 + ey);
+            for (int i = t; i < nr; i += NT) {
+                if (i < 4 * (ex + 4)) {
+                    const int r = i / (ex + 4);
+                    halo(i - r * (ex + 4) - 2, r < 2 ? r - 2 : ey + r - 2);
+                } else {
+                    const int j = i - 4 * (ex + 4), k = j & 3;
+                    halo(k < 2 ? k - 2 : ex + k - 2, j >> 2);
+                }
+            }
         }
         if (own) {
             dphi = phi_dev_<QF>(A, f, t_dR[y], t_dRlo[y]);
@@ -100,15 +116,26 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
     };
     Real gpx, gpy;   // grad phi of the thread's own node
     if (own) put_n(lx, ly, gpx, gpy);
-    for (int i = NT - 1 - t; i < 2 * (ex + 2 + ey); i += NT) {
+    {
         Real gx, gy;
-        if (i < 2 * (ex + 2)) put_n(i < ex + 2 ? i - 1 : i - (ex + 2) - 1, i < ex + 2 ? -1 : ey, gx, gy);
-        else put_n((i & 1) ? -1 : ex, (i - 2 * (ex + 2)) >> 1, gx, gy);
+        if constexpr (G::FIXED) {   // the last warps: the rows below and above, then the sides
+            const int i = NT - 1 - t;
+            if (i < 2 * 32) {
+                if ((i & 31) < ex) put_n(i & 31, i < 32 ? -1 : ey, gx, gy);
+            } else if (i < 2 * 32 + 2 * (ey + 2)) {
+                put_n((i & 1) ? -1 : ex, ((i - 2 * 32) >> 1) - 1, gx, gy);
+            }
+        } else {
+            for (int i = NT - 1 - t; i < 2 * (ex + 2 + ey); i += NT) {
+                if (i < 2 * (ex + 2)) put_n(i < ex + 2 ? i - 1 : i - (ex + 2) - 1, i < ex + 2 ? -1 : ey, gx, gy);
+                else put_n((i & 1) ? -1 : ex, (i - 2 * (ex + 2)) >> 1, gx, gy);
+            }
+        }
     }
+    Real rx[RX_N];   // the row's reference values (on their way across the barrier)
+    if (own) load_rowref_(A.rowx + (long long)y * RX_N, rx);
     __syncthreads();
     if (own) {
-        Real rx[RX_N];
-        load_rowref_(A.rowx + (long long)y * RX_N, rx);
         const R2 *n = s_n + (ly + 1) * SX, *q = s_sp + (ly + 1) * SX;
         node_step_<Real, Store, QF, QT>(A, x, y, dphi, gpx, gpy, lx + 1, n - SX, n, n + SX, q - SX, q, q + SX, fm, hm,
                                         g, rx[RX_PHI0], rx[RX_TH0], rx[RX_C01], rx[RX_P1]);
@@ -120,7 +147,7 @@ __device__ __forceinline__ void tile_body(const StepArgs<Real, Store> &A, int tx
 // before it, so all memory of earlier steps is visible and every launch ends after its
 // predecessor.  Saves 2.5 us of 6 us a step at 128 x 32.  FP64 lets the next launch start only at its
 // own end: its CTAs would otherwise settle beside running ones and leave other SMs empty (200 x 100,
-// tiles of 128: 62 us a step instead of 47).
+// tiles of 128: 62 us a step instead of 47; see also tile_smem).
 template <typename Real> __device__ __forceinline__ void let_next_start_early_()
 {
     if (sizeof(Real) == 4) pdl_launch_next_();
@@ -131,7 +158,7 @@ template <typename Real> __device__ __forceinline__ void let_next_start_late_()
 }
 
 template <typename Real, typename Store, int QF, int QT>
-__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store>::CTAS)
+__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store, QF, QT>::CTAS)
 tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -144,7 +171,7 @@ tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty)
 // Many channels in one launch: CTA i works on tile (ctas[i].y, ctas[i].z) of case ctas[i].x, whose
 // arguments it copies to shared memory (before the wait: they are constant).
 template <typename Real, typename Store, int QF, int QT>
-__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store>::CTAS)
+__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store, QF, QT>::CTAS)
 tile_batch_kernel(const StepArgs<Real, Store> *__restrict__ cases, const int4 *__restrict__ ctas,
                   const int *__restrict__ active, int tx, int ty)
 {
@@ -165,7 +192,7 @@ tile_batch_kernel(const StepArgs<Real, Store> *__restrict__ cases, const int4 *_
 
 // The same with up to PACK_CASES channels' arguments in the launch's parameters.
 template <typename Real, typename Store, int QF, int QT>
-__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store>::CTAS)
+__global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store, QF, QT>::CTAS)
 tile_pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *active, int tx, int ty)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -176,32 +203,53 @@ tile_pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *ac
     let_next_start_late_<Real>();
 }
 
-template <typename Real> static size_t tile_smem(int tx, int ty)
+// Dynamic shared memory of a launch of `tiles` tiles.  In FP64 a step takes as long as the SM with the
+// most tiles, so no SM may take more than its share: the request is raised until only that many
+// CTAs fit (otherwise CTAs settle two to an SM while the launch before still holds others: 33 us
+// instead of 24 a step at 200 x 100 with 130 tiles on 152 SMs).
+template <typename Real> static size_t tile_smem(int tx, int ty, long long tiles, int sms)
 {
-    return ((size_t)(ty + 4) * (tx + 4) + 4 * (size_t)(ty + 2) * (tx + 2)) * sizeof(Real);
+    const size_t need = ((size_t)(ty + 4) * (tx + 4) + 4 * (size_t)(ty + 2) * (tx + 2)) * sizeof(Real);
+    const long long share = (tiles + sms - 1) / sms;   // CTAs an SM has to take
+    if (sizeof(Real) == 4 || share > 4) return need;
+    // 228 KiB per SM, 1 KiB of it reserved per CTA; one CTA may have 227 KiB
+    const size_t most = (size_t)(228 / (share + 1)) * 1024;   // share + 1 CTAs of more than this do not fit
+    return need > most ? need : most;
+}
+
+// FP64 launches may ask for more than 48 KiB.
+template <typename K> static void allow_smem(K kernel, size_t bytes)
+{
+    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, int tx, int ty)
+cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const StepShape &shape)
 {
-    PdlLaunch l(dim3((A.nx + tx - 1) / tx, (A.ny + ty - 1) / ty), dim3((tx * ty + 31) / 32 * 32),
-                tile_smem<Real>(tx, ty), s);
+    const int tx = shape.tx, ty = shape.ty, gx = (A.nx + tx - 1) / tx, gy = (A.ny + ty - 1) / ty;
+    PdlLaunch l(dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
+                tile_smem<Real>(tx, ty, (long long)gx * gy, shape.sms), s);
+    allow_smem(tile_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
     return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active,
-                              int tx, int ty, cudaStream_t s)
+                              const StepShape &shape, cudaStream_t s)
 {
-    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty), s);
+    const int tx = shape.tx, ty = shape.ty;
+    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty, n_ctas, shape.sms), s);
+    allow_smem(tile_batch_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
     return cudaLaunchKernelEx(&l.cfg, tile_batch_kernel<Real, Store, QF, QT>, cases, ctas, active, tx, ty);
 }
 
 template <typename Real, typename Store, int QF, int QT>
-cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int tx, int ty,
+cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, const StepShape &shape,
                              cudaStream_t s)
 {
-    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty), s);
+    const int tx = shape.tx, ty = shape.ty;
+    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty, n_ctas, shape.sms), s);
+    allow_smem(tile_pack_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
     return cudaLaunchKernelEx(&l.cfg, tile_pack_kernel<Real, Store, QF, QT>, B, active, tx, ty);
 }
 
@@ -209,11 +257,11 @@ cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const 
 // instruction), so what counts is the FP64 instructions of the SM with the most tiles: warps of
 // nodes, the inner ring's normals, the outer ring's phi, and a start-up of ~150 (the shapes this
 // ranks first are within 3 % of the best measured at 200 x 100, 160 x 320 and 1024 x 256).
-template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx, long long ny, int sms, int *tx, int *ty)
+template <typename Real, typename Store, int QF, int QT> StepShape choose_tile(int nx, long long ny, int sms)
 {
     using G = TileGeo<Real, Store>;
-    *tx = G::TX, *ty = G::NT / G::TX;
-    if (G::FIXED) return;
+    StepShape best_shape = {0, G::TX, G::NT / G::TX, sms};
+    if (G::FIXED) return best_shape;
     const double node = 260.0 + 14.0 * (QF + QT - 10), normal = 36.0, pull = 13.0, start = 150.0;
     auto warps = [](int n) { return double((n + 31) / 32); };
     double best = -1.0;
@@ -222,17 +270,18 @@ template <typename Real, typename Store, int QF, int QT> void choose_tile(int nx
             const long long tiles = a * ((ny + h - 1) / h);
             const double cost = double((tiles + sms - 1) / sms) *
                                 (warps(w * h) * node + warps(2 * (w + 2 + h)) * normal + warps(4 * (w + 4 + h)) * pull + start);
-            if (best < 0.0 || cost < best) best = cost, *tx = w, *ty = h;
+            if (best < 0.0 || cost < best) best = cost, best_shape.tx = w, best_shape.ty = h;
         }
+    return best_shape;
 }
 
-#define LBM_INST(R, S, QF, QT)                                                                                  \
-    template cudaError_t launch_tile<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, int, int);            \
-    template cudaError_t launch_tile_batch<R, S, QF, QT>(const StepArgs<R, S> *, const int4 *, int, const int *, \
-                                                         int, int, cudaStream_t);                              \
-    template cudaError_t launch_tile_pack<R, S, QF, QT>(const BatchPack<R, S> &, int, const int *, int, int,    \
-                                                        cudaStream_t);                                         \
-    template void choose_tile<R, S, QF, QT>(int, long long, int, int *, int *);
+#define LBM_INST(R, S, QF, QT)                                                                                    \
+    template cudaError_t launch_tile<R, S, QF, QT>(const StepArgs<R, S> &, cudaStream_t, const StepShape &);       \
+    template cudaError_t launch_tile_batch<R, S, QF, QT>(const StepArgs<R, S> *, const int4 *, int, const int *,    \
+                                                         const StepShape &, cudaStream_t);                        \
+    template cudaError_t launch_tile_pack<R, S, QF, QT>(const BatchPack<R, S> &, int, const int *,                 \
+                                                        const StepShape &, cudaStream_t);                         \
+    template StepShape choose_tile<R, S, QF, QT>(int, long long, int);
 LBM_INST(double, double, 5, 5)
 LBM_INST(double, double, 5, 9)
 LBM_INST(double, double, 9, 5)
