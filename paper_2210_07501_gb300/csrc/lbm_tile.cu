@@ -5,9 +5,9 @@
 // at 1024 x 256 (256 CTAs of 8 + 6 rows; 8.8 here).  Here every node has its thread; the two rows and columns
 // around a tile are pulled again by its CTA (phi; sigma and p on the inner ring), the normals of
 // the inner ring are formed again, and the step is one latency: load, barrier, normals,
-// barrier, collide, store.  Bound in FP32 arithmetic by instruction issue (~640 a node, half of the
-// cycles) and the latency of the two barriers, in FP64 by the FP64 pipe.  The arithmetic of a node is that of lbm_node.cuh, so the
-// results are the march's bit for bit.
+// barrier, collide, store.  Bound in FP32 arithmetic by instruction issue and the latency
+// of the loads and of the two barriers, in FP64 by the FP64 pipe.  The arithmetic of a node is that of
+// lbm_node.cuh, so the results are the march's bit for bit.
 #include "lbm_internal.h"
 #include "lbm_node.cuh"
 
@@ -159,12 +159,14 @@ template <typename Real> __device__ __forceinline__ void let_next_start_late_()
 
 template <typename Real, typename Store, int QF, int QT>
 __global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store, QF, QT>::CTAS)
-tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty)
+tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty, int gx)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     let_next_start_early_<Real>();
+    int bx = blockIdx.x, by = blockIdx.y;
+    if (gx) by = bx / gx, bx -= by * gx;   // more tile rows than a grid has in y
     pdl_wait_();
-    tile_body<Real, Store, QF, QT>(A, tx, ty, blockIdx.x, blockIdx.y, smem);
+    tile_body<Real, Store, QF, QT>(A, tx, ty, bx, by, smem);
     let_next_start_late_<Real>();
 }
 
@@ -227,10 +229,11 @@ template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const StepShape &shape)
 {
     const int tx = shape.tx, ty = shape.ty, gx = (A.nx + tx - 1) / tx, gy = (A.ny + ty - 1) / ty;
-    PdlLaunch l(dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
+    const bool flat = gy > 65535;
+    PdlLaunch l(flat ? dim3((unsigned)gx * gy) : dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
                 tile_smem<Real>(tx, ty, (long long)gx * gy, shape.sms), s);
     allow_smem(tile_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
-    return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty);
+    return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty, flat ? gx : 0);
 }
 
 template <typename Real, typename Store, int QF, int QT>
@@ -265,9 +268,9 @@ template <typename Real, typename Store, int QF, int QT> StepShape choose_tile(i
     const double node = 260.0 + 14.0 * (QF + QT - 10), normal = 36.0, pull = 13.0, start = 150.0;
     auto warps = [](int n) { return double((n + 31) / 32); };
     double best = -1.0;
-    for (int a = (nx + 63) / 64; a <= (nx + 7) / 8; ++a)
-        for (int w = (nx + a - 1) / a, h = 2; h <= 32 && w * h <= G::NT; ++h) {
-            const long long tiles = a * ((ny + h - 1) / h);
+    for (int w = nx < 64 ? nx : 64; w >= 8 || w == nx; --w)
+        for (int h = 2; h <= 32 && w * h <= G::NT; ++h) {
+            const long long tiles = (nx + w - 1) / w * ((ny + h - 1) / h);
             const double cost = double((tiles + sms - 1) / sms) *
                                 (warps(w * h) * node + warps(2 * (w + 2 + h)) * normal + warps(4 * (w + 4 + h)) * pull + start);
             if (best < 0.0 || cost < best) best = cost, best_shape.tx = w, best_shape.ty = h;

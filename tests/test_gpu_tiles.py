@@ -32,6 +32,21 @@ def test_tiles_equal_marching_strips(precision, qf, qt, nx, ny):
         assert np.array_equal(got[0][k], got[1][k]), k
 
 
+def test_more_tile_rows_than_a_grid_has():
+    """A channel of more than 65535 rows of tiles (their launch is one-dimensional)."""
+    from paper_2210_07501_gb300 import Lbm
+    w = WL.channel(3, 524300, 524290.0, W=3.0, sigma1=-3e-4, heat_periods=1)
+    got = []
+    for rows in (0, 64):
+        g = Lbm(w["domain"], w["params"], precision="fp32")
+        g.lbm_set_segment(rows)
+        g.lbm_step(3)
+        got.append(g.lbm_fields())
+        g.close()
+    for k in got[0]:
+        assert np.array_equal(got[0][k], got[1][k]), k
+
+
 @pytest.mark.parametrize("precision,n", [("fp32", 32), ("fp32", 33), ("fp64", 1), ("fp64", 33), ("fp16", 32)])
 def test_batches_of_any_number_equal_single_channels(precision, n):
     """Batches of up to 32 channels carry their arguments in the launch's parameters, larger ones read
