@@ -34,18 +34,8 @@ template <typename A> __device__ __forceinline__ A from_f(float v)
     if constexpr (std::is_same<A, __nv_bfloat16>::value) return __float2bfloat16_rn(v);
     else return v;
 }
-// an input value as the activation type holds it; a result as the output holds it (rounded
-// to the activation type also where it is handed out in float)
-template <typename A, typename In> __device__ __forceinline__ float load_as(In v)
-{
-    if constexpr (std::is_same<In, A>::value) return to_f(v);
-    else return to_f(from_f<A>(v));
-}
-template <typename A, typename Out> __device__ __forceinline__ Out store_as(float v)
-{
-    if constexpr (std::is_same<Out, A>::value) return from_f<A>(v);
-    else return to_f(from_f<A>(v));
-}
+// a float as the activation type holds it
+template <typename A> __device__ __forceinline__ float rounded(float v) { return to_f(from_f<A>(v)); }
 __device__ __forceinline__ float silu(float z) { return z / (1.0f + __expf(-z)); }
 __device__ __forceinline__ float dsilu(float z)
 {
@@ -53,13 +43,33 @@ __device__ __forceinline__ float dsilu(float z)
     return s * (1.0f + z * (1.0f - s));
 }
 
+// four consecutive aligned values
+__device__ __forceinline__ void load4(const float *p, float *v)
+{
+    const float4 u = *reinterpret_cast<const float4 *>(p);
+    v[0] = u.x, v[1] = u.y, v[2] = u.z, v[3] = u.w;
+}
+__device__ __forceinline__ void store4(float *p, const float *v)
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void load4(const __nv_bfloat16 *p, __nv_bfloat16 *v)
+{
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    reinterpret_cast<uint32_t *>(v)[0] = u.x, reinterpret_cast<uint32_t *>(v)[1] = u.y;
+}
+__device__ __forceinline__ void store4(__nv_bfloat16 *p, const __nv_bfloat16 *v)
+{
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+    *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
+}
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // ---- 3x3 convolutions on the FP32 pipes ----------------------------------------------------
-// Forward (BWD = false): y[b][co][h][w] = bias[co] + sum_{ci, dy, dx} w[co][ci][dy][dx] a[b][ci][h+dy-1][w+dx-1],
-// a = x (first layer) or silu(x).  Data gradient (BWD = true): the same sum over the layer's output
-// channels with the kernel flipped, times silu'(z) of the pixel.
+// Forward (BWD = false): y[b][co][h][w] = bias[co] + sum_{ci, dy, dx} w[co][ci][dy][dx] a[b][ci][h+dy-1][w+dx-1].
+// Data gradient (BWD = true): the same sum over the layer's output channels with the kernel flipped, times
+// silu'(z) of the pixel.
 //
 // Bound: FP32 multiply-adds (2.4 G per 32 -> 32 layer at batch 16 of 256 x 64: 62 us at 80 TFLOP/s).  The
 // weights are kept in FP32 and the sums in FP32 in one order (per input channel the nine taps in
@@ -68,9 +78,10 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // with the layer's channels swapped (weight_place, kept by set_params and the Adam step).
 // A thread holds 4 pixels of a row x COG output channels: per weight quad from shared memory (one
 // 16-byte broadcast) 8 packed FMAs (two channels each), per input channel 18 input values for 36 taps.
-// 124 us a 32 -> 32 layer (304 us with one pixel a thread and one scalar FMA per weight read), half of
-// the FP32 peak; the rest is staging (silu and its division on every input, 1.3 times with the
-// halo) that the four CTAs per SM overlap only in part.  Tiles of 16 rows: 141 us.
+// The inputs come as the values that are multiplied, in float (silu is applied once, where the layer
+// before stores), so staging is asynchronous copies, the next channels' while these are multiplied.
+// 110 us a 32 -> 32 layer at 16 x 256 x 64, 0.6 of the FP32 peak (304 us with one pixel a thread and one
+// scalar FMA per weight read; 124 with silu and its division applied on staging).
 constexpr int CCH = 8;         // input channels staged per pass
 template <int CO, int COG_, int TWQ_, int TH_> struct Tile {
     static constexpr int COG = COG_, TWQ = TWQ_, TH = TH_;   // channels a thread, pixel quads a row, rows
@@ -78,62 +89,80 @@ template <int CO, int COG_, int TWQ_, int TH_> struct Tile {
     static constexpr int NT = NC < 128 ? 128 : NC;           // threads (all stage)
 };
 
-// The rows iy < ROWS (image rows h0 - 1 + iy, zero outside) and columns ix < COLS + 2 (image columns
-// w0 - 1 + ix, wrapped; columns past the wrapped one are zero, they are not used) of nc planes of x,
-// through f, into dst[c * PLANE + iy * PW + ix].  NT threads: COLS by row, then the two edge
-// columns; U loads of a thread in flight (one at a time left the kernels waiting for memory two
-// thirds of their time).
-template <int NT, int COLS, int ROWS, int PW, int PLANE, int U, typename In, typename F>
-__device__ __forceinline__ void stage_planes(const In *x, int nc, int h0, int w0, int H, int W, float *dst, F f)
+// ---- staging by asynchronous copies ----
+__device__ __forceinline__ void copy_async16(float *dst, const float *src, bool in)
 {
-    constexpr int RG = NT / COLS;
-    const int col = threadIdx.x % COLS, ww0 = w0 + col, rows = nc * ROWS;
-    const int wc = ww0 < W ? ww0 : (ww0 == W ? 0 : -1);
-    for (int r0 = threadIdx.x / COLS; r0 < rows; r0 += RG * U) {
-        In v[U];
-        bool in[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int r = r0 + u * RG, c = r / ROWS, hh = h0 + r - c * ROWS - 1;
-            in[u] = r < rows && hh >= 0 && hh < H && wc >= 0;
-            if (in[u]) v[u] = x[((long long)c * H + hh) * W + wc];
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int r = r0 + u * RG, c = r / ROWS;
-            if (r < rows) dst[c * PLANE + (r - c * ROWS) * PW + col + 1] = in[u] ? f(v[u]) : 0.f;
-        }
-    }
-    for (int e = threadIdx.x; e < 2 * rows; e += NT) {
-        const int r = e >> 1, c = r / ROWS, hh = h0 + r - c * ROWS - 1, ix = e & 1 ? COLS + 1 : 0;
-        int ww = w0 - 1 + ix;
-        ww = ww < 0 ? W - 1 : (ww < W ? ww : (ww == W ? 0 : -1));
-        const bool in = hh >= 0 && hh < H && ww >= 0;
-        dst[c * PLANE + (r - c * ROWS) * PW + ix] = in ? f(x[((long long)c * H + hh) * W + ww]) : 0.f;
-    }
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 16 : 0)
+                 : "memory");
 }
-// 16-byte aligned words of global memory into shared memory (cp.async; stage_wait before use)
-template <int NT> __device__ __forceinline__ void stage_words(const float *src, int n4, float *dst)
+__device__ __forceinline__ void copy_async4(float *dst, const float *src, bool in)
 {
-    for (int e = threadIdx.x; e < n4; e += NT)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + 4 * e)),
-                     "l"(src + 4 * e)
-                     : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(in ? 4 : 0)
+                 : "memory");
 }
-__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int CI, int CO, typename T, bool BWD, bool ACT, typename In, typename A, typename Out>
+// The rows iy < ROWS (image rows h0 - 1 + iy, zero outside) of nc planes of x into dst[c PLANE + iy PW +
+// 4 + column]: COLS columns from w0 on, the column before at 3 and the one after (wrapped: the image
+// is periodic in x; past the wrapped one zero).  vec: W a multiple of 4 and x on a 16-byte boundary.
+template <int NT, int COLS, int ROWS, int PW, int PLANE>
+__device__ __forceinline__ void stage_planes(const float *x, int nc, int h0, int w0, int H, int W, float *dst, bool vec)
+{
+    const int rows = nc * ROWS;
+    if (vec) {
+        for (int e = threadIdx.x; e < rows * (COLS / 4); e += NT) {
+            const int r = e / (COLS / 4), q = e % (COLS / 4), c = r / ROWS, iy = r - c * ROWS, hh = h0 + iy - 1;
+            const int ww = w0 + 4 * q;
+            float *d = dst + c * PLANE + iy * PW + 4 + 4 * q;
+            const bool in = hh >= 0 && hh < H;
+            const float *row = x + ((long long)c * H + (in ? hh : 0)) * W;
+            if (ww < W) copy_async16(d, row + ww, in);
+            else *reinterpret_cast<float4 *>(d) = make_float4(ww == W && in ? row[0] : 0.f, 0.f, 0.f, 0.f);
+        }
+        for (int e = threadIdx.x; e < 2 * rows; e += NT) {
+            const int r = e >> 1, c = r / ROWS, iy = r - c * ROWS, hh = h0 + iy - 1;
+            const int ww = e & 1 ? w0 + COLS : (w0 == 0 ? W - 1 : w0 - 1);
+            const bool in = hh >= 0 && hh < H && ww <= W;
+            copy_async4(dst + c * PLANE + iy * PW + (e & 1 ? 4 + COLS : 3),
+                        x + ((long long)c * H + (in ? hh : 0)) * W + (ww < W ? ww : 0), in);
+        }
+    } else {
+        for (int e = threadIdx.x; e < rows * (COLS + 2); e += NT) {
+            const int r = e / (COLS + 2), ix = e - r * (COLS + 2), c = r / ROWS, iy = r - c * ROWS, hh = h0 + iy - 1;
+            const int ww = w0 + ix - 1;
+            const bool in = hh >= 0 && hh < H && ww <= W;
+            copy_async4(dst + c * PLANE + iy * PW + 3 + ix,
+                        x + ((long long)c * H + (in ? hh : 0)) * W + (ww < 0 ? W - 1 : (ww < W ? ww : 0)), in);
+        }
+    }
+}
+
+template <int CI, int CO, typename T, bool BWD, bool LAST, typename A, typename Out>
 __global__ void __launch_bounds__(T::NT, 512 / T::NT)
-conv3x3(const In *x, const float *wgt, const float *bias, const A *zin, Out *y, int H, int W)
+conv3x3(const float *x, const float *wgt, const float *bias, const A *zin, Out *y, float *act, int H, int W, bool vec_in)
 {
     constexpr int COG = T::COG, TWQ = T::TWQ, TH = T::TH, NT = T::NT;
-    constexpr int PW = TWQ * 4 + 4, PLANE = (TH + 2) * PW;
-    __shared__ __align__(16) float s_x[CCH * PLANE];
-    __shared__ __align__(16) float s_w[CCH * 9 * CO];
+    constexpr int PW = TWQ * 4 + 8, PLANE = (TH + 2) * PW, NCHUNK = (CI + CCH - 1) / CCH;
+    constexpr int STAGES = NCHUNK > 1 ? 2 : 1;
+    __shared__ __align__(16) float s_x[STAGES][CCH * PLANE];
+    __shared__ __align__(16) float s_w[STAGES][CCH * 9 * CO];
     const int q = threadIdx.x % TWQ, row = threadIdx.x / TWQ % TH, cg = threadIdx.x / (TWQ * TH);
     const bool on = T::NC == NT || threadIdx.x < T::NC;
-    const int w0 = blockIdx.x * (TWQ * 4), h0 = blockIdx.y * TH, b = blockIdx.z;
+    const int tw = (W + TWQ * 4 - 1) / (TWQ * 4), ty = blockIdx.x / tw, b = blockIdx.z;
+    const int w0 = (blockIdx.x - ty * tw) * (TWQ * 4), h0 = ty * TH;
     lbm::pdl_wait_();   // (no __restrict__: nothing may be read before the wait)
+    auto stage = [&](int k) {   // channels k CCH .. of the input and their weights, one copy group
+        const int c0 = k * CCH, nc = CI - c0 < CCH ? CI - c0 : CCH;
+        for (int e = threadIdx.x; e < nc * 9 * CO / 4; e += NT)
+            copy_async16(s_w[k % STAGES] + 4 * e, wgt + c0 * 9 * CO + 4 * e, true);
+        stage_planes<NT, TWQ * 4, TH + 2, PW, PLANE>(x + ((long long)b * CI + c0) * H * W, nc, h0, w0, H, W,
+                                                     s_x[k % STAGES], vec_in);
+        copy_commit();
+    };
+    stage(0);
     float2 acc[4][COG / 2];
 #pragma unroll
     for (int j = 0; j < COG / 2; ++j) {
@@ -141,65 +170,98 @@ conv3x3(const In *x, const float *wgt, const float *bias, const A *zin, Out *y, 
 #pragma unroll
         for (int p = 0; p < 4; ++p) acc[p][j] = v;
     }
-    for (int c0 = 0; c0 < CI; c0 += CCH) {
-        const int nc = CI - c0 < CCH ? CI - c0 : CCH;
-        if (c0) __syncthreads();
-        stage_words<NT>(wgt + c0 * 9 * CO, nc * 9 * CO / 4, s_w);
-        stage_planes<NT, TWQ * 4, TH + 2, PW, PLANE, (TWQ > 4 ? 10 : 5)>(
-            x + ((long long)b * CI + c0) * H * W, nc, h0, w0, H, W, s_x, [](In v) {
-                const float u = BWD ? to_f(v) : load_as<A>(v);
-                return ACT ? silu(u) : u;
-            });
-        stage_wait();
-        __syncthreads();
-        if (!on) continue;
 #pragma unroll 1
-        for (int c = 0; c < nc; ++c) {
-            const float *xs = s_x + c * PLANE + row * PW + 4 * q;
-            float xv[3][6];
+    for (int k = 0; k < NCHUNK; ++k) {
+        if (k + 1 < NCHUNK) {
+            stage(k + 1);
+            copy_wait<1>();
+        } else {
+            copy_wait<0>();
+        }
+        __syncthreads();
+        const int nc = CI - k * CCH < CCH ? CI - k * CCH : CCH;
+        if (on)
+#pragma unroll 1
+            for (int c = 0; c < nc; ++c) {
+                const float *xs = s_x[k % STAGES] + c * PLANE + row * PW + 4 * q;
+                float xv[3][6];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const float4 u = *reinterpret_cast<const float4 *>(xs + i * PW);
-                const float2 v = *reinterpret_cast<const float2 *>(xs + i * PW + 4);
-                xv[i][0] = u.x, xv[i][1] = u.y, xv[i][2] = u.z, xv[i][3] = u.w, xv[i][4] = v.x, xv[i][5] = v.y;
-            }
-            const float *ws = s_w + c * 9 * CO + cg * COG;
+                for (int i = 0; i < 3; ++i) {
+                    const float4 u = *reinterpret_cast<const float4 *>(xs + i * PW + 4);
+                    xv[i][0] = xs[i * PW + 3], xv[i][1] = u.x, xv[i][2] = u.y, xv[i][3] = u.z, xv[i][4] = u.w;
+                    xv[i][5] = xs[i * PW + 8];
+                }
+                const float *ws = s_w[k % STAGES] + c * 9 * CO + cg * COG;
 #pragma unroll
-            for (int j = 0; j < COG / 2; j += 2) {
-                float2 sa[4], sb[4];
+                for (int j = 0; j < COG / 2; j += 2) {
+                    float2 sa[4], sb[4];
 #pragma unroll
-                for (int p = 0; p < 4; ++p) sa[p] = sb[p] = f2(0.f, 0.f);
+                    for (int p = 0; p < 4; ++p) sa[p] = sb[p] = f2(0.f, 0.f);
 #pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float4 u = *reinterpret_cast<const float4 *>(ws + k * CO + 2 * j);
+                    for (int t = 0; t < 9; ++t) {
+                        const float4 u = *reinterpret_cast<const float4 *>(ws + t * CO + 2 * j);
+#pragma unroll
+                        for (int p = 0; p < 4; ++p) {
+                            const float v = xv[t / 3][t % 3 + p];
+                            sa[p] = fma2(f2(u.x, u.y), f2(v, v), sa[p]);
+                            sb[p] = fma2(f2(u.z, u.w), f2(v, v), sb[p]);
+                        }
+                    }
 #pragma unroll
                     for (int p = 0; p < 4; ++p) {
-                        const float v = xv[k / 3][k % 3 + p];
-                        sa[p] = fma2(f2(u.x, u.y), f2(v, v), sa[p]);
-                        sb[p] = fma2(f2(u.z, u.w), f2(v, v), sb[p]);
+                        acc[p][j] = __fadd2_rn(acc[p][j], sa[p]);
+                        acc[p][j + 1] = __fadd2_rn(acc[p][j + 1], sb[p]);
                     }
                 }
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    acc[p][j] = __fadd2_rn(acc[p][j], sa[p]);
-                    acc[p][j + 1] = __fadd2_rn(acc[p][j + 1], sb[p]);
-                }
             }
-        }
+        if (k + 1 < NCHUNK) __syncthreads();   // the next round's copies go where this one read
     }
     lbm::pdl_launch_next_();
     const int ho = h0 + row, wo = w0 + 4 * q;
     if (!on || ho >= H) return;
+    const bool quad = W % 4 == 0;   // then the four pixels lie in the image together, aligned in the library's buffers
 #pragma unroll
     for (int j = 0; j < COG; ++j) {
         const long long o = (((long long)b * CO + cg * COG + j) * H + ho) * W + wo;
+        float v[4];
 #pragma unroll
-        for (int p = 0; p < 4; ++p)
-            if (wo + p < W) {
-                const float v = j & 1 ? acc[p][j / 2].y : acc[p][j / 2].x;
-                if constexpr (BWD) y[o + p] = v * dsilu(to_f(zin[o + p]));
-                else y[o + p] = store_as<A, Out>(v);
+        for (int p = 0; p < 4; ++p) v[p] = j & 1 ? acc[p][j / 2].y : acc[p][j / 2].x;
+        if constexpr (BWD) {
+            if (quad) {
+                if (wo < W) {
+                    __align__(8) A z[4];
+                    load4(zin + o, z);
+                    *reinterpret_cast<float4 *>(y + o) = make_float4(v[0] * dsilu(to_f(z[0])), v[1] * dsilu(to_f(z[1])),
+                                                                     v[2] * dsilu(to_f(z[2])), v[3] * dsilu(to_f(z[3])));
+                }
+            } else {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    if (wo + p < W) y[o + p] = v[p] * dsilu(to_f(zin[o + p]));
             }
+        } else if constexpr (LAST) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+                if (wo + p < W) {
+                    if constexpr (std::is_same<Out, A>::value) y[o + p] = from_f<A>(v[p]);
+                    else y[o + p] = rounded<A>(v[p]);
+                }
+        } else {   // the pre-activation as the activation type holds it, and silu of that
+            __align__(8) A z[4];
+            float s[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) z[p] = from_f<A>(v[p]), s[p] = silu(to_f(z[p]));
+            if (quad) {
+                if (wo < W) {
+                    store4(y + o, z);
+                    *reinterpret_cast<float4 *>(act + o) = make_float4(s[0], s[1], s[2], s[3]);
+                }
+            } else {
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    if (wo + p < W) y[o + p] = z[p], act[o + p] = s[p];
+            }
+        }
     }
 }
 
@@ -210,17 +272,18 @@ conv3x3(const In *x, const float *wgt, const float *bias, const A *zin, Out *y, 
 // 16-byte shared loads (the inputs by lane, the dz by broadcast).  A CTA walks over tiles of 8 x 32
 // pixels: the sums of a tile (128 terms each) are added to the CTA's, so no chain is longer than before
 // (256), and only gridDim partial sums reach memory (before: one per 16 x 16 tile, reduced by one
-// strided thread per result, 154 us a layer).  158 us a 32 -> 32 layer, 718 us with one FMA per two
+// strided thread per result, 154 us a layer).  140 us a 32 -> 32 layer, 718 us with one FMA per two
 // shared loads.
 constexpr int GW = 32, GH = 8, GT = 256;
-constexpr int GP = GW + 4, GPLANE = (GH + 2) * GP + 4;   // plane stride = 4 x odd words: no bank conflicts
+constexpr int GP = GW + 8, GPLANE = (GH + 2) * GP + 4;   // plane stride = 4 x odd words: no bank conflicts
 static_assert(GPLANE % 32 % 8 == 4, "16-byte loads of 8 lanes must hit distinct banks");
 constexpr int GD = GH * GW;
 template <int CI, int CO> constexpr int grad_groups() { return GT / (CI * CO / 4) < GH ? GT / (CI * CO / 4) : GH; }
 template <int CI, int CO> constexpr size_t grad_smem() { return (CI * GPLANE + CO * GD) * sizeof(float); }
 
-template <int CI, int CO, bool ACT, typename In, typename A>
-__global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz, float *part, int H, int W, int B)
+template <int CI, int CO>
+__global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *dz, float *part, int H, int W, int B,
+                                                   bool vec_in)
 {
     constexpr int NG = grad_groups<CI, CO>(), PER = CI * CO / 4, NW = CO * CI * 9;
     constexpr int BL = GT / CO;   // threads per bias sum
@@ -238,19 +301,23 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz,
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int b = tile / (tw * th), r0 = tile - b * (tw * th), h0 = r0 / tw * GH, w0 = r0 % tw * GW;
         __syncthreads();
-        stage_planes<GT, GW, GH + 2, GP, GPLANE, 10>(x + (long long)b * CI * H * W, CI, h0, w0, H, W, s_a, [](In v) {
-            const float u = load_as<A>(v);
-            return ACT ? silu(u) : u;
-        });
-        for (int e = t; e < CO * GD; e += GT) {   // dz, zero outside: element-wise asynchronous copies
-            const int c = e / GD, r = e - c * GD, hh = h0 + r / GW, ww = w0 + r % GW;
-            const bool in = hh < H && ww < W;
-            const float *src = dz + (((long long)b * CO + c) * H + (in ? hh : 0)) * W + (in ? ww : 0);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(s_d + e)),
-                         "l"(src), "r"(in ? 4 : 0)
-                         : "memory");
+        stage_planes<GT, GW, GH + 2, GP, GPLANE>(x + (long long)b * CI * H * W, CI, h0, w0, H, W, s_a, vec_in);
+        const float *dzb = dz + (long long)b * CO * H * W;   // dz: zero outside
+        if (W % 4 == 0) {
+            for (int e = t; e < CO * GD / 4; e += GT) {
+                const int c = e / (GD / 4), r = e - c * (GD / 4), hh = h0 + r / (GW / 4), ww = w0 + r % (GW / 4) * 4;
+                const bool in = hh < H && ww < W;
+                copy_async16(s_d + 4 * e, dzb + ((long long)c * H + (in ? hh : 0)) * W + (in ? ww : 0), in);
+            }
+        } else {
+            for (int e = t; e < CO * GD; e += GT) {
+                const int c = e / GD, r = e - c * GD, hh = h0 + r / GW, ww = w0 + r % GW;
+                const bool in = hh < H && ww < W;
+                copy_async4(s_d + e, dzb + ((long long)c * H + (in ? hh : 0)) * W + (in ? ww : 0), in);
+            }
         }
-        stage_wait();
+        copy_commit();
+        copy_wait<0>();
         __syncthreads();
         {
             float s = 0.f;   // the thread's share of a bias sum: columns t % BL, + BL, ..
@@ -267,9 +334,13 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz,
 #pragma unroll 1
         for (int y = grp; y < GH; y += NG) {
             const float *as = s_a + ci * GPLANE + y * GP, *ds = s_d + 4 * cog * GD + y * GW;
-            float4 cur[3];
+            float4 cur[3];      // columns c .. c + 3 of the image rows y - 1 .. y + 1, and the one before
+            float before[3];
 #pragma unroll
-            for (int i = 0; i < 3; ++i) cur[i] = *reinterpret_cast<const float4 *>(as + i * GP);
+            for (int i = 0; i < 3; ++i) {
+                before[i] = as[i * GP + 3];
+                cur[i] = *reinterpret_cast<const float4 *>(as + i * GP + 4);
+            }
 #pragma unroll 2
             for (int c = 0; c < GW; c += 4) {
                 float4 d[4];
@@ -277,9 +348,10 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz,
                 for (int i = 0; i < 4; ++i) d[i] = *reinterpret_cast<const float4 *>(ds + i * GD + c);
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
-                    const float4 u = cur[i], n = *reinterpret_cast<const float4 *>(as + i * GP + c + 4);
-                    const float2 p0[3] = {f2(u.x, u.y), f2(u.y, u.z), f2(u.z, u.w)};
-                    const float2 p1[3] = {f2(u.z, u.w), f2(u.w, n.x), f2(n.x, n.y)};
+                    const float4 u = cur[i], n = *reinterpret_cast<const float4 *>(as + i * GP + c + 8);
+                    const float2 m = f2(u.y, u.z);
+                    const float2 p0[3] = {f2(before[i], u.x), f2(u.x, u.y), m};
+                    const float2 p1[3] = {m, f2(u.z, u.w), f2(u.w, n.x)};
 #pragma unroll
                     for (int o = 0; o < 4; ++o)
 #pragma unroll
@@ -287,6 +359,7 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const In *x, const float *dz,
                             acc[o][3 * i + k] = fma2(p0[k], f2(d[o].x, d[o].y), acc[o][3 * i + k]);
                             acc[o][3 * i + k] = fma2(p1[k], f2(d[o].z, d[o].w), acc[o][3 * i + k]);
                         }
+                    before[i] = u.w;
                     cur[i] = n;
                 }
             }
@@ -348,6 +421,13 @@ __global__ void mse_grad(const A *__restrict__ y, const float *__restrict__ t, l
         __syncthreads();
     }
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+}
+
+// The input as the activation type holds it, in float (what the convolutions read).
+template <typename A> __global__ void round_input(const float *__restrict__ x, float *__restrict__ y, long long n)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        y[i] = rounded<A>(x[i]);
 }
 
 // Where parameter i = weight [co][ci][k] of its layer goes in the two layouts the convolutions read;
@@ -433,7 +513,8 @@ struct lbm_cnn {
     Layers L;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;   // params, grads, Adam state
     float *pf = nullptr, *pb = nullptr;   // the weights as the convolutions read them (weight_place)
-    void *act[NL + 1] = {nullptr};    // act[l+1] = pre-activation output of layer l (act[0]: the caller's input)
+    void *z[NL + 1] = {nullptr};      // z[l+1] = pre-activation output of layer l, in the activation type
+    float *in[NL] = {nullptr};        // what layer l reads, in float: the rounded input (BF16), silu(z[l])
     float *dz[2] = {nullptr, nullptr};
     float *part = nullptr;            // partial weight gradients
     double *loss_part = nullptr, *loss_host = nullptr;
@@ -441,6 +522,9 @@ struct lbm_cnn {
 };
 
 static thread_local char g_cnn_err[160] = "";
+
+// Whether rows of W floats at x can be copied 16 bytes at a time.
+static bool aligned_rows(const void *x, int W) { return W % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0; }
 
 template <typename K, typename... Args>
 static cudaError_t go(lbm_cnn *c, K kernel, dim3 grid, int block, size_t smem, Args... args)
@@ -451,30 +535,39 @@ static cudaError_t go(lbm_cnn *c, K kernel, dim3 grid, int block, size_t smem, A
 
 // One convolution.  Tiles of 32 x 8 pixels (16 channels a thread) where they fill the GPU, else of
 // 16 x 8 (8 channels a thread: half the pixels per CTA, 1.25 times the time per pixel).
-template <int CI, int CO, bool BWD, bool ACT, typename In, typename A, typename Out>
-static cudaError_t conv(lbm_cnn *c, int B, const In *x, const float *w, const float *bias, const A *zin, Out *y)
+template <int CI, int CO, bool BWD, bool LAST, typename A, typename Out>
+static cudaError_t conv(lbm_cnn *c, int B, const float *x, const float *w, const float *bias, const A *zin, Out *y, float *act)
 {
     using Big = Tile<CO, CO < 16 ? CO : 16, 8, 8>;
     using Small = Tile<CO, CO < 8 ? CO : 8, 4, 8>;
-    const dim3 gb((c->W + 31) / 32, (c->H + 7) / 8, B), gs((c->W + 15) / 16, (c->H + 7) / 8, B);
-    const long long nb = (long long)gb.x * gb.y * gb.z, ns = (long long)gs.x * gs.y * gs.z;
+    const int rows = (c->H + 7) / 8;
+    const dim3 gb((unsigned)((c->W + 31) / 32) * rows, 1, B), gs((unsigned)((c->W + 15) / 16) * rows, 1, B);
+    const long long nb = (long long)gb.x * B, ns = (long long)gs.x * B;
     const double tb = 2.0 * ((nb + 4 * c->sms - 1) / (4 * c->sms)), ts = 1.25 * ((ns + 4 * c->sms - 1) / (4 * c->sms));
+    const bool vec = aligned_rows(x, c->W);
     if (tb <= ts)
-        return go(c, conv3x3<CI, CO, Big, BWD, ACT, In, A, Out>, gb, Big::NT, 0, x, w, bias, zin, y, c->H, c->W);
-    return go(c, conv3x3<CI, CO, Small, BWD, ACT, In, A, Out>, gs, Small::NT, 0, x, w, bias, zin, y, c->H, c->W);
+        return go(c, conv3x3<CI, CO, Big, BWD, LAST, A, Out>, gb, Big::NT, 0, x, w, bias, zin, y, act, c->H, c->W, vec);
+    return go(c, conv3x3<CI, CO, Small, BWD, LAST, A, Out>, gs, Small::NT, 0, x, w, bias, zin, y, act, c->H, c->W, vec);
 }
+
+// What the first layer reads: the caller's input, or a copy rounded to the activation type.
+static const float *first_input(const lbm_cnn *c, const float *x) { return c->bf16 ? c->in[0] : x; }
 
 // Forward pass; the last layer's output goes to y (its activation type, or float).
 template <typename A, typename Out> static cudaError_t cnn_forward_impl(lbm_cnn *c, const float *x, int B, Out *y)
 {
     const A *none = nullptr;
+    float *no_act = nullptr;
     const float *w = c->pf, *p = c->p;
     const int *ow = c->L.off_w, *ob = c->L.off_b;
-    cudaError_t e = conv<CH[0], 32, false, false>(c, B, x, w + ow[0], p + ob[0], none, (A *)c->act[1]);
-    for (int l = 1; l < NL - 1 && e == cudaSuccess; ++l)
-        e = conv<32, 32, false, true>(c, B, (const A *)c->act[l], w + ow[l], p + ob[l], none, (A *)c->act[l + 1]);
+    if (c->bf16) round_input<A><<<1024, 256, 0, c->stream>>>(x, c->in[0], (long long)B * CH[0] * c->H * c->W);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = conv<32, 4, false, true>(c, B, (const A *)c->act[NL - 1], w + ow[NL - 1], p + ob[NL - 1], none, y);
+        e = conv<CH[0], 32, false, false>(c, B, first_input(c, x), w + ow[0], p + ob[0], none, (A *)c->z[1], c->in[1]);
+    for (int l = 1; l < NL - 1 && e == cudaSuccess; ++l)
+        e = conv<32, 32, false, false>(c, B, (const float *)c->in[l], w + ow[l], p + ob[l], none, (A *)c->z[l + 1], c->in[l + 1]);
+    if (e == cudaSuccess)
+        e = conv<32, 4, false, true>(c, B, (const float *)c->in[NL - 1], w + ow[NL - 1], p + ob[NL - 1], none, y, no_act);
     return e;
 }
 
@@ -485,15 +578,15 @@ static int grad_ctas(const lbm_cnn *c, int B)
     return (int)(tiles < 2 * c->sms ? tiles : 2 * c->sms);
 }
 
-template <int CI, int CO, bool ACT, typename In, typename A>
-static cudaError_t conv_gradient(lbm_cnn *c, int l, int B, const In *x, const float *dz)
+template <int CI, int CO> static cudaError_t conv_gradient(lbm_cnn *c, int l, int B, const float *x, const float *dz)
 {
     constexpr size_t sm = grad_smem<CI, CO>();
-    auto *kernel = conv_grad<CI, CO, ACT, In, A>;
+    auto *kernel = conv_grad<CI, CO>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const int ctas = grad_ctas(c, B);
     if (e == cudaSuccess)
-        e = go(c, kernel, dim3(ctas), GT, sm, x, dz, c->part + (size_t)ctas * c->L.off_w[l], c->H, c->W, B);
+        e = go(c, kernel, dim3(ctas), GT, sm, x, dz, c->part + (size_t)ctas * c->L.off_w[l], c->H, c->W, B,
+               aligned_rows(x, c->W));
     return e;
 }
 
@@ -502,21 +595,23 @@ static cudaError_t cnn_backward_impl(lbm_cnn *c, const float *x, int B, const fl
 {
     const long long nout = (long long)B * CH[NL] * c->H * c->W;
     const int lb = 512;
-    mse_grad<A><<<lb, 256, 0, c->stream>>>((const A *)c->act[NL], target, nout, c->dz[0], c->loss_part);
+    mse_grad<A><<<lb, 256, 0, c->stream>>>((const A *)c->z[NL], target, nout, c->dz[0], c->loss_part);
     cudaError_t e = cudaGetLastError();
     const float *w = c->pb, *none = nullptr;
     const int *ow = c->L.off_w;
-    const A *in = (const A *)c->act[NL - 1];
-    if (e == cudaSuccess) e = conv_gradient<32, 4, true, A, A>(c, NL - 1, B, in, c->dz[0]);
-    if (e == cudaSuccess) e = conv<4, 32, true, false>(c, B, (const float *)c->dz[0], w + ow[NL - 1], none, in, c->dz[1]);
+    float *no_act = nullptr;
+    if (e == cudaSuccess) e = conv_gradient<32, 4>(c, NL - 1, B, c->in[NL - 1], c->dz[0]);
+    if (e == cudaSuccess)
+        e = conv<4, 32, true, false>(c, B, (const float *)c->dz[0], w + ow[NL - 1], none, (const A *)c->z[NL - 1], c->dz[1],
+                                     no_act);
     int cur = 1;
     for (int l = NL - 2; l > 0 && e == cudaSuccess; --l, cur = 1 - cur) {
-        in = (const A *)c->act[l];
-        e = conv_gradient<32, 32, true, A, A>(c, l, B, in, c->dz[cur]);
+        e = conv_gradient<32, 32>(c, l, B, c->in[l], c->dz[cur]);
         if (e == cudaSuccess)
-            e = conv<32, 32, true, false>(c, B, (const float *)c->dz[cur], w + ow[l], none, in, c->dz[1 - cur]);
+            e = conv<32, 32, true, false>(c, B, (const float *)c->dz[cur], w + ow[l], none, (const A *)c->z[l],
+                                          c->dz[1 - cur], no_act);
     }
-    if (e == cudaSuccess) e = conv_gradient<CH[0], 32, false, float, A>(c, 0, B, x, c->dz[cur]);
+    if (e == cudaSuccess) e = conv_gradient<CH[0], 32>(c, 0, B, first_input(c, x), c->dz[cur]);
     if (e == cudaSuccess)
         e = go(c, reduce_parts, dim3((c->n_params + 31) / 32), 256, 0, (const float *)c->part, grad_ctas(c, B), c->L, c->g);
     if (e != cudaSuccess) return e;
@@ -552,7 +647,9 @@ void lbm_cnn_destroy(lbm_cnn *c)
     for (float *f : fs)
         if (f) cudaFree(f);
     for (int l = 0; l <= NL; ++l)
-        if (c->act[l]) cudaFree(c->act[l]);
+        if (c->z[l]) cudaFree(c->z[l]);
+    for (float *f : c->in)
+        if (f) cudaFree(f);
     if (c->loss_part) cudaFree(c->loss_part);
     if (c->loss_host) cudaFreeHost(c->loss_host);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -587,7 +684,9 @@ int lbm_cnn_create(int32_t H, int32_t W, int32_t batch_max, int32_t bf16_activat
     const long long plane = (long long)H * W;
     bool ok = true;
     for (float **f : {&c->p, &c->pf, &c->pb, &c->g, &c->m, &c->v}) ok = ok && cudaMalloc((void **)f, off * sizeof(float)) == cudaSuccess;
-    for (int l = 1; l <= NL && ok; ++l) ok = cudaMalloc(&c->act[l], (size_t)batch_max * CH[l] * plane * asz) == cudaSuccess;
+    for (int l = 1; l <= NL && ok; ++l) ok = cudaMalloc(&c->z[l], (size_t)batch_max * CH[l] * plane * asz) == cudaSuccess;
+    for (int l = c->bf16 ? 0 : 1; l < NL && ok; ++l)
+        ok = cudaMalloc((void **)&c->in[l], (size_t)batch_max * CH[l] * plane * sizeof(float)) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k) ok = cudaMalloc((void **)&c->dz[k], (size_t)batch_max * 32 * plane * sizeof(float)) == cudaSuccess;
     int dev = 0;
     ok = ok && cudaGetDevice(&dev) == cudaSuccess &&
@@ -654,8 +753,8 @@ int lbm_cnn_forward(lbm_cnn *c, const float *x, int32_t B, float *y)
 int lbm_cnn_gradients(lbm_cnn *c, const float *x, const float *target, int32_t B, float *grad_host, double *loss)
 {
     if (!c || !x || !target || B < 1 || B > c->Bmax) return LBM_EINVAL;
-    cudaError_t e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, x, B, (__nv_bfloat16 *)c->act[NL])
-                            : cnn_forward_impl<float>(c, x, B, (float *)c->act[NL]);
+    cudaError_t e = c->bf16 ? cnn_forward_impl<__nv_bfloat16>(c, x, B, (__nv_bfloat16 *)c->z[NL])
+                            : cnn_forward_impl<float>(c, x, B, (float *)c->z[NL]);
     if (e == cudaSuccess)
         e = c->bf16 ? cnn_backward_impl<__nv_bfloat16>(c, x, B, target, loss)
                     : cnn_backward_impl<float>(c, x, B, target, loss);
