@@ -200,7 +200,10 @@ template <typename R, typename S, int QF, int QT> struct ShapesFn {
         if (e != cudaSuccess) return e;
         out->tile = choose_tile<R, S, QF, QT>(h->nx, ny_total, sms);
         out->march = StepShape{auto_segment<R, S, QF, QT>(h->nx, h->ny), 0, 0, sms};
-        out->automatic = h->nx * ny_total <= tile_nodes_max(h->prec) ? out->tile : out->march;
+        // (a grid has 65535 tile rows; a channel of more marches, in segments of some hundred rows)
+        const bool fits = (h->ny + out->tile.ty - 1) / out->tile.ty <= 65535;
+        if (!fits) out->tile = out->march;
+        out->automatic = fits && h->nx * ny_total <= tile_nodes_max(h->prec) ? out->tile : out->march;
         return cudaGetLastError();
     }
 };
@@ -887,7 +890,7 @@ int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows)
     cand[nc++] = h->shapes.march;
     const int fixed[] = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256};
     for (int f : fixed)
-        if (f < h->ny && f != h->shapes.march.rows && nc < 16) cand[nc++] = StepShape{f, 0, 0, 0};
+        if (f < h->ny && f != h->shapes.march.rows && (h->ny + f - 1) / f <= 65535 && nc < 16) cand[nc++] = StepShape{f, 0, 0, 0};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));

@@ -159,14 +159,12 @@ template <typename Real> __device__ __forceinline__ void let_next_start_late_()
 
 template <typename Real, typename Store, int QF, int QT>
 __global__ void __launch_bounds__(TileGeo<Real, Store>::NT, TileGeo<Real, Store, QF, QT>::CTAS)
-tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty, int gx)
+tile_kernel(const __grid_constant__ StepArgs<Real, Store> A, int tx, int ty)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     let_next_start_early_<Real>();
-    int bx = blockIdx.x, by = blockIdx.y;
-    if (gx) by = bx / gx, bx -= by * gx;   // more tile rows than a grid has in y
     pdl_wait_();
-    tile_body<Real, Store, QF, QT>(A, tx, ty, bx, by, smem);
+    tile_body<Real, Store, QF, QT>(A, tx, ty, blockIdx.x, blockIdx.y, smem);
     let_next_start_late_<Real>();
 }
 
@@ -199,9 +197,11 @@ tile_pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *ac
 {
     extern __shared__ __align__(16) unsigned char smem[];
     let_next_start_early_<Real>();
-    const int c = pack_case_(B, blockIdx.x), i = blockIdx.x - B.start[c], by = i / B.cols[c], bx = i - by * B.cols[c];
+    const int c = pack_case_(B, blockIdx.x);
+    const int on = active[c];   // (host copies set it between launches that follow one another)
+    const int i = blockIdx.x - B.start[c], by = i / B.cols[c], bx = i - by * B.cols[c];
     pdl_wait_();
-    if (active[c]) tile_body<Real, Store, QF, QT>(B.a[c], tx, ty, bx, by, smem);
+    if (on) tile_body<Real, Store, QF, QT>(B.a[c], tx, ty, bx, by, smem);
     let_next_start_late_<Real>();
 }
 
@@ -229,11 +229,10 @@ template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const StepShape &shape)
 {
     const int tx = shape.tx, ty = shape.ty, gx = (A.nx + tx - 1) / tx, gy = (A.ny + ty - 1) / ty;
-    const bool flat = gy > 65535;
-    PdlLaunch l(flat ? dim3((unsigned)gx * gy) : dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
+    PdlLaunch l(dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
                 tile_smem<Real>(tx, ty, (long long)gx * gy, shape.sms), s);
     allow_smem(tile_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
-    return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty, flat ? gx : 0);
+    return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty);
 }
 
 template <typename Real, typename Store, int QF, int QT>

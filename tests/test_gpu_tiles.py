@@ -33,13 +33,15 @@ def test_tiles_equal_marching_strips(precision, qf, qt, nx, ny):
 
 
 def test_more_tile_rows_than_a_grid_has():
-    """A channel of more than 65535 rows of tiles (their launch is one-dimensional)."""
+    """A channel of more than 65535 rows of tiles, the most a grid has: the rule takes the march."""
     from paper_2210_07501_gb300 import Lbm
     w = WL.channel(3, 524300, 524290.0, W=3.0, sigma1=-3e-4, heat_periods=1)
     got = []
     for rows in (0, 64):
         g = Lbm(w["domain"], w["params"], precision="fp32")
         g.lbm_set_segment(rows)
+        if rows == 0:
+            assert g.lbm_autotune(1) > 0
         g.lbm_step(3)
         got.append(g.lbm_fields())
         g.close()
