@@ -137,8 +137,8 @@ def ncu_traffic():
     try:
         with open(path) as f:
             d = json.load(f)
-        h = hashlib.sha256(open(os.path.join(csrc, "lbm_step.cu"), "rb").read() +
-                           open(os.path.join(csrc, "lbm_device.cuh"), "rb").read()).hexdigest()[:16]
+        h = hashlib.sha256(b"".join(open(os.path.join(csrc, n), "rb").read() for n in
+                                    ("lbm_step.cu", "lbm_node.cuh", "lbm_device.cuh"))).hexdigest()[:16]
         return d["dram_bytes_per_launch_full_size"] if d.get("source_sha256_16") == h else None
     except Exception:
         return None
@@ -307,7 +307,8 @@ def bench_gpu(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": ncu_traffic() if args.precision == PRECISION else None,
                      "bytes_per_node": bpn, "peak_source": peak_kind,
-                     "kernel": f"lbm::march_kernel<{KERNEL_TYPES[args.precision]},5,5,128> "
+                     "kernel": f"lbm::{'tile' if args.precision == 'fp16' and not args.segment else 'march'}_kernel"
+                               f"<{KERNEL_TYPES[args.precision]},5,5> "
                                "(+ reductions every 100 steps in the region)"},
         "e2e": e2e,
         "gpu_launches": gpu_launches,

@@ -498,8 +498,9 @@ __device__ __forceinline__ void collide_flow_(float *g, float rho, float dp, flo
 // counted in FP64 instructions.  Central moments relax to their equilibria and are shifted back by
 // F(-u); since most of them are replaced by their equilibria, the shifted result (raw moments of
 // the stored deviation) has a closed form in which every product of a velocity with a moment is
-// formed once.  Against relaxing the central moments and applying the full shift: ~300 instead of
-// 352 FP64 instructions a node (D2Q9 + D2Q5 + D2Q5, tile kernel), 201 -> 160 us a step at 1024 x 256,
+// formed once.  Against relaxing the central moments and applying the full shift: 273 FP64
+// instructions a node (DFMA + DADD + DMUL, tiles of 1024 x 256 with their halos; 365 in the marching
+// kernel before, which has fewer halo nodes), 201 -> 160 us a step at 1024 x 256,
 // 32 -> 25 us at 200 x 100 with three D2Q9 lattices.  (FP32 keeps the packed forms above: these gained
 // 3 % at 1024 x 256 and nothing at 8192 x 2048, and FP16 storage turns their other last bits into
 // whole units of its own.)  Every multiply-add is written out,
