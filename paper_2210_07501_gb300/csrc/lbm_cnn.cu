@@ -707,11 +707,8 @@ int lbm_cnn_create(int32_t H, int32_t W, int32_t batch_max, int32_t bf16_activat
             h[c->L.off_w[l] + i] = (float)((2.0 * u01 - 1.0) * a);
         }
     }
-    cudaError_t e = cudaMemcpy(c->p, h.data(), off * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(c->m, 0, off * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(c->v, 0, off * sizeof(float));
-    if (e == cudaSuccess) e = lay_out_weights(c);
-    if (e != cudaSuccess) { lbm_cnn_destroy(c); return LBM_ECUDA; }
+    const int rc = lbm_cnn_set_params(c, h.data());   // on the network's stream, like all that reads them
+    if (rc != LBM_OK) { lbm_cnn_destroy(c); return rc; }
     *out = c;
     return LBM_OK;
 }
