@@ -73,6 +73,15 @@ static int cuda_fail(cudaError_t e, const char *what)
         if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
     } while (0)
 
+// Host data to the device, on the stream whose kernels read it: a plain cudaMemcpy runs on the legacy
+// default stream, which orders nothing for a non-blocking one, and may return before pageable data
+// has reached the device.  Returns when the source may be changed.
+static cudaError_t upload(void *dst, const void *src, size_t bytes, cudaStream_t s)
+{
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+}
+
 template <typename Real> static Phys<Real> cast_phys(const Phys<double> &d)
 {
     Phys<Real> p;
@@ -388,17 +397,17 @@ static int build_phase_reference(lbm_handle *h)
     }
     cudaError_t e;
     if (h->rsize == 8) {
-        e = cudaMemcpy(h->rtab, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(h->rowx, rx.data(), rx.size() * sizeof(double), cudaMemcpyHostToDevice);
+        e = upload(h->rtab, tab.data(), tab.size() * sizeof(double), h->stream);
+        if (e == cudaSuccess) e = upload(h->rowx, rx.data(), rx.size() * sizeof(double), h->stream);
     } else {
         std::vector<float> tf(tab.size()), rf(rx.size());
         for (size_t i = 0; i < tab.size(); ++i) tf[i] = (float)tab[i];
         for (size_t i = 0; i < rx.size(); ++i) rf[i] = (float)rx[i];
-        e = cudaMemcpy(h->rtab, tf.data(), tf.size() * sizeof(float), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(h->rowx, rf.data(), rf.size() * sizeof(float), cudaMemcpyHostToDevice);
+        e = upload(h->rtab, tf.data(), tf.size() * sizeof(float), h->stream);
+        if (e == cudaSuccess) e = upload(h->rowx, rf.data(), rf.size() * sizeof(float), h->stream);
     }
-    if (e == cudaSuccess) e = cudaMemcpy(h->phi0, phi0.data(), ny * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(h->fref, r.data(), r.size() * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = upload(h->phi0, phi0.data(), ny * sizeof(double), h->stream);
+    if (e == cudaSuccess) e = upload(h->fref, r.data(), r.size() * sizeof(double), h->stream);
     return e == cudaSuccess ? LBM_OK : cuda_fail(e, "reference tables");
 }
 
@@ -543,16 +552,16 @@ int lbm_create(const lbm_domain *domain, const lbm_params *params, void *stream,
             }
         cudaError_t ce;
         if (h->rsize == 8) {
-            ce = cudaMemcpy(h->twall, tw, 3 * (size_t)h->nx * sizeof(double), cudaMemcpyHostToDevice);
+            ce = upload(h->twall, tw, 3 * (size_t)h->nx * sizeof(double), h->stream);
         } else {
             float *twf = (float *)malloc(3 * (size_t)h->nx * sizeof(float));
             if (!twf) { free(tw); free_all(h); delete h; return LBM_ENOMEM; }
             for (int i = 0; i < 3 * h->nx; ++i) twf[i] = (float)tw[i];
-            ce = cudaMemcpy(h->twall, twf, 3 * (size_t)h->nx * sizeof(float), cudaMemcpyHostToDevice);
+            ce = upload(h->twall, twf, 3 * (size_t)h->nx * sizeof(float), h->stream);
             free(twf);
         }
         free(tw);
-        if (ce != cudaSuccess) { free_all(h); delete h; return cuda_fail(ce, "cudaMemcpy(twall)"); }
+        if (ce != cudaSuccess) { free_all(h); delete h; return cuda_fail(ce, "upload(twall)"); }
     }
     rc = lbm_init_fields(h, nullptr, nullptr, nullptr, nullptr, nullptr);
     if (rc) {
@@ -989,7 +998,7 @@ template <typename R, typename S, int QF, int QT> struct BatchArgsFn {
                     cudaError_t e = cudaMalloc(&dst, sz * b->n);
                     if (e != cudaSuccess) return e;
                 }
-                cudaError_t e = cudaMemcpy(dst, a.data(), sz * b->n, cudaMemcpyHostToDevice);
+                cudaError_t e = upload(dst, a.data(), sz * b->n, b->stream);
                 if (e != cudaSuccess) return e;
             }
         return cudaSuccess;
@@ -1030,7 +1039,7 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
         cudaError_t e = cudaMalloc((void **)&b->d_ctas, t.size() * sizeof(int4));
         if (e != cudaSuccess) return e;
         b->n_ctas = (int)t.size();
-        return cudaMemcpy(b->d_ctas, t.data(), t.size() * sizeof(int4), cudaMemcpyHostToDevice);
+        return upload(b->d_ctas, t.data(), t.size() * sizeof(int4), b->stream);
     }
 };
 
@@ -1130,13 +1139,13 @@ int lbm_batch_create(int32_t n, const lbm_domain *domains, const lbm_params *par
               cudaMalloc((void **)&b->d_reduce, (size_t)n * sizeof(ReduceCase)) == cudaSuccess &&
               cudaMallocHost((void **)&b->h_results, (4 * (size_t)n + 1) * sizeof(double)) == cudaSuccess;
     if (!ok) { cudaGetLastError(); lbm_batch_destroy(b); return LBM_ENOMEM; }
-    cudaError_t e = cudaMemcpy(b->d_active, b->active.data(), n * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(b->d_results, 0, (4 * (size_t)n + 1) * sizeof(double));
+    cudaError_t e = upload(b->d_active, b->active.data(), n * sizeof(int), b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_results, 0, (4 * (size_t)n + 1) * sizeof(double), b->stream);
     std::vector<ReduceCase> rc_cases;
     for (const lbm_handle *h : b->h)
         rc_cases.push_back(ReduceCase{h->macro, h->uprev, h->partials, (long long)h->nx * h->ny});
     if (e == cudaSuccess)
-        e = cudaMemcpy(b->d_reduce, rc_cases.data(), n * sizeof(ReduceCase), cudaMemcpyHostToDevice);
+        e = upload(b->d_reduce, rc_cases.data(), n * sizeof(ReduceCase), b->stream);
     if (e == cudaSuccess) e = dispatch<BatchArgsFn>(b->h[0], b);
     // the shapes for as many rows of the widest channel as the batch has nodes; marching segments of
     // 32 rows until tuned
