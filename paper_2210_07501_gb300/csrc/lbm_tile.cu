@@ -10,6 +10,7 @@
 // lbm_node.cuh, so the results are the march's bit for bit.
 #include "lbm_internal.h"
 #include "lbm_node.cuh"
+#include "lbm_once.h"
 
 namespace lbm {
 
@@ -209,50 +210,59 @@ tile_pack_kernel(const __grid_constant__ BatchPack<Real, Store> B, const int *ac
 // most tiles, so no SM may take more than its share: the request is raised until only that many
 // CTAs fit (otherwise CTAs settle two to an SM while the launch before still holds others: 33 us
 // instead of 24 a step at 200 x 100 with 130 tiles on 152 SMs).
+constexpr int SM_SMEM_KIB = 228;                          // 1 KiB of it reserved per CTA
+constexpr size_t TILE_SMEM_MAX = SM_SMEM_KIB / 2 * 1024;   // the largest request: one tile per SM
 template <typename Real> static size_t tile_smem(int tx, int ty, long long tiles, int sms)
 {
     const size_t need = ((size_t)(ty + 4) * (tx + 4) + 4 * (size_t)(ty + 2) * (tx + 2)) * sizeof(Real);
     const long long share = (tiles + sms - 1) / sms;   // CTAs an SM has to take
     if (sizeof(Real) == 4 || share > 4) return need;
-    // 228 KiB per SM, 1 KiB of it reserved per CTA; one CTA may have 227 KiB
-    const size_t most = (size_t)(228 / (share + 1)) * 1024;   // share + 1 CTAs of more than this do not fit
+    const size_t most = (size_t)(SM_SMEM_KIB / (share + 1)) * 1024;   // share + 1 CTAs of more than this do not fit
     return need > most ? need : most;
 }
 
-// FP64 launches may ask for more than 48 KiB.
-template <typename K> static void allow_smem(K kernel, size_t bytes)
+// A launch of one of the tile kernels.  FP64 requests may exceed the 48 KiB that a kernel may ask for
+// untold: the limit goes to their maximum once per kernel and device, not to each launch's own
+// request (with two threads stepping channels of different size, one lowered it between the
+// other's setting and launch).
+template <auto kernel, typename Real, typename... Args>
+static cudaError_t launch_tiles(dim3 grid, const StepShape &shape, cudaStream_t s, Args... args)
 {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const int tx = shape.tx, ty = shape.ty;
+    PdlLaunch l(grid, dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty, (long long)grid.x * grid.y, shape.sms), s);
+    if constexpr (sizeof(Real) == 8) {
+        static OncePerDevice limit;
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess)
+            e = (cudaError_t)limit.run(dev, [] {
+                return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM_MAX);
+            });
+        if (e != cudaSuccess) return e;
+    }
+    return cudaLaunchKernelEx(&l.cfg, kernel, args..., tx, ty);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const StepShape &shape)
 {
-    const int tx = shape.tx, ty = shape.ty, gx = (A.nx + tx - 1) / tx, gy = (A.ny + ty - 1) / ty;
-    PdlLaunch l(dim3(gx, gy), dim3((tx * ty + 31) / 32 * 32),
-                tile_smem<Real>(tx, ty, (long long)gx * gy, shape.sms), s);
-    allow_smem(tile_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
-    return cudaLaunchKernelEx(&l.cfg, tile_kernel<Real, Store, QF, QT>, A, tx, ty);
+    const dim3 grid((A.nx + shape.tx - 1) / shape.tx, (A.ny + shape.ty - 1) / shape.ty);
+    return launch_tiles<tile_kernel<Real, Store, QF, QT>, Real, const StepArgs<Real, Store> &>(grid, shape, s, A);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active,
                               const StepShape &shape, cudaStream_t s)
 {
-    const int tx = shape.tx, ty = shape.ty;
-    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty, n_ctas, shape.sms), s);
-    allow_smem(tile_batch_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
-    return cudaLaunchKernelEx(&l.cfg, tile_batch_kernel<Real, Store, QF, QT>, cases, ctas, active, tx, ty);
+    return launch_tiles<tile_batch_kernel<Real, Store, QF, QT>, Real>(dim3(n_ctas), shape, s, cases, ctas, active);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, const StepShape &shape,
                              cudaStream_t s)
 {
-    const int tx = shape.tx, ty = shape.ty;
-    PdlLaunch l(dim3(n_ctas), dim3((tx * ty + 31) / 32 * 32), tile_smem<Real>(tx, ty, n_ctas, shape.sms), s);
-    allow_smem(tile_pack_kernel<Real, Store, QF, QT>, l.cfg.dynamicSmemBytes);
-    return cudaLaunchKernelEx(&l.cfg, tile_pack_kernel<Real, Store, QF, QT>, B, active, tx, ty);
+    return launch_tiles<tile_pack_kernel<Real, Store, QF, QT>, Real, const BatchPack<Real, Store> &>(dim3(n_ctas), shape, s,
+                                                                                                B, active);
 }
 
 // Tile shape.  FP32 arithmetic: 32 x 8.  FP64 is bound by the SM's one FP64 pipe (16 cycles a warp
