@@ -16,6 +16,7 @@
 
 #include "lbm_internal.h"
 #include "lbm_node.cuh"
+#include "lbm_once.h"
 
 namespace lbm {
 
@@ -502,42 +503,52 @@ int step_strip_width()
 }
 
 // Dynamic shared memory of the step kernels (the staging ring); the attribute that allows
-// it is set once per kernel instance, with the carveout at its shared-memory maximum.
-template <typename Real, typename Store, int QF, int QT>
-static int prepare_kernels()
+// it is set once per kernel instance and device, with the carveout at its shared-memory maximum.
+template <typename Real, typename Store, int QF, int QT> constexpr int march_smem()
+{
+    return StageGeo<Real, Store, QF, QT, march_width<Real>()>::DYN;
+}
+template <typename Real, typename Store, int QF, int QT> static cudaError_t prepare_kernels()
 {
     constexpr int TX = march_width<Real>();
-    constexpr int dyn = StageGeo<Real, Store, QF, QT, TX>::DYN;
-    static bool done = false;
-    if (!done) {
-        cudaFuncSetAttribute(march_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        cudaFuncSetAttribute(batch_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        cudaFuncSetAttribute(pack_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        cudaFuncSetAttribute(pack_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(march_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
-        cudaFuncSetAttribute(batch_kernel<Real, Store, QF, QT, TX>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             100);
-        done = true;
-    }
-    return dyn;
+    static OncePerDevice attributes;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)attributes.run(dev, [] {
+        auto set = [](auto *kernel) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       march_smem<Real, Store, QF, QT>());
+            return e == cudaSuccess ? cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) : e;
+        };
+        cudaError_t e = set(march_kernel<Real, Store, QF, QT, TX>);
+        if (e == cudaSuccess) e = set(batch_kernel<Real, Store, QF, QT, TX>);
+        if (e == cudaSuccess) e = set(pack_kernel<Real, Store, QF, QT, TX>);
+        return (int)e;
+    });
+}
+template <typename Real, typename Store, int QF, int QT, typename... Params, typename... Args>
+static cudaError_t launch_strips(void (*kernel)(Params...), dim3 grid, cudaStream_t s, const Args &...args)
+{
+    const cudaError_t e = prepare_kernels<Real, Store, QF, QT>();
+    if (e != cudaSuccess) return e;
+    PdlLaunch l(grid, dim3(march_width<Real>() + 32), march_smem<Real, Store, QF, QT>(), s);
+    return cudaLaunchKernelEx(&l.cfg, kernel, args...);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_batch(const StepArgs<Real, Store> *cases, const int4 *ctas, int n_ctas, const int *active, int seg,
                          cudaStream_t s)
 {
-    constexpr int TX = march_width<Real>();
-    PdlLaunch l(dim3(n_ctas), dim3(TX + 32), prepare_kernels<Real, Store, QF, QT>(), s);
-    return cudaLaunchKernelEx(&l.cfg, batch_kernel<Real, Store, QF, QT, TX>, cases, ctas, active, seg);
+    return launch_strips<Real, Store, QF, QT>(batch_kernel<Real, Store, QF, QT, march_width<Real>()>, dim3(n_ctas), s, cases,
+                                              ctas, active, seg);
 }
 
 template <typename Real, typename Store, int QF, int QT>
 cudaError_t launch_march_pack(const BatchPack<Real, Store> &B, int n_ctas, const int *active, int seg, cudaStream_t s)
 {
-    constexpr int TX = march_width<Real>();
-    PdlLaunch l(dim3(n_ctas), dim3(TX + 32), prepare_kernels<Real, Store, QF, QT>(), s);
-    return cudaLaunchKernelEx(&l.cfg, pack_kernel<Real, Store, QF, QT, TX>, B, active, seg);
+    return launch_strips<Real, Store, QF, QT>(pack_kernel<Real, Store, QF, QT, march_width<Real>()>, dim3(n_ctas), s, B,
+                                              active, seg);
 }
 
 // Segment length.  FP32 arithmetic, from the waves of resident CTAs and the rows per segment plus the
@@ -572,11 +583,12 @@ template <typename Real, typename Store, int QF, int QT>
 int auto_segment(int nx, int ny)
 {
     constexpr int TX = march_width<Real>();
-    const int dyn = prepare_kernels<Real, Store, QF, QT>();
+    if (prepare_kernels<Real, Store, QF, QT>() != cudaSuccess) return ny;   // (the launch returns the error)
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_kernel<Real, Store, QF, QT, TX>, TX + 32, dyn);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_kernel<Real, Store, QF, QT, TX>, TX + 32,
+                                                  march_smem<Real, Store, QF, QT>());
     return choose_segment((nx + TX - 1) / TX, ny, sms * (per_sm > 0 ? per_sm : 1), sizeof(Real) == 8);
 }
 
@@ -585,9 +597,8 @@ cudaError_t launch_march(const StepArgs<Real, Store> &A, cudaStream_t s, int row
 {
     constexpr int TX = march_width<Real>();
     const int seg = rows < A.ny ? rows : A.ny;
-    PdlLaunch l(dim3((A.nx + TX - 1) / TX, (A.ny + seg - 1) / seg), dim3(TX + 32),
-                prepare_kernels<Real, Store, QF, QT>(), s);
-    return cudaLaunchKernelEx(&l.cfg, march_kernel<Real, Store, QF, QT, TX>, A, seg);
+    return launch_strips<Real, Store, QF, QT>(march_kernel<Real, Store, QF, QT, TX>,
+                                              dim3((A.nx + TX - 1) / TX, (A.ny + seg - 1) / seg), s, A, seg);
 }
 
 #define LBM_INST(R, S, QF, QT)                                                                              \

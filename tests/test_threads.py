@@ -53,6 +53,14 @@ def test_set_up_once_on_every_device(tmp_path):
     assert subprocess.run([str(exe)], capture_output=True, text=True, timeout=60).stdout.strip() == "0"
 
 
+def test_kernel_attributes_are_set_once_on_every_device():
+    """Attributes hold on one device: a flag per process left the kernels of the second device without
+    their shared memory, and nothing ordered a second thread's launch after the settings."""
+    for name in ("lbm_step.cu", "lbm_tile.cu"):
+        code = open(os.path.join(ROOT, "paper_2210_07501_gb300", "csrc", name)).read()
+        assert "cudaFuncSetAttribute" in code and "OncePerDevice" in code and "static bool" not in code, name
+
+
 @pytest.mark.gpu
 def test_two_threads_step_channels_of_different_size():
     """FP64 tiles ask for shared memory by the channel's size.  Two handles of one lattice pair, each
