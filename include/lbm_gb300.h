@@ -65,7 +65,8 @@ typedef struct lbm_handle lbm_handle;
 
 /* Lattice and discretisation (Sec. 2.1, Sec. 4). */
 typedef struct {
-    int32_t nx, ny;        /* nodes; nx >= 3, ny >= 3, ny * (nx rounded up to 64) < 2^31 */
+    int32_t nx, ny;        /* nodes; nx >= 3, ny >= 3, ny * (nx rounded up to 64) < 2^29   */
+                           /* (LBM_FP64), 2^30 (LBM_FP32), 2^31 (LBM_FP16)                 */
     int32_t heat_periods;  /* cosine periods of the bottom-wall temperature along x (>= 0) */
     int32_t q_phi;         /* 5 or 9: phase-field lattice                                  */
     int32_t q_T;           /* 5 or 9: energy lattice                                       */

@@ -253,10 +253,12 @@ static int validate(const lbm_domain *d, const lbm_params *p)
 {
     if (!d || !p) return LBM_EINVAL;
     if (d->nx < 3 || d->ny < 3) return LBM_EINVAL;
-    // element offsets inside one population plane are 32-bit
-    if ((long long)d->ny * (((long long)d->nx + 63) / 64 * 64) >= (1LL << 31)) return LBM_EINVAL;
     if ((d->q_phi != 5 && d->q_phi != 9) || (d->q_T != 5 && d->q_T != 9)) return LBM_EINVAL;
     if (d->precision < LBM_FP64 || d->precision > LBM_FP16 || d->heat_periods < 0) return LBM_EINVAL;
+    // byte offsets inside one population plane are unsigned 32-bit (loads and stores of lbm_node.cuh),
+    // element offsets int: a larger plane would wrap onto itself
+    const long long plane = (long long)d->ny * (((long long)d->nx + 63) / 64 * 64);
+    if (plane * (long long)store_size(d->precision) >= (1LL << 32) || plane >= (1LL << 31)) return LBM_EINVAL;
     if (!(d->W > 0.0) || !(d->b > 0.0) || !(d->b < d->ny)) return LBM_EINVAL;
     if (!(p->tau_flow > 0.5) || !(p->tau_T > 0.5) || !(p->tau_phi > 0.5)) return LBM_EINVAL;
     if (!(p->visc_ratio > 0.0) || !(p->cond_ratio > 0.0) || !(p->rho_bottom > 0.0) || !(p->rho_top > 0.0))
