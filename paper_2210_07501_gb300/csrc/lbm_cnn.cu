@@ -63,6 +63,15 @@ __device__ __forceinline__ void store4(__nv_bfloat16 *p, const __nv_bfloat16 *v)
     const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
     *reinterpret_cast<uint2 *>(p) = make_uint2(w[0], w[1]);
 }
+// s + c + x -> s + c: x onto the sum s, the rounding error onto c (Knuth's two-sum: exact in s + c). total: the
+// sum rounded once; an infinite or overflowed s has no error to add.
+__device__ __forceinline__ void add_exact(float &s, float &c, float x)
+{
+    const float t = s + x, z = t - s;
+    c += (s - (t - z)) + (x - z);
+    s = t;
+}
+__device__ __forceinline__ float total(float s, float c) { return isfinite(s) ? s + c : s; }
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
@@ -268,20 +277,25 @@ conv3x3(const float *x, const float *wgt, const float *bias, const A *zin, Out *
 // ---- weight and bias gradients -------------------------------------------------------------
 // dw[co][ci][k] = sum_p a[ci][p + k] dz[co][p], db[co] = sum_p dz[co][p], over all pixels.  A contraction
 // over the pixels with 32 x 288 results: a thread holds 4 output channels x 1 input channel x 9 taps, each as
-// the packed sums of its even and odd columns (72 registers); per four pixels 72 packed FMAs on 3 + 4
+// the packed sums of its even and odd columns (72 registers; with the operands 128, so the 36 sums
+// over the tiles are spilled and touched once a tile); per four pixels 72 packed FMAs on 3 + 4
 // 16-byte shared loads (the inputs by lane, the dz by broadcast).  A CTA walks over tiles of 8 x 32
-// pixels: the sums of a tile (128 terms each) are added to the CTA's, so no chain is longer than before
-// (256), and only gridDim partial sums reach memory (before: one per 16 x 16 tile, reduced by one
+// pixels, and only gridDim partial sums reach memory (before: one per 16 x 16 tile, reduced by one
 // strided thread per result, 154 us a layer).  140 us a 32 -> 32 layer, 718 us with one FMA per two
 // shared loads.
-constexpr int GW = 32, GH = 8, GT = 256;
+// Order of the sums: the two chains of 128 pixels of a tile, up to GRUN tiles in FP32 (so no FP32 chain is
+// longer than the 256 pixels of a 16 x 16 tile), and those runs, where a CTA has more tiles than one
+// (LONG), with their rounding errors carried along.  Carrying them tile by tile cost 4 % of a training
+// step at 16 x 256 x 64 (3 to 4 tiles a CTA), the code for it alone 1 %, hence the two instances;
+// without it the gradients of 16 x 512 x 512 images of constant dz were 4e-7 off.
+constexpr int GW = 32, GH = 8, GT = 256, GRUN = 4;
 constexpr int GP = GW + 8, GPLANE = (GH + 2) * GP + 4;   // plane stride = 4 x odd words: no bank conflicts
 static_assert(GPLANE % 32 % 8 == 4, "16-byte loads of 8 lanes must hit distinct banks");
 constexpr int GD = GH * GW;
 template <int CI, int CO> constexpr int grad_groups() { return GT / (CI * CO / 4) < GH ? GT / (CI * CO / 4) : GH; }
 template <int CI, int CO> constexpr size_t grad_smem() { return (CI * GPLANE + CO * GD) * sizeof(float); }
 
-template <int CI, int CO>
+template <int CI, int CO, bool LONG>
 __global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *dz, float *part, int H, int W, int B,
                                                    bool vec_in)
 {
@@ -291,7 +305,10 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *
     float *s_d = s_a + CI * GPLANE;
     const int t = threadIdx.x, ci = t % CI, cog = t / CI % (CO / 4), grp = t / PER;
     const bool on = grp < NG;
-    float tot[4][9], db = 0.f;
+    float tot[4][9], db = 0.f, db_err = 0.f;
+    float sum[LONG ? 36 : 1], err[LONG ? 36 : 1];   // LONG: the earlier runs' sums, once flushed
+    int n_run = 0;                                  // tiles in tot
+    bool flushed = false;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -323,7 +340,7 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *
             float s = 0.f;   // the thread's share of a bias sum: columns t % BL, + BL, ..
             const float *d = s_d + t / BL * GD;
             for (int p = t % BL; p < GD; p += BL) s += d[p];
-            db += s;
+            add_exact(db, db_err, s);
         }
         if (!on) continue;
         float2 acc[4][9];
@@ -368,7 +385,25 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int k = 0; k < 9; ++k) tot[i][k] += acc[i][k].x + acc[i][k].y;
+        if constexpr (LONG)
+            if (++n_run == GRUN && tile + gridDim.x < tiles) {
+#pragma unroll
+                for (int i = 0; i < 36; ++i) {
+                    if (!flushed) sum[i] = err[i] = 0.f;
+                    add_exact(sum[i], err[i], tot[i / 9][i % 9]);
+                    tot[i / 9][i % 9] = 0.f;
+                }
+                flushed = true;
+                n_run = 0;
+            }
     }
+    if constexpr (LONG)
+        if (flushed)
+#pragma unroll
+            for (int i = 0; i < 36; ++i) {
+                add_exact(sum[i], err[i], tot[i / 9][i % 9]);
+                tot[i / 9][i % 9] = total(sum[i], err[i]);
+            }
     lbm::pdl_launch_next_();
     // the pixel groups' sums onto the first group's, in sequence, through shared memory
     if constexpr (NG > 1) {
@@ -376,13 +411,18 @@ __global__ void __launch_bounds__(GT, 2) conv_grad(const float *x, const float *
         __syncthreads();
         if (on && grp > 0)
 #pragma unroll
-            for (int i = 0; i < 36; ++i) s_a[((grp - 1) * 36 + i) * PER + t % PER] = tot[i / 9][i % 9];
+            for (int i = 0; i < 36; ++i)
+                s_a[((grp - 1) * 36 + i) * PER + t % PER] = tot[i / 9][i % 9];
         __syncthreads();
         if (grp == 0)
-            for (int g = 0; g < NG - 1; ++g)
 #pragma unroll
-                for (int i = 0; i < 36; ++i) tot[i / 9][i % 9] += s_a[(g * 36 + i) * PER + t];
+            for (int i = 0; i < 36; ++i) {
+                float v = tot[i / 9][i % 9], e = 0.f;
+                for (int g = 0; g < NG - 1; ++g) add_exact(v, e, s_a[(g * 36 + i) * PER + t]);
+                tot[i / 9][i % 9] = total(v, e);
+            }
     }
+    db = total(db, db_err);
     float *out = part + (long long)blockIdx.x * (NW + CO);
     if (grp == 0)
 #pragma unroll
@@ -572,18 +612,19 @@ template <typename A, typename Out> static cudaError_t cnn_forward_impl(lbm_cnn 
 }
 
 // Two CTAs per SM walk over the tiles (fewer where there are fewer tiles).
+static long long grad_tiles(const lbm_cnn *c, int B) { return (long long)((c->W + GW - 1) / GW) * ((c->H + GH - 1) / GH) * B; }
 static int grad_ctas(const lbm_cnn *c, int B)
 {
-    const long long tiles = (long long)((c->W + GW - 1) / GW) * ((c->H + GH - 1) / GH) * B;
+    const long long tiles = grad_tiles(c, B);
     return (int)(tiles < 2 * c->sms ? tiles : 2 * c->sms);
 }
 
 template <int CI, int CO> static cudaError_t conv_gradient(lbm_cnn *c, int l, int B, const float *x, const float *dz)
 {
     constexpr size_t sm = grad_smem<CI, CO>();
-    auto *kernel = conv_grad<CI, CO>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const int ctas = grad_ctas(c, B);
+    auto *kernel = grad_tiles(c, B) > (long long)GRUN * ctas ? conv_grad<CI, CO, true> : conv_grad<CI, CO, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e == cudaSuccess)
         e = go(c, kernel, dim3(ctas), GT, sm, x, dz, c->part + (size_t)ctas * c->L.off_w[l], c->H, c->W, B,
                aligned_rows(x, c->W));

@@ -1,4 +1,6 @@
-"""The surrogate network beyond its accuracy at ordinary sizes: its state on creation."""
+"""The surrogate network beyond its accuracy at ordinary sizes: its state on creation, gradient sums over
+many pixels."""
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -30,3 +32,59 @@ def test_new_network_runs_on_the_parameters_it_reports(pkg, own_stream):
         torch.cuda.synchronize()
         assert float(y0.abs().max()) > 0 and torch.equal(y0, y1), seed
         net.close()
+
+
+CH = (12, 32, 32, 32, 32, 32, 4)
+
+
+def exact_network(pkg, B, H, W):
+    """A network (FP32 activations) whose gradients are known sums: the first layer's output is its
+    bias, 32 (silu(32) = 32 and silu'(32) = 1 in FP32); the identity, then channel sums less 256: outputs
+    zero.  With targets -d, every gradient is a sum of 2 d / (outputs) over pixels, times 32 in
+    the weights behind the first layer (32 -> 32 layers: between equal channels too)."""
+    net = pkg.Cnn(H, W, batch_max=B, bf16=False)
+    p = []
+    for l in range(6):
+        ci, co = CH[l], CH[l + 1]
+        w, b = np.zeros((co, ci, 3, 3), np.float32), np.zeros(co, np.float32)
+        if l == 0:
+            b[:] = 32.0
+        elif l < 5:
+            w[np.arange(co), np.arange(ci), 1, 1] = 1.0
+        else:
+            w[np.arange(ci) % co, np.arange(ci), 1, 1] = 1.0
+            b[:] = -256.0
+        p += [w.ravel(), b]
+    net.set_params(np.concatenate(p))
+    return net
+
+
+def layers_of(grad):
+    out, o = [], 0
+    for l in range(6):
+        n = CH[l] * CH[l + 1] * 9
+        out.append((grad[o:o + n].reshape(CH[l + 1], CH[l], 3, 3), grad[o + n:o + n + CH[l + 1]]))
+        o += n + CH[l + 1]
+    return out
+
+
+def test_weight_gradients_over_many_tiles(pkg):
+    """4.2 M pixels, 16384 tiles of the weight gradient, ~54 a CTA.  dz is one number whose sums over a tile are
+    exact in FP32, so what is measured is the sum over the tiles: as good as FP64's, rounded once per
+    CTA and once at the end (2^-24 each).  Summed in FP32 over a CTA's tiles it is 4e-7 off."""
+    B, H, W = 16, 512, 512
+    net = exact_network(pkg, B, H, W)
+    d = 5020203 / 2.0 ** 23
+    x = torch.ones((B, 12, H, W), device="cuda")
+    t = torch.full((B, 4, H, W), -d, device="cuda")
+    grad, _ = net.gradients(x, t)
+    net.close()
+    dz = 2.0 * d / (B * 4 * H * W)
+    full, edge = dz * B * H * W, dz * B * (H - 1) * W     # a tap in the row, in the row above or below
+    taps = np.array([edge, full, edge])[:, None] * np.ones((1, 3))
+    worst = 0.0
+    for l, (w, b) in enumerate(layers_of(grad.astype(np.float64))):
+        expect = taps * (1.0 if l == 0 else 32.0)
+        worst = max(worst, np.max(np.abs(w / expect - 1.0)), np.max(np.abs(b / full - 1.0)))
+    print(f"largest relative error of a gradient: {worst:.2e}")
+    assert worst <= 1.3e-7
