@@ -510,10 +510,15 @@ __global__ void __launch_bounds__(256) reduce_parts(const float *part, int n_par
             s = t;
         }
     }
-    sh[g][lane] = (double)s + (double)c;
+    double d = (double)s + (double)c;
+    if (!isfinite(s)) {   // infinite or overflowed: its rounding errors mean nothing
+        d = 0.0;
+        for (int p = g; p < n_part; p += 8) d += p0[(long long)p * n];
+    }
+    sh[g][lane] = d;
     __syncthreads();
     if (g == 0 && j < L.n) {
-        double d = sh[0][lane];
+        d = sh[0][lane];
         for (int i = 1; i < 8; ++i) d += sh[i][lane];
         grad[j] = (float)d;
     }

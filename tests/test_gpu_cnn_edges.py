@@ -1,5 +1,5 @@
 """The surrogate network beyond its accuracy at ordinary sizes: its state on creation, gradient sums over
-many pixels."""
+many pixels and of extreme values."""
 import numpy as np
 import pytest
 
@@ -37,10 +37,10 @@ def test_new_network_runs_on_the_parameters_it_reports(pkg, own_stream):
 CH = (12, 32, 32, 32, 32, 32, 4)
 
 
-def exact_network(pkg, B, H, W):
+def exact_network(pkg, B, H, W, z=32.0):
     """A network (FP32 activations) whose gradients are known sums: the first layer's output is its
-    bias, 32 (silu(32) = 32 and silu'(32) = 1 in FP32); the identity, then channel sums less 256: outputs
-    zero.  With targets -d, every gradient is a sum of 2 d / (outputs) over pixels, times 32 in
+    bias z >= 32 (silu(z) = z and silu'(z) = 1 in FP32); the identity, then channel sums less 8 z: outputs
+    zero.  With targets -d, every gradient is a sum of 2 d / (outputs) over pixels, times z in
     the weights behind the first layer (32 -> 32 layers: between equal channels too)."""
     net = pkg.Cnn(H, W, batch_max=B, bf16=False)
     p = []
@@ -48,12 +48,12 @@ def exact_network(pkg, B, H, W):
         ci, co = CH[l], CH[l + 1]
         w, b = np.zeros((co, ci, 3, 3), np.float32), np.zeros(co, np.float32)
         if l == 0:
-            b[:] = 32.0
+            b[:] = z
         elif l < 5:
             w[np.arange(co), np.arange(ci), 1, 1] = 1.0
         else:
             w[np.arange(ci) % co, np.arange(ci), 1, 1] = 1.0
-            b[:] = -256.0
+            b[:] = -8.0 * z
         p += [w.ravel(), b]
     net.set_params(np.concatenate(p))
     return net
@@ -88,3 +88,20 @@ def test_weight_gradients_over_many_tiles(pkg):
         worst = max(worst, np.max(np.abs(w / expect - 1.0)), np.max(np.abs(b / full - 1.0)))
     print(f"largest relative error of a gradient: {worst:.2e}")
     assert worst <= 1.3e-7
+
+
+def test_weight_gradients_of_extreme_values(pkg):
+    """An infinite dz makes the gradients it enters infinite and no others NaN; sums that overflow FP32 on the
+    way and not in the end (128 tiles, half of them +, half -) come out as in FP64: zero."""
+    H, W = 8, 32 * 128
+    net = exact_network(pkg, 1, H, W, z=128.0)
+    x = torch.ones((1, 12, H, W), device="cuda")
+    t = torch.zeros((1, 4, H, W), device="cuda")
+    t[0, 1, 3, 700] = -float("inf")
+    w, b = layers_of(net.gradients(x, t)[0])[5]
+    for a in (w, b):
+        assert np.all(np.isposinf(a[1])) and np.all(a[[0, 2, 3]] == 0.0)
+    t[:, :, :, : W // 2], t[:, :, :, W // 2:] = -1.7e38, 1.7e38
+    w, b = layers_of(net.gradients(x, t)[0])[5]
+    net.close()
+    assert np.all(w == 0.0) and np.all(b == 0.0)
