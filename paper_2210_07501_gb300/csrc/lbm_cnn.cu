@@ -78,7 +78,7 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // ---- 3x3 convolutions on the FP32 pipes ----------------------------------------------------
 // Forward (BWD = false): y[b][co][h][w] = bias[co] + sum_{ci, dy, dx} w[co][ci][dy][dx] a[b][ci][h+dy-1][w+dx-1].
 // Data gradient (BWD = true): the same sum over the layer's output channels with the kernel flipped, times
-// silu'(z) of the pixel.
+// silu'(z) of the pixel; silu(z) goes to act if given, for the weight gradient that follows.
 //
 // Bound: FP32 multiply-adds (2.4 G per 32 -> 32 layer at batch 16 of 256 x 64: 62 us at 80 TFLOP/s).  The
 // weights are kept in FP32 and the sums in FP32 in one order (per input channel the nine taps in
@@ -242,11 +242,18 @@ conv3x3(const float *x, const float *wgt, const float *bias, const A *zin, Out *
                     load4(zin + o, z);
                     *reinterpret_cast<float4 *>(y + o) = make_float4(v[0] * dsilu(to_f(z[0])), v[1] * dsilu(to_f(z[1])),
                                                                      v[2] * dsilu(to_f(z[2])), v[3] * dsilu(to_f(z[3])));
+                    if (act)
+                        *reinterpret_cast<float4 *>(act + o) =
+                            make_float4(silu(to_f(z[0])), silu(to_f(z[1])), silu(to_f(z[2])), silu(to_f(z[3])));
                 }
             } else {
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
-                    if (wo + p < W) y[o + p] = v[p] * dsilu(to_f(zin[o + p]));
+                    if (wo + p < W) {
+                        const float z = to_f(zin[o + p]);
+                        y[o + p] = v[p] * dsilu(z);
+                        if (act) act[o + p] = silu(z);
+                    }
             }
         } else if constexpr (LAST) {
 #pragma unroll
@@ -559,7 +566,11 @@ struct lbm_cnn {
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;   // params, grads, Adam state
     float *pf = nullptr, *pb = nullptr;   // the weights as the convolutions read them (weight_place)
     void *z[NL + 1] = {nullptr};      // z[l+1] = pre-activation output of layer l, in the activation type
-    float *in[NL] = {nullptr};        // what layer l reads, in float: the rounded input (BF16), silu(z[l])
+    // Of what the layers read, in float (the rounded input with BF16 activations, then silu(z[l])), only what
+    // is being read is held: forward, the layers' in the two dz, the input's in act; backward, the last two
+    // layers' where the forward pass left them, then act, formed again from z beside each data
+    // gradient.  (Kept for every layer they took 688 bytes a pixel, 1272 in all with BF16; now 712.)
+    float *act = nullptr;
     float *dz[2] = {nullptr, nullptr};
     float *part = nullptr;            // partial weight gradients
     double *loss_part = nullptr, *loss_host = nullptr;
@@ -595,8 +606,13 @@ static cudaError_t conv(lbm_cnn *c, int B, const float *x, const float *w, const
     return go(c, conv3x3<CI, CO, Small, BWD, LAST, A, Out>, gs, Small::NT, 0, x, w, bias, zin, y, act, c->H, c->W, vec);
 }
 
-// What the first layer reads: the caller's input, or a copy rounded to the activation type.
-static const float *first_input(const lbm_cnn *c, const float *x) { return c->bf16 ? c->in[0] : x; }
+// What the first layer reads: the caller's input, or a copy in act rounded to the activation type.
+template <typename A> static cudaError_t first_input(lbm_cnn *c, const float *x, int B, const float **in)
+{
+    *in = c->bf16 ? c->act : x;
+    if (c->bf16) round_input<A><<<1024, 256, 0, c->stream>>>(x, c->act, (long long)B * CH[0] * c->H * c->W);
+    return cudaGetLastError();
+}
 
 // Forward pass; the last layer's output goes to y (its activation type, or float).
 template <typename A, typename Out> static cudaError_t cnn_forward_impl(lbm_cnn *c, const float *x, int B, Out *y)
@@ -605,14 +621,14 @@ template <typename A, typename Out> static cudaError_t cnn_forward_impl(lbm_cnn 
     float *no_act = nullptr;
     const float *w = c->pf, *p = c->p;
     const int *ow = c->L.off_w, *ob = c->L.off_b;
-    if (c->bf16) round_input<A><<<1024, 256, 0, c->stream>>>(x, c->in[0], (long long)B * CH[0] * c->H * c->W);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = conv<CH[0], 32, false, false>(c, B, first_input(c, x), w + ow[0], p + ob[0], none, (A *)c->z[1], c->in[1]);
+    const float *in;
+    cudaError_t e = first_input<A>(c, x, B, &in);
+    if (e == cudaSuccess) e = conv<CH[0], 32, false, false>(c, B, in, w + ow[0], p + ob[0], none, (A *)c->z[1], c->dz[0]);
     for (int l = 1; l < NL - 1 && e == cudaSuccess; ++l)
-        e = conv<32, 32, false, false>(c, B, (const float *)c->in[l], w + ow[l], p + ob[l], none, (A *)c->z[l + 1], c->in[l + 1]);
+        e = conv<32, 32, false, false>(c, B, (const float *)c->dz[(l - 1) & 1], w + ow[l], p + ob[l], none, (A *)c->z[l + 1],
+                                       c->dz[l & 1]);
     if (e == cudaSuccess)
-        e = conv<32, 4, false, true>(c, B, (const float *)c->in[NL - 1], w + ow[NL - 1], p + ob[NL - 1], none, y, no_act);
+        e = conv<32, 4, false, true>(c, B, (const float *)c->dz[(NL - 2) & 1], w + ow[NL - 1], p + ob[NL - 1], none, y, no_act);
     return e;
 }
 
@@ -641,23 +657,27 @@ static cudaError_t cnn_backward_impl(lbm_cnn *c, const float *x, int B, const fl
 {
     const long long nout = (long long)B * CH[NL] * c->H * c->W;
     const int lb = 512;
-    mse_grad<A><<<lb, 256, 0, c->stream>>>((const A *)c->z[NL], target, nout, c->dz[0], c->loss_part);
+    mse_grad<A><<<lb, 256, 0, c->stream>>>((const A *)c->z[NL], target, nout, c->act, c->loss_part);
     cudaError_t e = cudaGetLastError();
-    const float *w = c->pb, *none = nullptr;
+    const float *w = c->pb, *none = nullptr, *in;
     const int *ow = c->L.off_w;
-    float *no_act = nullptr;
-    if (e == cudaSuccess) e = conv_gradient<32, 4>(c, NL - 1, B, c->in[NL - 1], c->dz[0]);
+    float *no_act = nullptr, *last = c->act;
+    // the inputs of the last two layers are in dz[0] and dz[1]
+    if (e == cudaSuccess) e = conv_gradient<32, 4>(c, NL - 1, B, c->dz[0], last);
     if (e == cudaSuccess)
-        e = conv<4, 32, true, false>(c, B, (const float *)c->dz[0], w + ow[NL - 1], none, (const A *)c->z[NL - 1], c->dz[1],
-                                     no_act);
+        e = conv<4, 32, true, false>(c, B, (const float *)last, w + ow[NL - 1], none, (const A *)c->z[NL - 1], c->dz[0], no_act);
+    if (e == cudaSuccess) e = conv_gradient<32, 32>(c, NL - 2, B, c->dz[1], c->dz[0]);
+    if (e == cudaSuccess)
+        e = conv<32, 32, true, false>(c, B, (const float *)c->dz[0], w + ow[NL - 2], none, (const A *)c->z[NL - 2], c->dz[1],
+                                      no_act);
     int cur = 1;
-    for (int l = NL - 2; l > 0 && e == cudaSuccess; --l, cur = 1 - cur) {
-        e = conv_gradient<32, 32>(c, l, B, c->in[l], c->dz[cur]);
-        if (e == cudaSuccess)
-            e = conv<32, 32, true, false>(c, B, (const float *)c->dz[cur], w + ow[l], none, (const A *)c->z[l],
-                                          c->dz[1 - cur], no_act);
+    for (int l = NL - 3; l > 0 && e == cudaSuccess; --l, cur = 1 - cur) {   // the data gradient first: it forms the input
+        e = conv<32, 32, true, false>(c, B, (const float *)c->dz[cur], w + ow[l], none, (const A *)c->z[l], c->dz[1 - cur],
+                                      c->act);
+        if (e == cudaSuccess) e = conv_gradient<32, 32>(c, l, B, c->act, c->dz[cur]);
     }
-    if (e == cudaSuccess) e = conv_gradient<CH[0], 32>(c, 0, B, first_input(c, x), c->dz[cur]);
+    if (e == cudaSuccess) e = first_input<A>(c, x, B, &in);
+    if (e == cudaSuccess) e = conv_gradient<CH[0], 32>(c, 0, B, in, c->dz[cur]);
     if (e == cudaSuccess)
         e = go(c, reduce_parts, dim3((c->n_params + 31) / 32), 256, 0, (const float *)c->part, grad_ctas(c, B), c->L, c->g);
     if (e != cudaSuccess) return e;
@@ -689,13 +709,11 @@ void lbm_cnn_destroy(lbm_cnn *c)
 {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    float *fs[] = {c->p, c->pf, c->pb, c->g, c->m, c->v, c->dz[0], c->dz[1], c->part};
+    float *fs[] = {c->p, c->pf, c->pb, c->g, c->m, c->v, c->dz[0], c->dz[1], c->act, c->part};
     for (float *f : fs)
         if (f) cudaFree(f);
     for (int l = 0; l <= NL; ++l)
         if (c->z[l]) cudaFree(c->z[l]);
-    for (float *f : c->in)
-        if (f) cudaFree(f);
     if (c->loss_part) cudaFree(c->loss_part);
     if (c->loss_host) cudaFreeHost(c->loss_host);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -731,8 +749,7 @@ int lbm_cnn_create(int32_t H, int32_t W, int32_t batch_max, int32_t bf16_activat
     bool ok = true;
     for (float **f : {&c->p, &c->pf, &c->pb, &c->g, &c->m, &c->v}) ok = ok && cudaMalloc((void **)f, off * sizeof(float)) == cudaSuccess;
     for (int l = 1; l <= NL && ok; ++l) ok = cudaMalloc(&c->z[l], (size_t)batch_max * CH[l] * plane * asz) == cudaSuccess;
-    for (int l = c->bf16 ? 0 : 1; l < NL && ok; ++l)
-        ok = cudaMalloc((void **)&c->in[l], (size_t)batch_max * CH[l] * plane * sizeof(float)) == cudaSuccess;
+    ok = ok && cudaMalloc((void **)&c->act, (size_t)batch_max * 32 * plane * sizeof(float)) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k) ok = cudaMalloc((void **)&c->dz[k], (size_t)batch_max * 32 * plane * sizeof(float)) == cudaSuccess;
     int dev = 0;
     ok = ok && cudaGetDevice(&dev) == cudaSuccess &&

@@ -1,5 +1,5 @@
-"""The surrogate network beyond its accuracy at ordinary sizes: its state on creation, gradient sums over
-many pixels and of extreme values."""
+"""The surrogate network beyond its accuracy at ordinary sizes: its state on creation, its memory, gradient
+sums over many pixels and of extreme values."""
 import numpy as np
 import pytest
 
@@ -32,6 +32,21 @@ def test_new_network_runs_on_the_parameters_it_reports(pkg, own_stream):
         torch.cuda.synchronize()
         assert float(y0.abs().max()) > 0 and torch.equal(y0, y1), seed
         net.close()
+
+
+@pytest.mark.parametrize("bf16,per_pixel", [(True, 752), (False, 1104)])
+def test_device_memory_per_pixel(pkg, bf16, per_pixel):
+    """What a network takes of the device grows by no more than 752 bytes a pixel with BF16 activations
+    (every layer's output once, two gradients and 144 bytes of partial sums: images and batches that
+    fit by that measure must keep fitting), 1104 with FP32's; and 64 MB whatever the size."""
+    torch.cuda.synchronize()
+    B, H, W = 8, 1024, 1024
+    free = torch.cuda.mem_get_info()[0]
+    net = pkg.Cnn(H, W, batch_max=B, bf16=bf16)
+    used = free - torch.cuda.mem_get_info()[0]
+    net.close()
+    print(f"{used / (B * H * W):.0f} bytes a pixel")
+    assert used <= per_pixel * B * H * W + (64 << 20)
 
 
 CH = (12, 32, 32, 32, 32, 32, 4)
