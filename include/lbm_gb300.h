@@ -150,9 +150,11 @@ int lbm_save(lbm_handle *h, const char *path);
 int lbm_load(lbm_handle *h, const char *path);
 
 /* Launch shape of the step (no counterpart in the paper): rows > 0: each CTA walks `rows`
- * consecutive rows of a 128-column strip; 0 = automatic: 2-D tiles on channels too small to
- * fill the GPU with strips, else strips with the length that minimises the waves of resident
- * CTAs times the rows each walks.  Affects speed only, never the results. */
+ * consecutive rows of a 128-column strip; LBM_SEGMENT_TILES: 2-D tiles (a channel of more than
+ * 65535 rows of tiles keeps strips); 0 = automatic: tiles on channels too small to fill the
+ * GPU with strips, else strips with the length that minimises the waves of resident CTAs times
+ * the rows each walks.  Affects speed only, never the results. */
+#define LBM_SEGMENT_TILES INT32_MAX
 int lbm_set_segment(lbm_handle *h, int32_t rows);
 
 /* Test hook for the fault path (not part of the method).  The step kernel stages its
@@ -167,10 +169,14 @@ int lbm_test_stall_copies(lbm_handle *h, int32_t on);
 
 /* Autotuner (no counterpart in the paper): times `reps` launches of the step for each
  * candidate shape (2-D tiles, strips with the automatic segment length, strips of 8 .. 256 rows
- * below ny) and keeps the fastest; *rows (may be NULL) receives the rows of its segments or
- * tiles.  The kernel is re-launched from the same input buffer, so the state and the step
- * count are unchanged.  Synchronises. */
+ * below ny) and keeps the fastest; *rows (may be NULL) receives what lbm_set_segment takes to
+ * choose it: the rows of its segments, or LBM_SEGMENT_TILES.  The kernel is re-launched from
+ * the same input buffer, so the state and the step count are unchanged.  Synchronises. */
 int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows);
+
+/* The launch shape in use (no counterpart in the paper): *cols = 0: strips, in segments of
+ * *rows rows; else tiles of *cols x *rows nodes.  Either pointer may be NULL. */
+int lbm_launch_shape(const lbm_handle *h, int32_t *cols, int32_t *rows);
 
 /* Bytes the step kernel moves per lattice node and step (populations read and written
  * once plus the stored pressure), for roofline accounting (no counterpart in the paper). */

@@ -21,6 +21,7 @@ from . import build as _build
 LBM_OK, LBM_EINVAL, LBM_ENOMEM, LBM_ECUDA, LBM_EUNSTABLE, LBM_ETIMEOUT, LBM_EIO, LBM_EDEVICE = 0, -1, -2, -3, -4, -5, -6, -7
 LBM_FP64, LBM_FP32, LBM_FP16 = 0, 1, 2
 LBM_DTYPE_F64, LBM_DTYPE_F32 = 0, 1
+LBM_SEGMENT_TILES = 2**31 - 1
 PRECISIONS = {"fp64": LBM_FP64, "fp32": LBM_FP32, "fp16": LBM_FP16}
 
 LIB_PATH = _build.LIB
@@ -69,6 +70,7 @@ SIGNATURES = {
     "lbm_set_segment": (ctypes.c_int, [_H, ctypes.c_int32]),
     "lbm_test_stall_copies": (ctypes.c_int, [_H, ctypes.c_int32]),
     "lbm_autotune": (ctypes.c_int, [_H, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
+    "lbm_launch_shape": (ctypes.c_int, [_H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "lbm_bytes_per_node": (ctypes.c_int, [_H, _I64P]),
     "lbm_launch_count": (ctypes.c_int, [_H, _I64P]),
     "lbm_reduce_fields_noalloc": (ctypes.c_int, [ctypes.c_void_p] * 6 + [ctypes.c_int64, ctypes.c_void_p,
@@ -269,6 +271,11 @@ class Lbm:
         r = ctypes.c_int32()
         _check(self._lib.lbm_autotune(self._h, int(reps), ctypes.byref(r)), "lbm_autotune")
         return r.value
+
+    def lbm_launch_shape(self) -> dict:
+        c, r = ctypes.c_int32(), ctypes.c_int32()
+        _check(self._lib.lbm_launch_shape(self._h, ctypes.byref(c), ctypes.byref(r)), "lbm_launch_shape")
+        return {"kind": "tiles" if c.value else "strips", "cols": c.value, "rows": r.value}
 
     def lbm_bytes_per_node(self) -> int:
         b = ctypes.c_int64()

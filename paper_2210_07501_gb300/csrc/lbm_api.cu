@@ -879,7 +879,8 @@ int lbm_load(lbm_handle *h, const char *path)
 int lbm_set_segment(lbm_handle *h, int32_t rows)
 {
     if (!h || rows < 0) return LBM_EINVAL;
-    h->shape = rows > 0 ? StepShape{rows, 0, 0, 0} : h->shapes.automatic;
+    if (rows == LBM_SEGMENT_TILES) h->shape = h->shapes.tile;
+    else h->shape = rows > 0 ? StepShape{rows, 0, 0, 0} : h->shapes.automatic;
     return LBM_OK;
 }
 
@@ -926,8 +927,16 @@ int lbm_autotune(lbm_handle *h, int32_t reps, int32_t *rows)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h->shape = rc == LBM_OK ? best : saved;
-    if (rows) *rows = h->shape.rows > 0 ? h->shape.rows : h->shape.ty;
+    if (rows) *rows = h->shape.rows > 0 ? h->shape.rows : LBM_SEGMENT_TILES;
     return rc;
+}
+
+int lbm_launch_shape(const lbm_handle *h, int32_t *cols, int32_t *rows)
+{
+    if (!h) return LBM_EINVAL;
+    if (cols) *cols = h->shape.rows > 0 ? 0 : h->shape.tx;
+    if (rows) *rows = h->shape.rows > 0 ? h->shape.rows : h->shape.ty;
+    return LBM_OK;
 }
 
 int lbm_bytes_per_node(const lbm_handle *h, int64_t *bytes)
