@@ -265,9 +265,9 @@ def bench_gpu(args):
         bpn = g.lbm_bytes_per_node()
         if args.segment:
             g.lbm_set_segment(args.segment)
-            seg_rows = args.segment
         else:
-            seg_rows = g.lbm_autotune(10)    # launch shape; leaves the state untouched
+            g.lbm_autotune(10)    # launch shape; leaves the state untouched
+        shape = g.lbm_launch_shape()
         # ---- device-resident throughput ----
         g.lbm_step(args.warmup)
         torch.cuda.synchronize()
@@ -302,12 +302,12 @@ def bench_gpu(args):
         "config": {"workload": WORKLOAD, "nx": nx, "ny": ny, "b": w["domain"]["b"], "W": w["domain"]["W"],
                    "lattices": "D2Q9 flow + D2Q5 phase field + D2Q5 energy", "storage": args.precision,
                    "check_interval": CHECK_INTERVAL, "l2": "working set 2.7 GB > L2 (no flush needed)",
-                   "segment_rows": seg_rows,
+                   "segment_rows": shape["rows"] if shape["kind"] == "strips" else None, "launch": shape,
                    "parallelism": f"replicas x{ws}"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": ncu_traffic() if args.precision == PRECISION else None,
                      "bytes_per_node": bpn, "peak_source": peak_kind,
-                     "kernel": f"lbm::{'tile' if args.precision == 'fp16' and not args.segment else 'march'}_kernel"
+                     "kernel": f"lbm::{'tile' if shape['kind'] == 'tiles' else 'march'}_kernel"
                                f"<{KERNEL_TYPES[args.precision]},5,5> "
                                "(+ reductions every 100 steps in the region)"},
         "e2e": e2e,

@@ -46,3 +46,23 @@ def test_rule(precision, nx, ny, kind):
         g.lbm_set_segment(LBM_SEGMENT_TILES)
         assert g.lbm_launch_shape()["kind"] == "strips"
     g.close()
+
+
+@pytest.mark.parametrize("args,kind", [(["--ny", "96"], None), (["--ny", "96", "--segment", "16"], "strips"),
+                                       (["--ny", "96", "--precision", "fp16", "--segment", "16"], "strips")])
+def test_bench_names_the_kernel_it_ran(args, kind):
+    """The line of the benchmark names the kernel and launch shape in use, as the library reports them
+    (kind None: whichever the autotuner took)."""
+    import json
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "bench.py", "--steps", "4", "--warmup", "3", "--no-e2e", "--no-cpu-baseline"] + args,
+                       cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    line = json.loads(r.stdout.strip().splitlines()[-1])
+    kind = kind or line["config"]["launch"]["kind"]
+    name = {"tiles": "lbm::tile_kernel", "strips": "lbm::march_kernel"}[kind]
+    assert line["config"]["launch"]["kind"] == kind and line["roofline"]["kernel"].startswith(name)
+    assert line["config"]["segment_rows"] == (line["config"]["launch"]["rows"] if kind == "strips" else None)
