@@ -342,7 +342,8 @@ def bench_sweep(args):
     t0 = time.perf_counter()
     b = pkg.LbmBatch(cases, precision="fp32")
     b.lbm_batch_set_check_interval(K)
-    rows = b.lbm_batch_autotune(5)
+    b.lbm_batch_autotune(5)
+    shape = b.lbm_batch_launch_shape()
     steps_b, conv_b = b.lbm_batch_run_to_steady(args.sweep_tol, args.sweep_max)
     t_batch = time.perf_counter() - t0
     size = b.lbm_batch_size()
@@ -366,7 +367,7 @@ def bench_sweep(args):
         "batched_s": t_batch, "per_case_s": t_single, "speedup": t_single / t_batch,
         "converged_batched": int(sum(conv_b)), "converged_per_case": int(sum(conv_s)),
         "same_steps": steps_b == steps_s, "batched_mlups": lu / t_batch / 1e6,
-        "batch_ctas": size["ctas"], "segment_rows": rows,
+        "batch_ctas": size["ctas"], "segment_rows": shape["rows"] if shape["kind"] == "strips" else None, "launch": shape,
         "steps": steps_b, "sites_total": sum(sites)}}
     print(json.dumps(line), flush=True)
     return 0

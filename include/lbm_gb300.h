@@ -232,9 +232,15 @@ int lbm_batch_create(int32_t n, const lbm_domain *domains, const lbm_params *par
 /* Steps per chunk and residual check (even, >= 2; default 100). */
 int lbm_batch_set_check_interval(lbm_batch *b, int32_t K);
 
+/* Launch shape of the batch, as lbm_set_segment and lbm_launch_shape for one channel (0: tiles
+ * while all channels together are too small to fill the GPU with strips, else strips in
+ * segments of 32 rows).  Affects speed only.  Setting it waits for the batch's work. */
+int lbm_batch_set_segment(lbm_batch *b, int32_t rows);
+int lbm_batch_launch_shape(const lbm_batch *b, int32_t *cols, int32_t *rows);
+
 /* Autotuner for the batch launch: times `reps` launches per candidate shape (tiles, segment
- * lengths) and keeps the fastest (state untouched); *rows receives the rows of its tiles or
- * segments.  Synchronises. */
+ * lengths) and keeps the fastest (state untouched); *rows receives what lbm_batch_set_segment
+ * takes to choose it.  Synchronises. */
 int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows);
 
 /* Advance every active channel by nsteps (a multiple of K).  Synchronises after every

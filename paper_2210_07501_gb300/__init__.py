@@ -79,6 +79,8 @@ SIGNATURES = {
                                         ctypes.c_void_p, ctypes.POINTER(_H)]),
     "lbm_batch_set_check_interval": (ctypes.c_int, [_H, ctypes.c_int32]),
     "lbm_batch_autotune": (ctypes.c_int, [_H, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32)]),
+    "lbm_batch_set_segment": (ctypes.c_int, [_H, ctypes.c_int32]),
+    "lbm_batch_launch_shape": (ctypes.c_int, [_H, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "lbm_batch_step": (ctypes.c_int, [_H, ctypes.c_int64]),
     "lbm_batch_run_to_steady": (ctypes.c_int, [_H, ctypes.c_double, ctypes.c_int64, _I64P,
                                                ctypes.POINTER(ctypes.c_int32)]),
@@ -129,6 +131,10 @@ def load(path: str | None = None):
 def _check(rc, where):
     if rc != LBM_OK:
         raise LbmError(rc, where)
+
+
+def _shape(cols, rows):
+    return {"kind": "tiles" if cols.value else "strips", "cols": cols.value, "rows": rows.value}
 
 
 def _dptr(a):
@@ -275,7 +281,7 @@ class Lbm:
     def lbm_launch_shape(self) -> dict:
         c, r = ctypes.c_int32(), ctypes.c_int32()
         _check(self._lib.lbm_launch_shape(self._h, ctypes.byref(c), ctypes.byref(r)), "lbm_launch_shape")
-        return {"kind": "tiles" if c.value else "strips", "cols": c.value, "rows": r.value}
+        return _shape(c, r)
 
     def lbm_bytes_per_node(self) -> int:
         b = ctypes.c_int64()
@@ -331,6 +337,14 @@ class LbmBatch:
         r = ctypes.c_int32()
         _check(self._lib.lbm_batch_autotune(self._h, int(reps), ctypes.byref(r)), "lbm_batch_autotune")
         return r.value
+
+    def lbm_batch_set_segment(self, rows: int):
+        _check(self._lib.lbm_batch_set_segment(self._h, int(rows)), "lbm_batch_set_segment")
+
+    def lbm_batch_launch_shape(self) -> dict:
+        c, r = ctypes.c_int32(), ctypes.c_int32()
+        _check(self._lib.lbm_batch_launch_shape(self._h, ctypes.byref(c), ctypes.byref(r)), "lbm_batch_launch_shape")
+        return _shape(c, r)
 
     def lbm_batch_step(self, n: int):
         _check(self._lib.lbm_batch_step(self._h, int(n)), "lbm_batch_step")

@@ -1218,8 +1218,27 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
         if (e != cudaSuccess) rc = cuda_fail(e, "lbm_batch_autotune");
     }
     b->graph_valid = false;
-    if (rows) *rows = b->shape.rows > 0 ? b->shape.rows : b->shape.ty;
+    if (rows) *rows = b->shape.rows > 0 ? b->shape.rows : LBM_SEGMENT_TILES;
     return rc;
+}
+
+int lbm_batch_set_segment(lbm_batch *b, int32_t rows)
+{
+    if (!b || rows < 0) return LBM_EINVAL;
+    const StepShape shape = rows == LBM_SEGMENT_TILES ? b->shapes.tile
+                            : rows > 0                ? StepShape{rows, 0, 0, 0}
+                                                      : b->shapes.automatic;
+    b->graph_valid = false;
+    CK(dispatch<BatchTableFn>(b->h[0], b, shape));
+    return LBM_OK;
+}
+
+int lbm_batch_launch_shape(const lbm_batch *b, int32_t *cols, int32_t *rows)
+{
+    if (!b) return LBM_EINVAL;
+    if (cols) *cols = b->shape.rows > 0 ? 0 : b->shape.tx;
+    if (rows) *rows = b->shape.rows > 0 ? b->shape.rows : b->shape.ty;
+    return LBM_OK;
 }
 
 int lbm_batch_step(lbm_batch *b, int64_t nsteps)
