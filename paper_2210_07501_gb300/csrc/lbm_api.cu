@@ -13,6 +13,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <array>
 #include <new>
 #include <vector>
 
@@ -774,16 +775,16 @@ int lbm_set_state(lbm_handle *h, const double *f, const double *g, const double 
 // ---- checkpoints ----
 static uint32_t crc32_update(uint32_t crc, const unsigned char *p, size_t n)
 {
-    static uint32_t table[256];
-    static bool init = false;
-    if (!init) {
+    // (initialised once, whichever thread saves or loads first)
+    static const std::array<uint32_t, 256> table = [] {
+        std::array<uint32_t, 256> t;
         for (uint32_t i = 0; i < 256; ++i) {
             uint32_t c = i;
             for (int k = 0; k < 8; ++k) c = (c & 1u) ? 0xEDB88320u ^ (c >> 1) : (c >> 1);
-            table[i] = c;
+            t[i] = c;
         }
-        init = true;
-    }
+        return t;
+    }();
     crc = ~crc;
     for (size_t i = 0; i < n; ++i) crc = table[(crc ^ p[i]) & 0xFFu] ^ (crc >> 8);
     return ~crc;

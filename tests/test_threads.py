@@ -61,6 +61,14 @@ def test_kernel_attributes_are_set_once_on_every_device():
         assert "cudaFuncSetAttribute" in code and "OncePerDevice" in code and "static bool" not in code, name
 
 
+def test_no_unordered_first_use():
+    """A plain static flag orders nothing: a second thread may see it set and the data behind it not (the
+    checksum table of checkpoints had one)."""
+    csrc = os.path.join(ROOT, "paper_2210_07501_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        assert "static bool" not in open(os.path.join(csrc, name)).read().replace("static bool aligned_rows(", ""), name
+
+
 @pytest.mark.gpu
 def test_two_threads_step_channels_of_different_size():
     """FP64 tiles ask for shared memory by the channel's size.  Two handles of one lattice pair, each
