@@ -196,6 +196,9 @@ template <typename R, typename S, int QF, int QT> struct StepFn {
 // 8192 x 2048.
 // FP16 storage is never bandwidth bound: 31 / 9.9 at 1024 x 256, 310 / 222 at 8192 x 1024.  FP64 (FP64 pipe):
 // 893 / 881 at 1501 x 1001, 1175 / 1226 at 2048 x 1024 (the march forms no normal twice).
+// Past the line it depends on the channel's width too, up to about twice the nodes: FP32 161 / 157 at 4096 x
+// 1300, 141 / 134 at 3000 x 1500; FP64 622 / 578 at 1100 x 1000, 738 / 612 at 523 x 2200 (narrow strips), which the
+// autotuner finds.
 static long long tile_nodes_max(int prec)
 {
     return prec == LBM_FP16 ? INT64_MAX : (prec == LBM_FP32 ? 1LL << 22 : 1LL << 20);

@@ -23,8 +23,10 @@ cudaError_t launch_tile(const StepArgs<Real, Store> &A, cudaStream_t s, const St
 
 // Many cases in one launch.  Up to PACK_CASES of them travel in the launch's parameters: their arguments
 // are then uniform values in constant memory, as those of a single channel are (fetched through
-// a pointer they cost ~160 instructions a node more and two dependent loads a CTA).  start[c]: first CTA
-// of case c (INT_MAX beyond the last case), cols[c]: its strips or tiles per row.
+// a pointer they cost ~160 instructions a node more and two dependent loads a CTA).  32, the power of
+// two that pack_case_ searches: a launch's parameters hold 32,764 bytes, and 32 cases take 27,904 (864 a
+// case in FP64).  start[c]: first CTA of case c (INT_MAX beyond the last case), cols[c]: its strips or
+// tiles per row.
 constexpr int PACK_CASES = 32;
 template <typename Real, typename Store> struct BatchPack {
     int start[PACK_CASES], cols[PACK_CASES];
@@ -53,7 +55,7 @@ cudaError_t launch_tile_pack(const BatchPack<Real, Store> &B, int n_ctas, const 
                              cudaStream_t s);
 // Columns per strip of the march.
 template <typename Real, typename Store, int QF, int QT> int step_strip_width();
-// Rows per segment of the march when none is set (whole waves of resident CTAs).
+// Rows per segment of the march when none is set (choose_segment).
 template <typename Real, typename Store, int QF, int QT> int auto_segment(int nx, int ny);
 // Tile shape for a channel on a device with `sms` SMs.
 template <typename Real, typename Store, int QF, int QT> StepShape choose_tile(int nx, long long ny, int sms);

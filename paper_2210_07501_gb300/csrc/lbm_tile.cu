@@ -21,8 +21,11 @@ template <typename Real, typename Store, int QF = 5, int QT = 5> struct TileGeo 
     static constexpr int NT = 256, TX = 32;
     // FP32: four CTAs per SM (64 registers; three: 9.8 us instead of 8.8 at 1024 x 256, five: 9.1, and 14.3
     // instead of 11.8 with three D2Q9 lattices).  FP16, latency bound on its smaller loads: five (48
-    // registers; 222 us at 8192 x 1024, 240 with four), four with two D2Q9 scalar lattices, which
-    // spill at 48.  FP64 takes the registers it needs.
+    // registers; 220 us at 8192 x 1024, 237 with four).  With one D2Q9 scalar lattice 16 to 28 bytes spill at
+    // 48 and five still win on large channels (271 us, 288 with four) and lose on small ones (1024 x
+    // 256: 13.1, 10.8); with two, four win (309 us, 329 with five).  The batch kernels take the same
+    // numbers; that of more than PACK_CASES channels spills up to 100 bytes (FP16), 20 (FP32).
+    // FP64 takes the registers it needs.
     static constexpr int CTAS = sizeof(Real) == 8 ? 1 : (sizeof(Store) == 2 && QF + QT < 18 ? 5 : 4);
 };
 
