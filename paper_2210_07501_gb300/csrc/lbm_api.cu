@@ -771,6 +771,7 @@ int lbm_set_state(lbm_handle *h, const double *f, const double *g, const double 
     }
     CK(cudaMemcpyAsync(h->staging, dp, N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     CK(dispatch<DpFn>(h, h->staging, 1));
+    CK(cudaMemsetAsync(h->result + 8, 0, sizeof(double), h->stream));   // a new state clears a fault
     CK(cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
