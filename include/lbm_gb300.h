@@ -234,7 +234,7 @@ int lbm_batch_set_check_interval(lbm_batch *b, int32_t K);
 
 /* Launch shape of the batch, as lbm_set_segment and lbm_launch_shape for one channel (0: tiles
  * while all channels together are too small to fill the GPU with strips, else strips in
- * segments of 32 rows).  Affects speed only.  Setting it waits for the batch's work. */
+ * segments of 32 rows).  Affects speed only. */
 int lbm_batch_set_segment(lbm_batch *b, int32_t rows);
 int lbm_batch_launch_shape(const lbm_batch *b, int32_t *cols, int32_t *rows);
 

@@ -1026,8 +1026,8 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
     {
         const int w = shape.rows > 0 ? step_strip_width<R, S, QF, QT>() : shape.tx;
         const int t_rows = shape.rows > 0 ? shape.rows : shape.ty;
-        b->shape = shape;
         if (b->n <= PACK_CASES) {
+            b->shape = shape;
             for (int par = 0; par < 2; ++par)
                 for (int m = 0; m < 2; ++m) {
                     b->pack[par][m].assign(sizeof(BatchPack<R, S>), 0);
@@ -1050,12 +1050,20 @@ template <typename R, typename S, int QF, int QT> struct BatchTableFn {
             for (int by = 0; by < segs; ++by)
                 for (int bx = 0; bx < strips; ++bx) t.push_back(make_int4(c, bx, by, 0));
         }
+        // the table in use stays until the new one is there: an error leaves the batch as it was
+        int4 *d = nullptr;
+        cudaError_t e = cudaMalloc((void **)&d, t.size() * sizeof(int4));
+        if (e == cudaSuccess) e = upload(d, t.data(), t.size() * sizeof(int4), b->stream);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (d) cudaFree(d);
+            return e;
+        }
         if (b->d_ctas) cudaFree(b->d_ctas);
-        b->d_ctas = nullptr;
-        cudaError_t e = cudaMalloc((void **)&b->d_ctas, t.size() * sizeof(int4));
-        if (e != cudaSuccess) return e;
+        b->d_ctas = d;
         b->n_ctas = (int)t.size();
-        return upload(b->d_ctas, t.data(), t.size() * sizeof(int4), b->stream);
+        b->shape = shape;
+        return cudaSuccess;
     }
 };
 
