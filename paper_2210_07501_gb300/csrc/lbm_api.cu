@@ -1238,8 +1238,10 @@ int lbm_batch_autotune(lbm_batch *b, int32_t reps, int32_t *rows)
 int lbm_batch_set_segment(lbm_batch *b, int32_t rows)
 {
     if (!b || rows < 0) return LBM_EINVAL;
+    int32_t tallest = 0;   // a segment ends with its channel
+    for (const lbm_handle *h : b->h) tallest = h->ny > tallest ? h->ny : tallest;
     const StepShape shape = rows == LBM_SEGMENT_TILES ? b->shapes.tile
-                            : rows > 0                ? StepShape{rows, 0, 0, 0}
+                            : rows > 0                ? StepShape{rows < tallest ? rows : tallest, 0, 0, 0}
                                                       : b->shapes.automatic;
     b->graph_valid = false;
     CK(dispatch<BatchTableFn>(b->h[0], b, shape));

@@ -78,6 +78,10 @@ def test_batch_shapes_of_the_rule():
         assert b.lbm_batch_launch_shape() == won
         b.lbm_batch_step(2)
         assert b.lbm_batch_diag(0)["steps"] == 4
+        b.lbm_batch_set_segment(LBM_SEGMENT_TILES - 1)     # one segment a strip
+        assert b.lbm_batch_launch_shape() == {"kind": "strips", "cols": 0, "rows": 512}
+        assert b.lbm_batch_size()["ctas"] == n * 512 // 128
+        b.lbm_batch_step(2)
         b.close()
 
 
